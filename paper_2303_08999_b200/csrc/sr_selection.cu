@@ -5,13 +5,9 @@
 //
 //  selection_gram_kernel   Gram statistics over sampled HR pixels (all pixels when no sample list is given): with
 //        z_l[i,c] = Phi_l[i] (dict_l . B_{i,c}) the response of atom l alone at pixel i, channel c (Eq. 6 with
-//        F_{W,beta} = Phi diag(beta) D), G = Z^T Z, b = Z^T h, hh = h^T h for the target image h. A CTA takes 32
-//        pixels at a time: patches B from the LR image (bicubic or bilinear taps, HR-clamped), responses, Z tile in
-//        shared memory, then a register-tiled fp32 rank update of its private G (thread = a TB x TB block). After
-//        every 32 pixels the fp32 block is added into the CTA's own slot of fp64 scratch memory, so fp32 only ever
-//        sums 32 c terms; a second kernel adds the slots in a fixed order (no atomics: results are reproducible).
-//        The arithmetic here is fp32 multiply-add on sampled pixels (the paper samples its LASSO features too): an
-//        offline tool, bound by the FMA pipe.
+//        F_{W,beta} = Phi diag(beta) D), G = Z^T Z, b = Z^T h, hh = h^T h for the target image h. Patches, responses and
+//        a register-tiled fp32 rank update, summed in fp64; every CTA leaves its sums in a slot of scratch memory and a
+//        second kernel adds the slots in a fixed order (no atomics: results are reproducible).
 //  selection_search_kernel   Algorithm 1 on G, b, hh in fp64 by ONE warp: LASSO by cyclic coordinate descent
 //        (Eq. 7), lambda doubling and bisection to || beta ||_0 ~ alpha_t L, least-squares re-fit of gamma on the
 //        support (Eq. 9, Cholesky), gamma folded into G and b, next alpha_t. A lane owns the vector elements lane,
@@ -24,9 +20,32 @@ namespace sr {
 
 namespace {
 
-constexpr int kGramThreads = 256;
-constexpr int kGramPixels = 32;       // pixels per chunk
 constexpr int kMaxSearchL = 128;
+
+// ---- Gram statistics -------------------------------------------------------------------------------------------------
+//
+// One CTA per SM: a rank group of 192 threads and two producer groups of 160. The producers take the chunks of the CTA
+// in turn; a chunk is PX pixels (rows = C PX <= 96 rows of Z, channel-major):
+//   1  patches    sPatch[tap][row]: separable up-sampling out of the pixels' LR windows, one thread per patch column
+//   2  responses  sZ[row][atom] = Phi * (dict . patch): 8 rows x T atoms per thread, both operands read as float4
+// The rank group turns the producers' Z into T x T blocks of the UPPER triangle of Z^T Z, one block per thread, the rows
+// dealt over groups of threads. The LR windows of a producer's next chunk travel (cp.async) behind stage 2, its
+// coefficients and targets from the end of stage 2 to the next chunk's stage 2: sampled pixels are scattered, every
+// coefficient is a 32-byte sector of its own, and that latency has to be covered.
+// fp32 only ever sums up to 96 terms: then a thread adds its block to the CTA's fp64 sums, which stay in shared memory
+// until the CTA is done.
+// Bound: the shared-memory pipe (about 60 % busy) and, beside it, the FMA pipe: a T x T block reads 2 T words for T^2
+// multiply-adds, sixteen clocks of either per warp and row at T = 8. 100 000 sampled pixels of a 1080p frame, D = 72,
+// k = 5, c = 3: 660 -> 176 us (before: an fp64 read-modify-write of the whole matrix in global memory per 32 pixels, one
+// response per thread with scalar loads, sixteen taps per patch element). Also tried: every warp in all three stages, two
+// CTAs per SM (304 us); scalar instead of packed multiply-adds with operands loaded a row ahead (226 us); a rank group
+// of 256 threads (193 us).
+constexpr int kGramRows = 96;          // most rows of Z per chunk, and most terms of an fp32 sum
+constexpr int kGramRank = 192;         // threads of the rank group: at least the 136 blocks of 128 atoms
+constexpr int kGramProd = 160;         // threads of a producer group
+constexpr int kGramThreads = kGramRank + 2 * kGramProd;
+constexpr int kGramMaxGroups = 16;
+constexpr int kGramSmemMax = 216 * 1024;      // dynamic shared memory of a CTA
 
 struct GramParams {
     const float* lr;
@@ -38,162 +57,416 @@ struct GramParams {
     int64_t count;            // sampled pixels (or n H W)
     Problem pb;
     double* slots;            // [ctas][Dp * Dp + Dp + 8]
-    int Dp;
+    int Dp;                   // row pitch of a slot's matrix (D rounded up to 16)
+    int px, rows;             // pixels and rows per chunk: px a multiple of 4 that divides kGramProd, rows = px * c
+    int nb, nblk, groups;     // blocks of T atoms, blocks of the upper triangle, row groups of the rank stage
+    int flush_every;          // chunks between two additions to the fp64 sums
+    int nw;                   // side of a pixel's LR window
+    uint32_t px_magic, nw_magic, nb_magic, r_magic, rows_magic;
+    int off_acc, off_set, set_floats;                    // shared-memory offsets in floats: fp64 sums, producer sets
+    int off_z, off_h, off_win, off_phi;                  // inside a producer's set (patches first)
 };
 
-__device__ __forceinline__ float coef_value(const void* coef, int f16, int64_t i)
+// floor(x / d) for 0 <= x < 2^29, magic = ceil(2^32 / d)
+__device__ __forceinline__ int gram_div(int x, int d, uint32_t magic) { return d == 1 ? x : (int)__umulhi((uint32_t)x, magic); }
+__device__ __forceinline__ void gram_cp4(void* dst, const void* src)
 {
-    return f16 ? __half2float(__ldg(reinterpret_cast<const __half*>(coef) + i)) : __ldg(reinterpret_cast<const float*>(coef) + i);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void gram_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void gram_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+__device__ __forceinline__ void gram_bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ void gram_bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+// named barriers: the rank group, the producers, Z of producer b complete, Z of producer b consumed
+enum { kBarRank = 1, kBarProd = 2, kBarFull = 4, kBarEmpty = 6 };
+
+// Column of atom l in a row of Z and in the transposed dictionary: at T = 8 the first and the second four atoms of all
+// blocks lie apart, so that neighbouring blocks' 16-byte loads are contiguous (no bank conflicts).
+template <int T> __device__ __forceinline__ int gram_col(int l, int nb)
+{
+    if (T == 4) return l;
+    return ((l & 4) ? nb * 4 : 0) + (l >> 3) * 4 + (l & 3);
 }
 
-template <int TB>
-__global__ void __launch_bounds__(kGramThreads) selection_gram_kernel(const GramParams p)
-{
-    extern __shared__ __align__(16) float gsm[];
-    const Problem& pb = p.pb;
-    const int C = pb.c, D = pb.D, kk = pb.k * pb.k, P = (pb.k - 1) / 2;
-    const int Dp = 16 * TB, rows = kGramPixels * C;
-    float* sDict = gsm;                                   // [D][kk]
-    float* sPatch = sDict + ((D * kk + 3) & ~3);          // [rows][kk]
-    float* sZ = sPatch + ((rows * kk + 3) & ~3);          // [rows][Dp]
-    float* sH = sZ + rows * Dp;                           // [rows]
-    __shared__ int64_t sPix[kGramPixels];                 // flat pixel index of each pixel of the chunk, -1 = none
-    const int tid = threadIdx.x, ti = tid >> 4, tj = tid & 15;
-    const int64_t HW = (int64_t)pb.H * pb.W;
-    const int slot_doubles = Dp * Dp + Dp + 8;
-    double* slot = p.slots + (int64_t)blockIdx.x * slot_doubles;
+struct __align__(16) GramPixel { int f, pix, Y, X; };                  // f = -1: no pixel
 
-    for (int i = tid; i < slot_doubles; i += kGramThreads) slot[i] = 0.0;     // the slot keeps the last call's contents
-    for (int i = tid; i < D * kk; i += kGramThreads) sDict[i] = __ldg(p.dict + i);
-    for (int i = tid; i < rows * Dp; i += kGramThreads) sZ[i] = 0.f;          // columns D..Dp-1 stay zero
+template <int K, int T>
+__global__ void __launch_bounds__(kGramThreads, 1) selection_gram_kernel(const __grid_constant__ GramParams p)
+{
+    constexpr int kk = K * K, P = (K - 1) / 2;
+    extern __shared__ __align__(16) float gsm[];
+    __shared__ GramPixel sPx[2][2][kGramRows];           // [producer][parity of its chunk count]
+    __shared__ __align__(16) int sPar[2][2][kGramRows];  // parity of the pixel's coefficient in plane 0 (which half of a word)
+    __shared__ int2 sLo[2][2][kGramRows];                // first LR row / column of its window
+    __shared__ float4 sW[kMaxScale];
+    __shared__ int sBase[kMaxScale];
+    const Problem& pb = p.pb;
+    const int C = pb.c, D = pb.D, PX = p.px, rows = p.rows, nb = p.nb, Dz = nb * T, RP = ((rows + 7) & ~7) + 4, r = pb.r, NW = p.nw;
+    const int tid = threadIdx.x;
+    float* sDict = gsm;                                  // [kk][Dz]
+    double* sG = reinterpret_cast<double*>(gsm + p.off_acc);          // [T * T][nblk], then b [Dz], then hh
+    double* sB = sG + T * T * p.nblk;
+    const int64_t HW = (int64_t)pb.H * pb.W;
+    const int hw_odd = (int)(HW & 1);
+    const int64_t all_chunks = (p.count + PX - 1) / PX;
+    const int chunks = (int)((all_chunks - blockIdx.x + gridDim.x - 1) / gridDim.x);   // of this CTA: blockIdx.x + j gridDim.x
+
+    // ---- set-up
+    for (int i = tid; i < T * T * p.nblk + Dz + 1; i += kGramThreads) sG[i] = 0.0;
+    for (int i = tid; i < kk * Dz; i += kGramThreads) sDict[i] = 0.f;
+    if (tid < kMaxScale) {
+        sW[tid] = make_float4(pb.ph.w[tid][0], pb.ph.w[tid][1], pb.ph.w[tid][2], pb.ph.w[tid][3]);
+        sBase[tid] = pb.ph.base[tid];
+    }
+    __syncthreads();
+    for (int i = tid; i < D * kk; i += kGramThreads) {
+        const int l = i / kk, j = i - l * kk;
+        sDict[j * Dz + gram_col<T>(l, nb)] = __ldg(p.dict + i);
+    }
     __syncthreads();
 
-    const int64_t chunks = (p.count + kGramPixels - 1) / kGramPixels;
-    for (int64_t ch = blockIdx.x; ch < chunks; ch += gridDim.x) {
-        if (tid < kGramPixels) {
-            const int64_t si = ch * kGramPixels + tid;
+    if (tid >= kGramRank) {
+        // =================================================================== producers
+        const int me = tid >= kGramRank + kGramProd ? 1 : 0, gt = tid - kGramRank - me * kGramProd, warp = gt >> 5, lane = gt & 31;
+        float* sPatch = gsm + p.off_set + me * p.set_floats;     // [kk][RP]
+        float* sZ = sPatch + p.off_z;                            // [rows][Dz]
+        float* sH = sPatch + p.off_h;                            // [2][kGramRows]
+        float* sWin = sPatch + p.off_win;                        // [rows][NW * NW]
+        uint32_t* sPhi = reinterpret_cast<uint32_t*>(sPatch + p.off_phi);   // phi_at(l, px): the 4-byte word that holds the coefficient
+        const int nw2 = NW * NW;
+        const uintptr_t coef_base = reinterpret_cast<uintptr_t>(p.coef);
+        const uintptr_t coef_end = coef_base + (uintptr_t)((int64_t)pb.n * D * HW) * (p.coef_f16 ? 2 : 4);
+        // [D][PX] with four words more after every eighth atom: the eight atoms apart that stage 2's lanes ask for at once
+        // start in different 16-byte bank groups
+        auto phi_at = [&](int l, int px) { return sPhi + l * PX + ((l >> 3) << 2) + px; };
+        auto first_tap = [&](int Zc, int& phase) {               // first LR tap of the (clamped) HR coordinate Zc, and its phase
+            const int q = gram_div(Zc, r, p.r_magic);
+            phase = Zc - q * r;
+            return q + sBase[phase];
+        };
+        auto load_pixels = [&](int j, int buf) {                 // pixels of this CTA's chunk j
+            if (gt >= PX) return;
+            const int64_t si = ((int64_t)blockIdx.x + (int64_t)j * gridDim.x) * PX + gt;
             int64_t flat = -1;
-            if (si < p.count) flat = p.samples ? __ldg(p.samples + si) : si;
-            if (flat < 0 || flat >= (int64_t)pb.n * HW) flat = -1;
-            sPix[tid] = flat;
-        }
-        __syncthreads();
-        // patches: B[(pixel, channel)][tap] = U_c at the clamped HR position
-        for (int e = tid; e < rows * kk; e += kGramThreads) {
-            const int row = e / kk, j = e - row * kk;
-            const int pi = row / C, c = row - pi * C;
-            const int64_t flat = sPix[pi];
-            float v = 0.f;
-            if (flat >= 0) {
-                const int f = (int)(flat / HW);
-                const int64_t pix = flat - (int64_t)f * HW;
-                const int Y = (int)(pix / pb.W), X = (int)(pix - (int64_t)Y * pb.W);
-                const int a = j / pb.k, b = j - a * pb.k;
-                v = bicubic_point(p.lr + ((int64_t)f * C + c) * pb.h * pb.w, pb.h, pb.w, pb.r, pb.ph,
-                                  clampi(Y + a - P, 0, pb.H - 1), clampi(X + b - P, 0, pb.W - 1));
+            if (j < chunks && si < p.count) flat = p.samples ? __ldg(p.samples + si) : si;
+            GramPixel g;
+            g.f = -1; g.pix = 0;
+            if (flat >= 0 && flat < (int64_t)pb.n * HW) {
+                g.f = (int)(flat / HW);
+                g.pix = (int)(flat - (int64_t)g.f * HW);
             }
-            sPatch[e] = v;
-        }
-        for (int row = tid; row < rows; row += kGramThreads) {
-            const int pi = row / C, c = row - pi * C;
-            const int64_t flat = sPix[pi];
-            float hv = 0.f;
-            if (flat >= 0) {
-                const int f = (int)(flat / HW);
-                hv = __ldg(p.target + ((int64_t)f * C + c) * HW + (flat - (int64_t)f * HW));
+            g.Y = g.pix / pb.W;
+            g.X = g.pix - g.Y * pb.W;
+            int ph;
+            sPx[me][buf][gt] = g;
+            sPar[me][buf][gt] = ((int)(coef_base >> 1) + (g.f & D & hw_odd) + g.pix) & 1;
+            sLo[me][buf][gt] = make_int2(first_tap(clampi(g.Y - P, 0, pb.H - 1), ph), first_tap(clampi(g.X - P, 0, pb.W - 1), ph));
+        };
+        auto fetch_windows = [&](int buf) {                      // a warp takes the windows of a pixel in all channels
+            const int hw = pb.h * pb.w;
+            for (int e = lane; e < nw2; e += 32) {
+                const int j = gram_div(e, NW, p.nw_magic), i = e - j * NW;
+                for (int px = warp; px < PX; px += kGramProd / 32) {
+                    const int f = sPx[me][buf][px].f;
+                    const int2 lo = sLo[me][buf][px];
+                    float* dst = sWin + px * nw2 + e;
+                    const float* src = p.lr + (int64_t)(f * C) * hw + clampi(lo.x + j, 0, pb.h - 1) * pb.w + clampi(lo.y + i, 0, pb.w - 1);
+                    if (f >= 0) {
+                        for (int c = 0; c < C; ++c) gram_cp4(dst + c * PX * nw2, src + (int64_t)c * hw);
+                    } else {
+                        for (int c = 0; c < C; ++c) dst[c * PX * nw2] = 0.f;
+                    }
+                }
             }
-            sH[row] = hv;
-        }
-        __syncthreads();
-        // responses: z[(pixel, channel)][l] = Phi_l[pixel] * (dict_l . B)
-        for (int e = tid; e < kGramPixels * D; e += kGramThreads) {
-            const int pi = e / D, l = e - pi * D;
-            const int64_t flat = sPix[pi];
-            float phi = 0.f;
-            if (flat >= 0) {
-                const int f = (int)(flat / HW);
-                phi = coef_value(p.coef, p.coef_f16, ((int64_t)f * D + l) * HW + (flat - (int64_t)f * HW));
+            gram_commit();
+        };
+        auto fetch_coefficients = [&](int buf) {                 // and the targets, into half `buf` of sH; a thread keeps its pixel
+            const int l0 = gram_div(gt, PX, p.px_magic), px = gt - l0 * PX, dl = gram_div(kGramProd, PX, p.px_magic);
+            const GramPixel g = sPx[me][buf][px];
+            if (g.f >= 0) {
+                const int64_t elem = ((int64_t)g.f * D + l0) * HW + g.pix;
+                if (p.coef_f16) {
+                    uintptr_t a = coef_base + (uintptr_t)elem * 2;
+#pragma unroll 4
+                    for (int l = l0; l < D; l += dl, a += (uintptr_t)(2 * HW) * dl) {
+                        const uintptr_t word = a & ~(uintptr_t)3;
+                        if (word >= coef_base && word + 4 <= coef_end) {
+                            gram_cp4(phi_at(l, px), reinterpret_cast<const void*>(word));
+                        } else {                                 // the first or last element, where the word reaches outside the tensor
+                            const uint32_t v = __ldg(reinterpret_cast<const unsigned short*>(a));
+                            *phi_at(l, px) = v << (8 * (int)(a & 2));
+                        }
+                    }
+                } else {
+                    const float* a = reinterpret_cast<const float*>(p.coef) + elem;
+#pragma unroll 4
+                    for (int l = l0; l < D; l += dl, a += HW * dl) gram_cp4(phi_at(l, px), a);
+                }
+                for (int c = l0; c < C; c += dl) gram_cp4(sH + buf * kGramRows + c * PX + px, p.target + ((int64_t)g.f * C + c) * HW + g.pix);
+            } else {
+                for (int l = l0; l < D; l += dl) *phi_at(l, px) = 0u;
+                for (int c = l0; c < C; c += dl) sH[buf * kGramRows + c * PX + px] = 0.f;
             }
-            const float* dl = sDict + l * kk;
-            for (int c = 0; c < C; ++c) {
-                const float* B = sPatch + (pi * C + c) * kk;
-                float resp = 0.f;
-                for (int j = 0; j < kk; ++j) resp = fmaf(dl[j], B[j], resp);
-                sZ[(pi * C + c) * Dp + l] = phi * resp;
+            gram_commit();
+        };
+
+        int buf = 0;
+        load_pixels(me, 0);
+        gram_bar_sync(kBarProd + me, kGramProd);
+        fetch_windows(0);
+        fetch_coefficients(0);
+        load_pixels(me + 2, 1);
+        for (int j = me; j < chunks; j += 2, buf ^= 1) {
+            gram_wait<1>();
+            gram_bar_sync(kBarProd + me, kGramProd);             // windows landed; the next chunk's pixels are known
+            // ---- stage 1: thread = one column of one row's patch; four horizontally filtered window rows slide down
+            for (int e = gt; e < rows * K; e += kGramProd) {
+                const int b = gram_div(e, rows, p.rows_magic), row = e - b * rows;
+                const int c = gram_div(row, PX, p.px_magic), px = row - c * PX;
+                const GramPixel g = sPx[me][buf][px];
+                const int2 lo = sLo[me][buf][px];
+                int phx;
+                const int xo = first_tap(clampi(g.X + b - P, 0, pb.W - 1), phx) - lo.y;
+                const float4 wx = sW[phx];
+                const float* win = sWin + row * nw2 + xo;
+                auto hor = [&](int i) {
+                    const float* s = win + i * NW;
+                    return fmaf(wx.w, s[3], fmaf(wx.z, s[2], fmaf(wx.y, s[1], wx.x * s[0])));
+                };
+                float t0 = hor(0), t1 = hor(1), t2 = hor(2), t3 = hor(3);
+                int cur = 0;
+#pragma unroll
+                for (int a = 0; a < K; ++a) {
+                    int phy;
+                    const int yo = first_tap(clampi(g.Y + a - P, 0, pb.H - 1), phy) - lo.x;
+                    if (yo > cur) {                              // by one: consecutive HR rows
+                        cur = yo;
+                        t0 = t1; t1 = t2; t2 = t3;
+                        t3 = hor(cur + 3);
+                    }
+                    const float4 wy = sW[phy];
+                    sPatch[(a * K + b) * RP + row] = fmaf(wy.w, t3, fmaf(wy.z, t2, fmaf(wy.y, t1, wy.x * t0)));
+                }
+            }
+            gram_wait<0>();
+            gram_bar_sync(kBarProd + me, kGramProd);             // patches complete, coefficients landed, windows consumed
+            fetch_windows(buf ^ 1);
+            if (j >= 2) gram_bar_sync(kBarEmpty + me, kGramRank + kGramProd);   // the rank group is done with this producer's last Z
+            // ---- stage 2: 8 rows x T atoms
+            for (int e = gt; e < ((rows + 7) >> 3) * nb; e += kGramProd) {
+                const int rg = gram_div(e, nb, p.nb_magic), t = e - rg * nb;
+                float2 z[8][T / 2];
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+#pragma unroll
+                    for (int q = 0; q < T / 2; ++q) z[i][q] = make_float2(0.f, 0.f);
+                const float* pp = sPatch + rg * 8;
+                const float* dp = sDict + t * 4;
+#pragma unroll 5
+                for (int i = 0; i < kk; ++i) {
+                    float pv[8];
+                    *reinterpret_cast<float4*>(pv) = *reinterpret_cast<const float4*>(pp + i * RP);
+                    *reinterpret_cast<float4*>(pv + 4) = *reinterpret_cast<const float4*>(pp + i * RP + 4);
+                    float2 dv[T / 2];
+                    *reinterpret_cast<float4*>(dv) = *reinterpret_cast<const float4*>(dp + i * Dz);
+                    if (T == 8) *reinterpret_cast<float4*>(dv + T / 2 - 2) = *reinterpret_cast<const float4*>(dp + i * Dz + nb * 4);
+#pragma unroll
+                    for (int u = 0; u < 8; ++u)
+#pragma unroll
+                        for (int q = 0; q < T / 2; ++q) z[u][q] = __ffma2_rn(make_float2(pv[u], pv[u]), dv[q], z[u][q]);
+                }
+#pragma unroll
+                for (int half = 0; half < 2; ++half) {           // four rows of one channel each
+                    const int row0 = rg * 8 + 4 * half;
+                    if (row0 < rows) {
+                        const int px0 = row0 - gram_div(row0, PX, p.px_magic) * PX;
+                        const int4 par = *reinterpret_cast<const int4*>(&sPar[me][buf][px0]);
+#pragma unroll
+                        for (int q = 0; q < T / 4; ++q) {        // atoms 4 q .. 4 q + 3 of the block
+                            float o[4][4];
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) {
+                                const int l = t * T + 4 * q + u;
+                                uint4 w = make_uint4(0u, 0u, 0u, 0u);
+                                if (l < D) w = *reinterpret_cast<const uint4*>(phi_at(l, px0));
+                                float f0, f1, f2, f3;
+                                if (p.coef_f16) {
+                                    const int odd = l & hw_odd;
+                                    f0 = __half2float(__ushort_as_half((unsigned short)(w.x >> (16 * (par.x ^ odd)))));
+                                    f1 = __half2float(__ushort_as_half((unsigned short)(w.y >> (16 * (par.y ^ odd)))));
+                                    f2 = __half2float(__ushort_as_half((unsigned short)(w.z >> (16 * (par.z ^ odd)))));
+                                    f3 = __half2float(__ushort_as_half((unsigned short)(w.w >> (16 * (par.w ^ odd)))));
+                                } else {
+                                    f0 = __uint_as_float(w.x); f1 = __uint_as_float(w.y); f2 = __uint_as_float(w.z); f3 = __uint_as_float(w.w);
+                                }
+                                o[0][u] = f0 * ((u & 1) ? z[4 * half + 0][2 * q + u / 2].y : z[4 * half + 0][2 * q + u / 2].x);
+                                o[1][u] = f1 * ((u & 1) ? z[4 * half + 1][2 * q + u / 2].y : z[4 * half + 1][2 * q + u / 2].x);
+                                o[2][u] = f2 * ((u & 1) ? z[4 * half + 2][2 * q + u / 2].y : z[4 * half + 2][2 * q + u / 2].x);
+                                o[3][u] = f3 * ((u & 1) ? z[4 * half + 3][2 * q + u / 2].y : z[4 * half + 3][2 * q + u / 2].x);
+                            }
+#pragma unroll
+                            for (int i = 0; i < 4; ++i)
+                                *reinterpret_cast<float4*>(sZ + (row0 + i) * Dz + q * nb * 4 + t * 4) = make_float4(o[i][0], o[i][1], o[i][2], o[i][3]);
+                        }
+                    }
+                }
+            }
+            __threadfence_block();                               // (bar.arrive orders nothing by itself for the reader's loads)
+            gram_bar_arrive(kBarFull + me, kGramRank + kGramProd);      // Z (and the targets) of this chunk are complete
+            gram_bar_sync(kBarProd + me, kGramProd);             // coefficients consumed
+            fetch_coefficients(buf ^ 1);
+            load_pixels(j + 4, buf);                             // this chunk's pixels are no longer needed
+        }
+        gram_wait<0>();
+    } else {
+        // =================================================================== rank update
+        const int grp = tid / p.nblk, blk = tid - grp * p.nblk;
+        const bool has_block = grp < p.groups;
+        int ti = 0, tj = blk;
+        while (tj >= nb - ti) { tj -= nb - ti; ++ti; }
+        tj += ti;
+        float2 acc[T][T / 2];
+        float bacc[T], hacc = 0.f;
+#pragma unroll
+        for (int a = 0; a < T; ++a) {
+            bacc[a] = 0.f;
+#pragma unroll
+            for (int b = 0; b < T / 2; ++b) acc[a][b] = make_float2(0.f, 0.f);
+        }
+        int since_flush = 0;
+        for (int j = 0; j < chunks; ++j) {
+            const int b2 = j & 1;
+            const float* sZ = gsm + p.off_set + b2 * p.set_floats + p.off_z;
+            const float* h = gsm + p.off_set + b2 * p.set_floats + p.off_h + ((j >> 1) & 1) * kGramRows;
+            gram_bar_sync(kBarFull + b2, kGramRank + kGramProd);
+            if (has_block) {
+#pragma unroll 2
+                for (int row = grp; row < rows; row += p.groups) {
+                    const float* zr = sZ + row * Dz;
+                    float za[T];
+                    float2 zb[T / 2];
+                    *reinterpret_cast<float4*>(za) = *reinterpret_cast<const float4*>(zr + ti * 4);
+                    *reinterpret_cast<float4*>(zb) = *reinterpret_cast<const float4*>(zr + tj * 4);
+                    if (T == 8) {
+                        *reinterpret_cast<float4*>(za + T - 4) = *reinterpret_cast<const float4*>(zr + nb * 4 + ti * 4);
+                        *reinterpret_cast<float4*>(zb + T / 2 - 2) = *reinterpret_cast<const float4*>(zr + nb * 4 + tj * 4);
+                    }
+#pragma unroll
+                    for (int a = 0; a < T; ++a)
+#pragma unroll
+                        for (int b = 0; b < T / 2; ++b) acc[a][b] = __ffma2_rn(make_float2(za[a], za[a]), zb[b], acc[a][b]);
+                    if (ti == tj) {
+                        const float hv = h[row];
+#pragma unroll
+                        for (int a = 0; a < T; ++a) bacc[a] = fmaf(za[a], hv, bacc[a]);
+                        hacc = fmaf(hv, hv, hacc);
+                    }
+                }
+            }
+            if (j + 2 < chunks) gram_bar_arrive(kBarEmpty + b2, kGramRank + kGramProd);
+            if (++since_flush >= p.flush_every || j + 1 == chunks) {
+                since_flush = 0;
+                // fp32 blocks into the fp64 sums. The groups hold partial sums of the same blocks: in step q group g adds
+                // row (g + q) mod m of its block, so that all groups work at once, never on the same row, and every
+                // sum is formed in a fixed order.
+                const int m = max(p.groups, T);
+                int want = grp;
+                for (int q = 0; q < m; ++q) {
+                    if (has_block) {
+#pragma unroll
+                        for (int a = 0; a < T; ++a) {
+                            if (a == want) {
+                                double v[T];
+#pragma unroll
+                                for (int b = 0; b < T; ++b) v[b] = sG[(a * T + b) * p.nblk + blk];
+#pragma unroll
+                                for (int b = 0; b < T / 2; ++b) {
+                                    v[2 * b] += (double)acc[a][b].x;
+                                    v[2 * b + 1] += (double)acc[a][b].y;
+                                    acc[a][b] = make_float2(0.f, 0.f);
+                                }
+#pragma unroll
+                                for (int b = 0; b < T; ++b) sG[(a * T + b) * p.nblk + blk] = v[b];
+                                if (ti == tj) {
+                                    sB[ti * T + a] += (double)bacc[a];
+                                    bacc[a] = 0.f;
+                                    if (ti == 0 && a == 0) { sB[Dz] += (double)hacc; hacc = 0.f; }
+                                }
+                            }
+                        }
+                    }
+                    if (++want == m) want = 0;
+                    gram_bar_sync(kBarRank, kGramRank);
+                }
             }
         }
-        __syncthreads();
-        // rank update of this thread's TB x TB block, then into the fp64 slot
-        float acc[TB][TB];
+        // ---- the CTA's slot: the upper triangle (block rows ti <= tj, whole blocks on the diagonal), b, hh
+        double* slot = p.slots + (int64_t)blockIdx.x * (p.Dp * p.Dp + p.Dp + 8);
+        if (grp == 0) {
 #pragma unroll
-        for (int a = 0; a < TB; ++a)
+            for (int a = 0; a < T; ++a)
 #pragma unroll
-            for (int b = 0; b < TB; ++b) acc[a][b] = 0.f;
-        float bacc[TB];
-#pragma unroll
-        for (int a = 0; a < TB; ++a) bacc[a] = 0.f;
-        float hacc = 0.f;
-        for (int row = 0; row < rows; ++row) {
-            const float* zr = sZ + row * Dp;
-            float za[TB], zb[TB];
-#pragma unroll
-            for (int a = 0; a < TB; ++a) { za[a] = zr[ti * TB + a]; zb[a] = zr[tj * TB + a]; }
-#pragma unroll
-            for (int a = 0; a < TB; ++a)
-#pragma unroll
-                for (int b = 0; b < TB; ++b) acc[a][b] = fmaf(za[a], zb[b], acc[a][b]);
-            if (tj == 0) {
-                const float hv = sH[row];
-#pragma unroll
-                for (int a = 0; a < TB; ++a) bacc[a] = fmaf(za[a], hv, bacc[a]);
-                if (ti == 0) hacc = fmaf(hv, hv, hacc);
-            }
+                for (int b = 0; b < T; ++b) slot[(ti * T + a) * p.Dp + tj * T + b] = sG[(a * T + b) * p.nblk + blk];
         }
-#pragma unroll
-        for (int a = 0; a < TB; ++a)
-#pragma unroll
-            for (int b = 0; b < TB; ++b) slot[(ti * TB + a) * Dp + tj * TB + b] += (double)acc[a][b];
-        if (tj == 0) {
-#pragma unroll
-            for (int a = 0; a < TB; ++a) slot[Dp * Dp + ti * TB + a] += (double)bacc[a];
-            if (ti == 0) slot[Dp * Dp + Dp] += (double)hacc;
-        }
-        __syncthreads();                                  // sZ, sPatch, sPix are rewritten by the next chunk
+        for (int i = tid; i < D; i += kGramRank) slot[p.Dp * p.Dp + i] = sB[i];
+        if (tid == 0) slot[p.Dp * p.Dp + p.Dp] = sB[Dz];
     }
 }
 
-__global__ void selection_gram_reduce_kernel(const double* slots, int nslots, int Dp, int D, double* G, double* b, double* hh)
+// Adds the slots in a fixed order: 32 elements per block, eight threads per element take every eighth slot, their sums
+// are added one after the other.
+constexpr int kReduceLanes = 8;
+__global__ void __launch_bounds__(32 * kReduceLanes) selection_gram_reduce_kernel(const double* slots, int nslots, int Dp, int D, double* G, double* b, double* hh)
 {
+    __shared__ double part[kReduceLanes][32];
     const int slot_doubles = Dp * Dp + Dp + 8;
     const int total = D * D + D + 1;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-        int src;
-        if (i < D * D) src = (i / D) * Dp + (i % D);
-        else if (i < D * D + D) src = Dp * Dp + (i - D * D);
-        else src = Dp * Dp + Dp;
-        double v = 0.0;
-        for (int s = 0; s < nslots; ++s) v += slots[(int64_t)s * slot_doubles + src];
+    const int i = blockIdx.x * 32 + threadIdx.x;
+    int src = -1;
+    if (i < D * D) {
+        const int row = i / D, col = i - row * D;
+        src = min(row, col) * Dp + max(row, col);         // only the upper triangle is in the slots
+    } else if (i < D * D + D) {
+        src = Dp * Dp + (i - D * D);
+    } else if (i < total) {
+        src = Dp * Dp + Dp;
+    }
+    double v = 0.0;
+    if (src >= 0) {
+#pragma unroll 8
+        for (int s = threadIdx.y; s < nslots; s += kReduceLanes) v += slots[(int64_t)s * slot_doubles + src];
+    }
+    part[threadIdx.y][threadIdx.x] = v;
+    __syncthreads();
+    if (threadIdx.y == 0 && src >= 0) {
+        for (int q = 1; q < kReduceLanes; ++q) v += part[q][threadIdx.x];
         if (i < D * D) G[i] = v;
         else if (i < D * D + D) b[i - D * D] = v;
         else *hh = v;
     }
 }
 
-template <int TB>
-cudaError_t launch_gram_tb(const GramParams& p, int ctas, size_t smem, cudaStream_t st)
+template <int K, int T>
+cudaError_t launch_gram_kt(const GramParams& p, int ctas, size_t smem, cudaStream_t st)
 {
-    auto kern = selection_gram_kernel<TB>;
+    auto kern = selection_gram_kernel<K, T>;
     static bool configured[64] = {false};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (!configured[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kGramSmemMax);
         if (e != cudaSuccess) return e;
         configured[dev] = true;
     }
     kern<<<ctas, kGramThreads, smem, st>>>(p);
     count_launches(1);
     return cudaGetLastError();
+}
+
+template <int K>
+cudaError_t launch_gram_k(const GramParams& p, int T, int ctas, size_t smem, cudaStream_t st)
+{
+    return T == 4 ? launch_gram_kt<K, 4>(p, ctas, smem, st) : launch_gram_kt<K, 8>(p, ctas, smem, st);
 }
 
 // ---- Algorithm 1 in one warp ---------------------------------------------------------------------------------------
@@ -476,28 +749,54 @@ cudaError_t launch_selection_gram(const float* lr, const void* coef, int coef_dt
     p.count = samples ? nsamples : (int64_t)pb.n * pb.H * pb.W;
     p.pb = pb;
     p.slots = slots;
-    const int TB = (pb.D + 15) / 16;
-    p.Dp = 16 * TB;
-    const int64_t chunks = (p.count + kGramPixels - 1) / kGramPixels;
-    int ctas = (int)(chunks < nslots ? chunks : nslots);
+    p.Dp = (pb.D + 15) / 16 * 16;
+    const int T = pb.D > 32 ? 8 : 4, kk = pb.k * pb.k;       // few atoms: smaller blocks, so that there are enough of them
+    p.nb = (pb.D + T - 1) / T;
+    p.nblk = p.nb * (p.nb + 1) / 2;
+    p.nw = (pb.k - 1 + pb.r - 1) / pb.r + 4;
+    const int Dz = p.nb * T;
+    auto up4 = [](int v) { return (v + 3) & ~3; };
+    // as many pixels per chunk as give at most 96 rows and fit; the divisors of 160 let a producer thread keep its pixel
+    int floats = 0;
+    for (int px : {80, 40, 32, 20, 16, 8, 4}) {
+        if (px * pb.c > kGramRows) continue;
+        p.px = px;
+        p.rows = px * pb.c;
+        p.off_acc = up4(kk * Dz);
+        p.off_set = p.off_acc + up4(2 * (T * T * p.nblk + Dz + 1));
+        p.off_z = up4(kk * (((p.rows + 7) & ~7) + 4));
+        p.off_h = p.off_z + p.rows * Dz;
+        p.off_win = p.off_h + 2 * kGramRows;
+        p.off_phi = p.off_win + up4(p.rows * p.nw * p.nw);
+        p.set_floats = p.off_phi + up4(pb.D * p.px + (pb.D >> 3) * 4);
+        floats = p.off_set + 2 * p.set_floats;
+        if ((size_t)floats * sizeof(float) <= (size_t)kGramSmemMax) break;
+        floats = 0;
+    }
+    if (floats == 0) return cudaErrorNotSupported;
+    const size_t smem = (size_t)floats * sizeof(float);
+    auto magic = [](int d) { return (uint32_t)((0x100000000ull + d - 1) / d); };
+    p.px_magic = magic(p.px); p.nw_magic = magic(p.nw); p.nb_magic = magic(p.nb); p.r_magic = magic(pb.r); p.rows_magic = magic(p.rows);
+    p.groups = kGramRank / p.nblk;
+    if (p.groups > kGramMaxGroups) p.groups = kGramMaxGroups;
+    const int rows_per_group = (p.rows + p.groups - 1) / p.groups;
+    p.flush_every = kGramRows / rows_per_group > 1 ? kGramRows / rows_per_group : 1;
+    const int64_t chunks = (p.count + p.px - 1) / p.px;
+    int64_t ctas = sm_count();
+    if (ctas > nslots) ctas = nslots;
+    if (ctas > chunks) ctas = chunks;
     if (ctas < 1) ctas = 1;
-    const int kk = pb.k * pb.k, rows = kGramPixels * pb.c;
-    const size_t smem = (size_t)(((pb.D * kk + 3) & ~3) + ((rows * kk + 3) & ~3) + rows * p.Dp + rows) * sizeof(float);
-    if (smem > 200 * 1024) return cudaErrorNotSupported;
     cudaError_t e;
-    switch (TB) {
-    case 1: e = launch_gram_tb<1>(p, ctas, smem, st); break;
-    case 2: e = launch_gram_tb<2>(p, ctas, smem, st); break;
-    case 3: e = launch_gram_tb<3>(p, ctas, smem, st); break;
-    case 4: e = launch_gram_tb<4>(p, ctas, smem, st); break;
-    case 5: e = launch_gram_tb<5>(p, ctas, smem, st); break;
-    case 6: e = launch_gram_tb<6>(p, ctas, smem, st); break;
-    case 7: e = launch_gram_tb<7>(p, ctas, smem, st); break;
-    case 8: e = launch_gram_tb<8>(p, ctas, smem, st); break;
+    switch (pb.k) {
+    case 1: e = launch_gram_k<1>(p, T, (int)ctas, smem, st); break;
+    case 3: e = launch_gram_k<3>(p, T, (int)ctas, smem, st); break;
+    case 5: e = launch_gram_k<5>(p, T, (int)ctas, smem, st); break;
+    case 7: e = launch_gram_k<7>(p, T, (int)ctas, smem, st); break;
+    case 9: e = launch_gram_k<9>(p, T, (int)ctas, smem, st); break;
     default: return cudaErrorNotSupported;
     }
     if (e != cudaSuccess) return e;
-    selection_gram_reduce_kernel<<<(pb.D * pb.D + pb.D + 1 + 255) / 256, 256, 0, st>>>(slots, ctas, p.Dp, pb.D, G, b, hh);
+    selection_gram_reduce_kernel<<<(pb.D * pb.D + pb.D + 1 + 31) / 32, dim3(32, kReduceLanes), 0, st>>>(slots, (int)ctas, p.Dp, pb.D, G, b, hh);
     count_launches(1);
     return cudaGetLastError();
 }

@@ -114,3 +114,17 @@ def test_search_end_to_end_finds_planted_atoms_and_feeds_the_subset_regression()
     assert np.abs(host(out) - want).max() <= TOL_F16
     assert np.mean((host(out) - target) ** 2) <= 0.03 * np.mean(target.astype(np.float64) ** 2)   # eight atoms of 72 keep the image
     assert sr.sr_device_status() == 0
+
+
+@pytest.mark.parametrize("D,k,r,h,w,dt,n,c,base", [(32, 3, 2, 9, 7, "f16", 1, 3, 0), (33, 5, 3, 7, 9, "f16", 2, 3, 0), (72, 5, 3, 7, 5, "f16", 1, 1, 2),
+                                                   (71, 7, 1, 9, 13, "f16", 1, 4, 0), (128, 9, 8, 2, 3, "f32", 1, 2, 0), (8, 3, 2, 5, 5, "f32", 3, 16, 0)])
+def test_gram_at_block_edges_and_odd_planes(D, k, r, h, w, dt, n, c, base):
+    # both block sizes on both sides of their atom limits, odd plane sizes (a binary16 coefficient in either half of its
+    # word, with the tensor's first or last element alone in one), more channels than a chunk has groups of rows
+    wl, lr, d, coef, target = _problem(D, k, r, h, w, dt, n, c, seed=D)
+    co = dev(coef)
+    if base:                                                  # a tensor that starts in the upper half of a word
+        room = torch.zeros(co.numel() + 8, dtype=co.dtype, device="cuda")
+        co = room[1:1 + co.numel()].view(co.shape).copy_(co)
+        assert co.data_ptr() % 4 == 2
+    _gram_close(sr.sr_selection_gram(dev(lr), co, dev(d), dev(target), None, r, k), *oracle.selection_gram(lr, coef, d, target, None, r, k))
