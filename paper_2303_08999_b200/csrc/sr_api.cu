@@ -515,7 +515,7 @@ int sr_selection_search(const double* G, const double* b, const double* hh, doub
         return SR_ERR_ALIGN;
     if (scratch_bytes < selection_search_scratch_bytes(D)) return SR_ERR_SHAPE;
     return launch_selection_search(G, b, hh, nrows, D, *o, idx_out, gamma_out, count_out, trace, steps_out,
-                                   static_cast<double*>(scratch), (cudaStream_t)stream) == cudaSuccess ? SR_OK : SR_ERR_CUDA;
+                                   (cudaStream_t)stream) == cudaSuccess ? SR_OK : SR_ERR_CUDA;
 }
 
 const char* sr_status_string(int status)

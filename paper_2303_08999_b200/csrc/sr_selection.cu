@@ -8,11 +8,11 @@
 //        F_{W,beta} = Phi diag(beta) D), G = Z^T Z, b = Z^T h, hh = h^T h for the target image h. Patches, responses and
 //        a register-tiled fp32 rank update, summed in fp64; every CTA leaves its sums in a slot of scratch memory and a
 //        second kernel adds the slots in a fixed order (no atomics: results are reproducible).
-//  selection_search_kernel   Algorithm 1 on G, b, hh in fp64 by ONE warp: LASSO by cyclic coordinate descent
+//  selection_search_kernel   Algorithm 1 on G, b, hh in fp64 by ONE thread block: LASSO by cyclic coordinate descent
 //        (Eq. 7), lambda doubling and bisection to || beta ||_0 ~ alpha_t L, least-squares re-fit of gamma on the
-//        support (Eq. 9, Cholesky), gamma folded into G and b, next alpha_t. A lane owns the vector elements lane,
-//        lane + 32, ...; every element-wise update and every sum runs in the same order as a sequential program, with
-//        separate multiplies and adds (no contraction), so the result does not depend on the parallelisation.
+//        support (Eq. 9, Cholesky), gamma folded into G and b, next alpha_t. Every element-wise update and every sum runs
+//        in the same order as a sequential program, with separate multiplies and adds (no contraction), so the result
+//        does not depend on the parallelisation.
 #include "sr_common.cuh"
 #include "sr_selection.cuh"
 
@@ -469,7 +469,23 @@ cudaError_t launch_gram_k(const GramParams& p, int T, int ctas, size_t smem, cud
     return T == 4 ? launch_gram_kt<K, 4>(p, ctas, smem, st) : launch_gram_kt<K, 8>(p, ctas, smem, st);
 }
 
-// ---- Algorithm 1 in one warp ---------------------------------------------------------------------------------------
+// ---- Algorithm 1 in one thread block -----------------------------------------------------------------------------------
+//
+// The sweeps of coordinate descent are one serial chain in fp64: coordinate l's step needs the residual that coordinate
+// l - 1's step left. One warp walks it; four warps share what is parallel (residuals, factorisation, re-scaling).
+// The active atoms are kept compacted (index 0 .. na - 1, order of the atoms), so no step ever looks at a dropped one.
+//
+// What bounds a sweep is the latency of that chain, so everything else is kept off it. Coordinates go in blocks of
+// eight: all lanes hold the block's eight residuals, make its eight steps redundantly and apply each step to the
+// residuals that follow in the block; the residuals of all atoms (lane, lane + 32, ...) get the eight steps afterwards,
+// in the same order, behind the next steps. A step is then ten dependent fp64 operations: two additions to the
+// thresholded numerator, five for the quotient, one for the step, a product and a sum to the next residual; no shuffle,
+// no shared-memory load and no branch among them. Every rounding is that of the sequential program, so the results are
+// the same bits.
+// 72 atoms down to 8 in four steps (about 90 solves, 90 000 steps): 46.0 -> 9.3 ms against one warp that kept residuals and
+// coefficients in shared memory and divided inside the chain.
+constexpr int kSearchThreads = 128;
+constexpr int kCdBlock = 8;
 
 struct SearchParams {
     const double* G;
@@ -483,163 +499,244 @@ struct SearchParams {
     int* count_out;
     double* trace;
     int* steps_out;
-    double* chol;         // scratch: [L][L]
-    int* status;
 };
 
 struct SearchState {
-    double* G;            // [L][Lp]
-    double *b, *beta, *r, *best, *cand, *gtot, *tmp;
-    uint8_t* active;
-    int* S;
-    int L, Lp, lane;
+    double* G;            // [L8][Lp], active atoms only; columns na .. na8 - 1 are zero
+    double* A;            // packed lower triangle
+    double *b, *beta, *r, *best, *cand, *gtot, *tmp, *prod;
+    double *diag, *rcp, *frz;   // G[l][l], 1 / G[l][l], and 0 or (atoms whose G[l][l] is not positive: never moved) infinity
+    int *S, *orig;        // support; compact index -> atom
+    int L8, Lp, na, na8, tid, lane;
     double nrows;
+    bool safe;            // every positive G[l][l] lies in [2^-300, 2^300]
 };
 
-__device__ __forceinline__ double bcast(double v, int src)
-{
-    int lo = __double2loint(v), hi = __double2hiint(v);
-    lo = __shfl_sync(0xffffffffu, lo, src);
-    hi = __shfl_sync(0xffffffffu, hi, src);
-    return __hiloint2double(hi, lo);
-}
+__host__ __device__ constexpr int search_l8(int L) { return (L + kCdBlock - 1) / kCdBlock * kCdBlock; }
 
-__device__ int count_nonzero(const SearchState& s, const double* beta)
+__device__ int count_nonzero(const SearchState& s, const double* beta)   // every warp counts for itself
 {
     int n = 0;
-    for (int l = s.lane; l < s.L; l += 32) n += (s.active[l] && beta[l] != 0.0) ? 1 : 0;
+    for (int l = s.lane; l < s.na; l += 32) n += beta[l] != 0.0 ? 1 : 0;
     for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
     return n;
 }
 
-// Eq. 7 by cyclic coordinate descent; beta in / out. Same operation order as a sequential loop over the atoms.
-__device__ int lasso_cd(const SearchState& s, double lambda, double* beta, double tol, int max_sweeps)
+// Diagonal, reciprocals and padding of the compacted matrix and vectors. Ends in a barrier.
+__device__ void prepare_active(SearchState& s)
 {
-    const int L = s.L, Lp = s.Lp;
-    for (int l = s.lane; l < L; l += 32) {
-        if (!s.active[l]) { beta[l] = 0.0; continue; }
+    s.na8 = search_l8(s.na);
+    int bad = 0;
+    for (int l = s.tid; l < s.L8; l += kSearchThreads) {
+        const double g = l < s.na ? s.G[l * s.Lp + l] : 0.0;
+        const bool live = g > 0.0;
+        s.diag[l] = g;
+        s.rcp[l] = live ? __drcp_rn(g) : 0.0;
+        s.frz[l] = live ? 0.0 : __longlong_as_double(0x7FF0000000000000ll);
+        if (live && !(g >= 0x1p-300 && g <= 0x1p300)) bad = 1;
+        if (l >= s.na) s.beta[l] = s.cand[l] = s.best[l] = s.r[l] = 0.0;
+        for (int m = s.na; m < s.na8; ++m) s.G[l * s.Lp + m] = 0.0;
+    }
+    s.safe = !__syncthreads_or(bad);
+}
+
+// num / g rounded to nearest. FAST: y = 1 / g rounded to nearest; an estimate is corrected twice by its exact remainder
+// (Markstein, IBM J. Res. Dev. 34 (1990): if q is one of the two neighbours of the quotient, y the rounded reciprocal
+// and the remainder exact, then q + remainder * y rounds to the rounded quotient; the first correction makes the
+// estimate such a neighbour). The caller has excluded operands that could under- or overflow on the way.
+template <bool FAST> __device__ __forceinline__ double cd_quotient(double num, double g, double y)
+{
+    if (!FAST) return __ddiv_rn(num, g);
+    double q = __dmul_rn(num, y);
+    q = __fma_rn(__fma_rn(-g, q, num), y, q);
+    return __fma_rn(__fma_rn(-g, q, num), y, q);
+}
+
+// Warp 0: sweeps over the active atoms until no coefficient moves by more than tol. Residuals in and out through s.r.
+// Returns the sweeps made, negative when it stopped because a step was too large for the fast quotient's range.
+template <int NK, bool FAST>
+__device__ __noinline__ int cd_sweeps(const SearchState& s, double thr, double* beta, double tol, int max_sweeps)
+{
+    const int Lp = s.Lp, na8 = s.na8;
+    double rr[NK];
+    const double* row[NK];
+#pragma unroll
+    for (int k = 0; k < NK; ++k) {
+        const int m = s.lane + 32 * k;
+        rr[k] = m < na8 ? s.r[m] : 0.0;
+        row[k] = s.G + min(m, s.L8 - 1) * Lp;
+    }
+    int sweep = 0;
+    bool too_large = false;
+    while (sweep < max_sweeps && !too_large) {
+        double moved = 0.0;
+#pragma unroll 1
+        for (int l0 = 0; l0 < na8; l0 += kCdBlock) {
+            double rk = rr[0];
+#pragma unroll
+            for (int k = 1; k < NK; ++k) rk = l0 >= 32 * k ? rr[k] : rk;
+            double rb[kCdBlock], d[kCdBlock], nb[kCdBlock];
+#pragma unroll
+            for (int i = 0; i < kCdBlock; ++i) rb[i] = __shfl_sync(0xffffffffu, rk, (l0 & 31) + i);
+            const double* Gb = s.G + l0 * Lp + l0;
+#pragma unroll
+            for (int i = 0; i < kCdBlock; ++i) {
+                const double g = s.diag[l0 + i], be = beta[l0 + i], fz = s.frz[l0 + i];
+                const double rho = __dadd_rn(rb[i], __dmul_rn(g, be));
+                const double q = cd_quotient<FAST>(__dadd_rn(rho, -copysign(thr, rho)), g, s.rcp[l0 + i]);
+                nb[i] = fabs(rho) > __dadd_rn(thr, fz) ? q : (fz > 0.0 ? be : 0.0);
+                d[i] = __dadd_rn(nb[i], -be);
+#pragma unroll
+                for (int j = i + 1; j < kCdBlock; ++j) rb[j] = __dadd_rn(rb[j], -__dmul_rn(d[i], Gb[j * Lp + i]));
+                moved = fmax(moved, fabs(d[i]));
+            }
+#pragma unroll
+            for (int i = 0; i < kCdBlock; ++i)
+#pragma unroll
+                for (int k = 0; k < NK; ++k) rr[k] = __dadd_rn(rr[k], -__dmul_rn(d[i], row[k][l0 + i]));
+            __syncwarp();
+            if (s.lane == 0) {
+#pragma unroll
+                for (int i = 0; i < kCdBlock; ++i) beta[l0 + i] = nb[i];
+            }
+            __syncwarp();
+        }
+        ++sweep;
+        if (moved <= tol) break;
+        if (FAST && !(moved < 0x1p200)) too_large = true;
+    }
+#pragma unroll
+    for (int k = 0; k < NK; ++k)
+        if (s.lane + 32 * k < na8) s.r[s.lane + 32 * k] = rr[k];
+    __syncwarp();
+    return too_large ? -sweep : sweep;
+}
+
+// Eq. 7 by cyclic coordinate descent; beta in / out. Same operation order as a sequential loop over the atoms. All
+// threads; starts after a barrier that made beta visible and ends in one.
+__device__ void lasso_cd(const SearchState& s, double lambda, double* beta, double tol, int max_sweeps)
+{
+    for (int l = s.tid; l < s.na; l += kSearchThreads) {
         double acc = 0.0;
-        for (int m = 0; m < L; ++m)
-            if (s.active[m]) acc = __dadd_rn(acc, __dmul_rn(s.G[l * Lp + m], beta[m]));
+#pragma unroll 8
+        for (int m = 0; m < s.na; ++m) acc = __dadd_rn(acc, __dmul_rn(s.G[l * s.Lp + m], beta[m]));
         s.r[l] = __dadd_rn(s.b[l], -acc);
     }
-    __syncwarp();
-    const double thr = __dmul_rn(__dmul_rn(0.5, lambda), s.nrows);
-    int sweep = 0;
-    for (; sweep < max_sweeps; ++sweep) {
-        double moved = 0.0;
-        for (int l = 0; l < L; ++l) {
-            if (!s.active[l]) continue;
-            const double gll = s.G[l * Lp + l];
-            if (!(gll > 0.0)) continue;
-            const int owner = l & 31;
-            double delta = 0.0, nb = 0.0;
-            if (s.lane == owner) {
-                const double rho = __dadd_rn(s.r[l], __dmul_rn(gll, beta[l]));
-                if (rho > thr) nb = __ddiv_rn(__dadd_rn(rho, -thr), gll);
-                else if (rho < -thr) nb = __ddiv_rn(__dadd_rn(rho, thr), gll);
-                delta = __dadd_rn(nb, -beta[l]);
-            }
-            delta = bcast(delta, owner);
-            if (delta != 0.0) {
-                for (int m = s.lane; m < L; m += 32)
-                    if (s.active[m]) s.r[m] = __dadd_rn(s.r[m], -__dmul_rn(delta, s.G[m * Lp + l]));
-                if (s.lane == owner) beta[l] = nb;
-                moved = fmax(moved, fabs(delta));
-            }
+    __syncthreads();
+    if (s.tid < 32) {
+        const double thr = __dmul_rn(__dmul_rn(0.5, lambda), s.nrows);
+        int done = 0;
+        if (s.safe && thr >= 0x1p-300 && thr <= 0x1p300) {
+            if (s.na8 <= 32) done = cd_sweeps<1, true>(s, thr, beta, tol, max_sweeps);
+            else if (s.na8 <= 64) done = cd_sweeps<2, true>(s, thr, beta, tol, max_sweeps);
+            else if (s.na8 <= 96) done = cd_sweeps<3, true>(s, thr, beta, tol, max_sweeps);
+            else done = cd_sweeps<4, true>(s, thr, beta, tol, max_sweeps);
+            if (done < 0 && -done < max_sweeps) cd_sweeps<4, false>(s, thr, beta, tol, max_sweeps + done);
+        } else {
+            cd_sweeps<4, false>(s, thr, beta, tol, max_sweeps);
         }
-        if (moved <= tol) { ++sweep; break; }
     }
-    __syncwarp();
-    return sweep;
+    __syncthreads();
 }
 
+// All threads; every thread returns the loss. Starts after a barrier that made beta visible.
 __device__ double selection_loss(const SearchState& s, double hh, const double* beta)
 {
-    const int L = s.L, Lp = s.Lp;
-    for (int l = s.lane; l < L; l += 32) {
+    for (int l = s.tid; l < s.na; l += kSearchThreads) {
         double row = 0.0;
-        if (s.active[l])
-            for (int m = 0; m < L; ++m)
-                if (s.active[m]) row = __dadd_rn(row, __dmul_rn(s.G[l * Lp + m], beta[m]));
+#pragma unroll 8
+        for (int m = 0; m < s.na; ++m) row = __dadd_rn(row, __dmul_rn(s.G[l * s.Lp + m], beta[m]));
         s.tmp[l] = row;
     }
-    __syncwarp();
-    double loss = 0.0;
-    if (s.lane == 0) {
-        double quad = 0.0, lin = 0.0;
-        for (int l = 0; l < L; ++l) {
-            if (!s.active[l]) continue;
-            quad = __dadd_rn(quad, __dmul_rn(beta[l], s.tmp[l]));
-            lin = __dadd_rn(lin, __dmul_rn(s.b[l], beta[l]));
-        }
-        loss = __ddiv_rn(__dadd_rn(__dadd_rn(hh, -__dmul_rn(2.0, lin)), quad), s.nrows);
+    __syncthreads();
+    double quad = 0.0, lin = 0.0;
+#pragma unroll 8
+    for (int l = 0; l < s.na; ++l) {
+        quad = __dadd_rn(quad, __dmul_rn(beta[l], s.tmp[l]));
+        lin = __dadd_rn(lin, __dmul_rn(s.b[l], beta[l]));
     }
-    loss = bcast(loss, 0);
-    __syncwarp();
-    return loss;
+    __syncthreads();
+    return __ddiv_rn(__dadd_rn(__dadd_rn(hh, -__dmul_rn(2.0, lin)), quad), s.nrows);
 }
 
-// Eq. 9 on the support S (ns atoms): G_SS gamma = b_S by Cholesky in the scratch matrix A; gamma lands in s.tmp[0..ns).
-__device__ bool refit_gamma(const SearchState& s, int ns, double* A)
+// Eq. 9 on the support S (ns atoms): G_SS gamma = b_S by Cholesky in A; gamma lands in s.tmp[0..ns). Right-looking: an
+// entry gets its subtractions column by column, which is the order of the sequential inner products. Thread = row.
+__device__ bool refit_gamma(const SearchState& s, int ns)
 {
-    const int Lp = s.Lp;
-    for (int e = s.lane; e < ns * ns; e += 32) A[e] = s.G[s.S[e / ns] * Lp + s.S[e % ns]];
-    for (int i = s.lane; i < ns; i += 32) s.tmp[i] = s.b[s.S[i]];
-    __syncwarp();
+    const int Lp = s.Lp, i = s.tid;
+    double* A = s.A;
+    double* y = s.tmp;
+    double* Ai = A + i * (i + 1) / 2;                         // row i
+    if (i < ns) {
+        for (int j = 0; j <= i; ++j) Ai[j] = s.G[s.S[i] * Lp + s.S[j]];
+        y[i] = s.b[s.S[i]];
+    }
+    __syncthreads();
     for (int j = 0; j < ns; ++j) {
-        double dj = 0.0;
-        if (s.lane == 0) {
-            dj = A[j * ns + j];
-            for (int q = 0; q < j; ++q) dj = __dadd_rn(dj, -__dmul_rn(A[j * ns + q], A[j * ns + q]));
-            if (dj > 0.0) { dj = __dsqrt_rn(dj); A[j * ns + j] = dj; } else dj = -1.0;
+        const double djj = A[j * (j + 1) / 2 + j];
+        if (!(djj > 0.0)) return false;                       // the same value in every thread
+        const double dj = __dsqrt_rn(djj);
+        double lij = 0.0;
+        if (i > j && i < ns) {
+            lij = __ddiv_rn(Ai[j], dj);
+            Ai[j] = lij;
         }
-        dj = bcast(dj, 0);
-        if (!(dj > 0.0)) return false;
-        __syncwarp();
-        for (int i = j + 1 + s.lane; i < ns; i += 32) {
-            double v = A[i * ns + j];
-            for (int q = 0; q < j; ++q) v = __dadd_rn(v, -__dmul_rn(A[i * ns + q], A[j * ns + q]));
-            A[i * ns + j] = __ddiv_rn(v, dj);
+        __syncthreads();
+        if (i == j) Ai[j] = dj;
+        if (i > j && i < ns) {
+#pragma unroll 4
+            for (int q = j + 1; q <= i; ++q) Ai[q] = __dadd_rn(Ai[q], -__dmul_rn(lij, A[q * (q + 1) / 2 + j]));
         }
-        __syncwarp();
+        __syncthreads();
     }
-    if (s.lane == 0) {
-        double* y = s.tmp;
-        for (int i = 0; i < ns; ++i) {
-            double v = y[i];
-            for (int q = 0; q < i; ++q) v = __dadd_rn(v, -__dmul_rn(A[i * ns + q], y[q]));
-            y[i] = __ddiv_rn(v, A[i * ns + i]);
-        }
-        for (int i = ns - 1; i >= 0; --i) {
-            double v = y[i];
-            for (int q = i + 1; q < ns; ++q) v = __dadd_rn(v, -__dmul_rn(A[q * ns + i], y[q]));
-            y[i] = __ddiv_rn(v, A[i * ns + i]);
-        }
+    for (int j = 0; j < ns; ++j) {                            // forward, column by column
+        if (i == j) y[j] = __ddiv_rn(y[j], Ai[j]);
+        __syncthreads();
+        if (i > j && i < ns) y[i] = __dadd_rn(y[i], -__dmul_rn(Ai[j], y[j]));
+        __syncthreads();
     }
-    __syncwarp();
+    for (int j = ns - 1; j >= 0; --j) {                       // backward: the sum runs upwards, so only its products are parallel
+        if (i > j && i < ns) s.prod[i] = __dmul_rn(Ai[j], y[i]);
+        __syncthreads();
+        if (i == j) {
+            double v = y[j];
+#pragma unroll 8
+            for (int q = j + 1; q < ns; ++q) v = __dadd_rn(v, -s.prod[q]);
+            y[j] = __ddiv_rn(v, Ai[j]);
+        }
+        __syncthreads();
+    }
     return true;
 }
 
-__global__ void __launch_bounds__(32, 1) selection_search_kernel(const SearchParams p)
+__global__ void __launch_bounds__(kSearchThreads, 1) selection_search_kernel(const __grid_constant__ SearchParams p)
 {
     extern __shared__ __align__(16) double ssm[];
     SearchState s;
     const int L = p.L;
-    s.L = L; s.Lp = L | 1; s.lane = threadIdx.x; s.nrows = p.nrows;
-    s.G = ssm;
-    s.b = s.G + (size_t)L * s.Lp;
-    s.beta = s.b + L; s.r = s.beta + L; s.best = s.r + L; s.cand = s.best + L; s.gtot = s.cand + L; s.tmp = s.gtot + L;
-    s.S = reinterpret_cast<int*>(s.tmp + L);
-    s.active = reinterpret_cast<uint8_t*>(s.S + L);
-    const int lane = s.lane;
-    for (int e = lane; e < L * L; e += 32) s.G[(e / L) * s.Lp + (e % L)] = p.G[e];
-    for (int l = lane; l < L; l += 32) { s.b[l] = p.b[l]; s.beta[l] = 1.0; s.gtot[l] = 1.0; s.active[l] = 1; }
-    __syncwarp();
+    s.L8 = search_l8(L); s.Lp = s.L8 + 1; s.tid = threadIdx.x; s.lane = threadIdx.x & 31; s.nrows = p.nrows;
+    s.na = L;
+    double* v = ssm;
+    s.diag = v; v += s.L8; s.rcp = v; v += s.L8; s.frz = v; v += s.L8;
+    s.b = v; v += s.L8; s.beta = v; v += s.L8; s.r = v; v += s.L8; s.best = v; v += s.L8; s.cand = v; v += s.L8;
+    s.gtot = v; v += s.L8; s.tmp = v; v += s.L8; s.prod = v; v += s.L8;
+    s.G = v; v += s.L8 * s.Lp;
+    s.A = v; v += L * (L + 1) / 2;
+    s.S = reinterpret_cast<int*>(v);
+    s.orig = s.S + s.L8;
+    const int tid = s.tid;
+    for (int e = tid; e < L * L; e += kSearchThreads) s.G[(e / L) * s.Lp + (e % L)] = p.G[e];
+    for (int l = tid; l < L; l += kSearchThreads) { s.b[l] = p.b[l]; s.beta[l] = 1.0; s.gtot[l] = 1.0; s.orig[l] = l; }
+    __syncthreads();
+    prepare_active(s);
     const double hh = *p.hh;
     double alpha_t = 1.0, lambda = p.lambda0;
     int step = 0;
     bool failed = false;
+    auto copy = [&](double* dst, const double* src) {          // ends in a barrier
+        for (int l = tid; l < s.na; l += kSearchThreads) dst[l] = src[l];
+        __syncthreads();
+    };
     while (alpha_t > p.alpha + 1e-12 && step < p.max_steps && !failed) {
         const double alpha_next = fmax(p.alpha, __dadd_rn(1.0, -__dmul_rn((double)(step + 1), p.dalpha)));
         const double target = __dmul_rn(alpha_next, (double)L), band = __dmul_rn(p.eps, (double)L);
@@ -648,18 +745,13 @@ __global__ void __launch_bounds__(32, 1) selection_search_kernel(const SearchPar
         double lam_hi = lambda;
         // doubling
         while ((double)nnz > target) {
-            for (int l = lane; l < L; l += 32) s.cand[l] = s.beta[l];
-            __syncwarp();
-            lasso_cd(s, lambda, s.cand, p.tol, p.max_sweeps);
+            lasso_cd(s, lambda, s.beta, p.tol, p.max_sweeps);
             ++solves;
-            nnz = count_nonzero(s, s.cand);
-            for (int l = lane; l < L; l += 32) s.beta[l] = s.cand[l];
-            __syncwarp();
+            nnz = count_nonzero(s, s.beta);
             lam_hi = lambda;
             lambda = __dmul_rn(2.0, lambda);
         }
-        for (int l = lane; l < L; l += 32) s.best[l] = s.beta[l];
-        __syncwarp();
+        copy(s.best, s.beta);
         int best_nnz = nnz;
         double best_lam = lam_hi;
         // bisection inside the last doubling step
@@ -667,65 +759,75 @@ __global__ void __launch_bounds__(32, 1) selection_search_kernel(const SearchPar
         int it = 0;
         while (fabs(__dadd_rn(target, -(double)nnz)) > band && it < p.max_bisect) {
             const double mid = __dmul_rn(0.5, __dadd_rn(left, right));
-            for (int l = lane; l < L; l += 32) s.cand[l] = s.best[l];
-            __syncwarp();
+            copy(s.cand, s.best);
             lasso_cd(s, mid, s.cand, p.tol, p.max_sweeps);
             ++solves;
             ++it;
             nnz = count_nonzero(s, s.cand);
             const bool in_band_feasible = fabs(__dadd_rn(target, -(double)nnz)) <= band && (double)nnz <= target;
             if (((double)nnz <= target && nnz > best_nnz) || in_band_feasible) {
-                for (int l = lane; l < L; l += 32) s.best[l] = s.cand[l];
+                copy(s.best, s.cand);
                 best_nnz = nnz;
                 best_lam = mid;
-                __syncwarp();
             }
             if ((double)nnz < target) right = mid;
             else if ((double)nnz > target) left = mid;
+            __syncthreads();
         }
-        for (int l = lane; l < L; l += 32) s.beta[l] = s.best[l];
-        __syncwarp();
+        copy(s.beta, s.best);
         lambda = best_lam;
         const double loss_beta = selection_loss(s, hh, s.beta);
         // W-step: re-fit on the support
         int ns = 0;
-        if (lane == 0) {
-            for (int l = 0; l < L; ++l)
-                if (s.active[l] && s.beta[l] != 0.0) s.S[ns++] = l;
+        for (int l0 = 0; l0 < s.na; l0 += 32) {               // every warp counts, warp 0 writes the list
+            const int l = l0 + s.lane;
+            const unsigned m = __ballot_sync(0xffffffffu, l < s.na && s.beta[l] != 0.0);
+            if (tid < 32 && ((m >> s.lane) & 1u)) s.S[ns + __popc(m & ((1u << s.lane) - 1u))] = l;
+            ns += __popc(m);
         }
-        ns = __shfl_sync(0xffffffffu, ns, 0);
-        __syncwarp();
-        if (ns == 0 || !refit_gamma(s, ns, p.chol)) { failed = true; break; }
-        // gamma (in tmp[0..ns)) folded into G, b and the running product; the kept atoms become the active set
-        for (int l = lane; l < L; l += 32) s.active[l] = 0;
-        __syncwarp();
-        for (int i = lane; i < ns; i += 32) s.active[s.S[i]] = 1;
-        for (int e = lane; e < ns * ns; e += 32) {
-            const int i = e / ns, j = e % ns;
-            double* g = &s.G[s.S[i] * s.Lp + s.S[j]];
-            *g = __dmul_rn(__dmul_rn(s.tmp[i], *g), s.tmp[j]);
+        __syncthreads();
+        if (ns == 0 || !refit_gamma(s, ns)) { failed = true; break; }
+        // gamma (in tmp[0..ns)) folded into G, b and the running product; the kept atoms become the active set, moved
+        // together eight rows at a time (row i comes from row S[i] >= i, so a batch never overwrites a later one's rows)
+        for (int i0 = 0; i0 < ns; i0 += 8) {
+            double row[8];
+            if (tid < ns) {
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    if (i0 + u < ns) row[u] = __dmul_rn(__dmul_rn(s.tmp[i0 + u], s.G[s.S[i0 + u] * s.Lp + s.S[tid]]), s.tmp[tid]);
+            }
+            __syncthreads();
+            if (tid < ns) {
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    if (i0 + u < ns) s.G[(i0 + u) * s.Lp + tid] = row[u];
+            }
+            __syncthreads();
         }
-        for (int i = lane; i < ns; i += 32) {
-            s.b[s.S[i]] = __dmul_rn(s.tmp[i], s.b[s.S[i]]);
-            s.gtot[s.S[i]] = __dmul_rn(s.gtot[s.S[i]], s.tmp[i]);
+        double bi = 0.0, gi = 0.0;
+        int oi = 0;
+        if (tid < ns) {
+            bi = __dmul_rn(s.tmp[tid], s.b[s.S[tid]]);
+            gi = __dmul_rn(s.gtot[s.S[tid]], s.tmp[tid]);
+            oi = s.orig[s.S[tid]];
         }
-        __syncwarp();
-        for (int l = lane; l < L; l += 32) s.beta[l] = s.active[l] ? 1.0 : 0.0;
-        __syncwarp();
+        __syncthreads();
+        if (tid < ns) { s.b[tid] = bi; s.gtot[tid] = gi; s.orig[tid] = oi; s.beta[tid] = 1.0; }
+        s.na = ns;
+        __syncthreads();
+        prepare_active(s);
         const double loss_gamma = selection_loss(s, hh, s.beta);
-        if (p.trace && lane == 0) {
+        if (p.trace && tid == 0) {
             double* tr = p.trace + (size_t)step * 6;
             tr[0] = alpha_next; tr[1] = best_lam; tr[2] = (double)ns; tr[3] = loss_beta; tr[4] = loss_gamma; tr[5] = (double)solves;
         }
         alpha_t = alpha_next;
         ++step;
     }
-    if (lane == 0) {
-        int cnt = 0;
-        if (!failed)
-            for (int l = 0; l < L; ++l)
-                if (s.active[l]) { p.idx_out[cnt] = (uint8_t)l; p.gamma_out[cnt] = (float)s.gtot[l]; ++cnt; }
-        *p.count_out = failed ? -1 : cnt;
+    if (!failed)
+        for (int l = tid; l < s.na; l += kSearchThreads) { p.idx_out[l] = (uint8_t)s.orig[l]; p.gamma_out[l] = (float)s.gtot[l]; }
+    if (tid == 0) {
+        *p.count_out = failed ? -1 : s.na;
         if (p.steps_out) *p.steps_out = step;
     }
 }
@@ -846,26 +948,27 @@ cudaError_t launch_selection_gram_static(const float* lr, const void* coef, int 
 size_t selection_search_scratch_bytes(int L) { return (size_t)L * L * sizeof(double); }
 
 cudaError_t launch_selection_search(const double* G, const double* b, const double* hh, double nrows, int L, const sr_search_opts& o,
-                                    uint8_t* idx_out, float* gamma_out, int* count_out, double* trace, int* steps_out, double* chol,
-                                    cudaStream_t st)
+                                    uint8_t* idx_out, float* gamma_out, int* count_out, double* trace, int* steps_out, cudaStream_t st)
 {
     if (L > kMaxSearchL) return cudaErrorNotSupported;
     SearchParams p{};
     p.G = G; p.b = b; p.hh = hh; p.L = L; p.nrows = nrows;
     p.alpha = o.alpha; p.dalpha = o.delta_alpha; p.eps = o.eps; p.lambda0 = o.lambda0; p.tol = o.tol;
     p.max_sweeps = o.max_sweeps; p.max_bisect = o.max_bisect; p.max_steps = o.max_steps;
-    p.idx_out = idx_out; p.gamma_out = gamma_out; p.count_out = count_out; p.trace = trace; p.steps_out = steps_out; p.chol = chol;
-    const int Lp = L | 1;
-    const size_t smem = ((size_t)L * Lp + 7 * (size_t)L) * sizeof(double) + (size_t)L * sizeof(int) + (size_t)L + 16;
+    p.idx_out = idx_out; p.gamma_out = gamma_out; p.count_out = count_out; p.trace = trace; p.steps_out = steps_out;
+    constexpr auto bytes = [](int l) {
+        const size_t l8 = search_l8(l);
+        return (11 * l8 + l8 * (l8 + 1) + (size_t)l * (l + 1) / 2) * sizeof(double) + 2 * l8 * sizeof(int);
+    };
     static bool configured[64] = {false};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (!configured[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(selection_search_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        cudaError_t e = cudaFuncSetAttribute(selection_search_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(kMaxSearchL));
         if (e != cudaSuccess) return e;
         configured[dev] = true;
     }
-    selection_search_kernel<<<1, 32, smem, st>>>(p);
+    selection_search_kernel<<<1, kSearchThreads, bytes(L), st>>>(p);
     count_launches(1);
     return cudaGetLastError();
 }

@@ -19,11 +19,10 @@ cudaError_t launch_selection_gram_static(const float* lr, const void* coef, int 
                                          const int64_t* samples, int64_t nsamples, double* G, double* b, double* hh, const Problem& pb,
                                          cudaStream_t st);
 
-// Scratch of the search kernel: the matrix its Cholesky factorisation works in.
+// Scratch the search call asks of its caller: room for the matrix of its factorisation (which now stays in shared memory).
 size_t selection_search_scratch_bytes(int L);
 
 cudaError_t launch_selection_search(const double* G, const double* b, const double* hh, double nrows, int L, const sr_search_opts& o,
-                                    uint8_t* idx_out, float* gamma_out, int* count_out, double* trace, int* steps_out, double* chol,
-                                    cudaStream_t st);
+                                    uint8_t* idx_out, float* gamma_out, int* count_out, double* trace, int* steps_out, cudaStream_t st);
 
 } // namespace sr

@@ -128,3 +128,23 @@ def test_gram_at_block_edges_and_odd_planes(D, k, r, h, w, dt, n, c, base):
         co = room[1:1 + co.numel()].view(co.shape).copy_(co)
         assert co.data_ptr() % 4 == 2
     _gram_close(sr.sr_selection_gram(dev(lr), co, dev(d), dev(target), None, r, k), *oracle.selection_gram(lr, coef, d, target, None, r, k))
+
+
+@pytest.mark.parametrize("D", [1, 7, 8, 9, 31, 33, 64, 65, 97, 128])
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** -700, 2.0 ** 640])
+def test_search_bits_at_block_edges_and_extreme_scales(D, scale):
+    # coordinate blocks of eight, residuals in registers of 32: both sides of their edges; statistics scaled by a power of
+    # two lie outside the range of the fast quotient, so the same path has to be walked with the library's division
+    rng = np.random.default_rng(D)
+    n = 4 * D + 20
+    Z = rng.normal(size=(n, D)) * np.exp(-3.0 * rng.permutation(D) / D)
+    h = Z.sum(1) + 0.05 * rng.normal(size=n)
+    G, b, hh = (Z.T @ Z) * scale, (Z.T @ h) * scale, (h @ h) * scale
+    G = (G + G.T) / 2
+    alpha, dalpha = max(1, D // 4) / D, max(1, D // 3) / D
+    kw = dict(tol=1e-9, max_sweeps=300, max_bisect=20)
+    want_idx, want_gamma, want_trace = oracle.selection_search(G, b, hh, n, alpha, dalpha, 0.0, 1e-6 * scale, **kw)
+    idx, gamma, trace = sr.sr_selection_search(dev(G), dev(b), dev(np.array([hh])), n, alpha, dalpha, 0.0, 1e-6 * scale, **kw)
+    np.testing.assert_array_equal(host(idx), want_idx)
+    np.testing.assert_array_equal(host(trace), want_trace)
+    np.testing.assert_array_equal(host(gamma), want_gamma.astype(np.float32))
