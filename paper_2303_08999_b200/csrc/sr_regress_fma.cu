@@ -6,6 +6,7 @@
 // (dictionary rows broadcast from shared memory), then y_c = F . B_c against an up-sampled tile with a
 // halo of p = (k-1)/2 that lives only in shared memory. Neither F nor the patch matrix B reaches HBM.
 #include "sr_common.cuh"
+#include "sr_regress_tile.cuh"
 
 namespace sr {
 
@@ -61,8 +62,16 @@ regress_fma_kernel(const float* __restrict__ lr, const CoefT* __restrict__ coef,
     };
     if (MODE == kModeDense) {
         const CoefT* cp = coef + (int64_t)f * D * HW + pix;
-#pragma unroll 4
-        for (int l = 0; l < D; ++l) accumulate(l, load_coef(cp, (int64_t)l * HW));
+        constexpr int AHEAD = 12;                            // loads in flight: small frames wait for nothing else
+        int l0 = 0;
+        for (; l0 + AHEAD <= D; l0 += AHEAD) {
+            float v[AHEAD];
+#pragma unroll
+            for (int u = 0; u < AHEAD; ++u) v[u] = load_coef(cp, (int64_t)(l0 + u) * HW);
+#pragma unroll
+            for (int u = 0; u < AHEAD; ++u) accumulate(l0 + u, v[u]);
+        }
+        for (; l0 < D; ++l0) accumulate(l0, load_coef(cp, (int64_t)l0 * HW));
     } else if (MODE == kModeIdx) {
         for (int q = 0; q < s; ++q) {
             const int a = min((int)__ldg(idx + ((int64_t)f * s + q) * HW + pix), D - 1);
@@ -191,6 +200,7 @@ cudaError_t launch_k(int mode, const float* lr, const void* coef, const uint8_t*
 cudaError_t launch_regress_fma(int mode, const float* lr, const void* coef, int coef_dtype, const uint8_t* idx,
                                const float* gamma, const float* dict, float* out, const Problem& pb, cudaStream_t st)
 {
+    if (regress_tile_supported(mode, coef_dtype, pb)) return launch_regress_tile(mode, lr, coef, idx, gamma, dict, out, pb, st);
     if (coef_dtype == SR_F16) return launch_k<__half>(mode, lr, coef, idx, gamma, dict, out, pb, st);
     return launch_k<float>(mode, lr, coef, idx, gamma, dict, out, pb, st);
 }

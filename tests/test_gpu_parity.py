@@ -306,3 +306,31 @@ def test_dictionary_magnitude_range_of_the_tensor_core_path(scale, bound):
     assert max_abs_err(got, oracle.dict_regress_dense(lr, coef, dict_, 2, 5)) <= bound
     got = host(sr.sr_dict_regress_selected(dev(lr), dev(coef), None, None, dev(dict_), 2, 5, 8))
     assert max_abs_err(got, oracle.dict_regress_selected(lr, coef, None, None, dict_, 2, 5, 8)) <= bound
+
+
+TILE_CASES = [  # k, c, h, w, scale, D: fp32 frames large enough for the register-tiled kernel, every atom size, both copy widths
+    (1, 1, 260, 300, 1, 5), (3, 3, 130, 161, 2, 9), (5, 3, 101, 87, 3, 72), (5, 4, 70, 69, 4, 7), (7, 3, 100, 95, 3, 16), (9, 2, 80, 64, 4, 8),
+    (5, 3, 97, 100, 3, 20), (5, 2, 280, 281, 1, 2)]
+
+
+@pytest.mark.parametrize("case", TILE_CASES, ids=lambda c: "-".join(map(str, c)))
+def test_register_tiled_fp32_dense_and_subset(case):
+    k, c, h, w, r, D = case
+    wl = sr_inputs.Workload("tile", 1, c, h, w, r, D=D, k=k, coef_dtype="f32")
+    lr, d, coef = sr_inputs.make_inputs(wl)
+    # (differences of Gaussians of one tap are 0 / 0: random atoms there)
+    d = signed_asymmetric_dictionary(d, seed=k) if k > 1 else np.random.default_rng(k).uniform(-1, 1, d.shape).astype(np.float32)
+    assert wl.npix >= 148 * 512
+    out = host(sr.sr_dict_regress_dense(dev(lr), dev(coef), dev(d), r, k))
+    assert max_abs_err(out, oracle.dict_regress_dense(lr, coef, d, r, k)) <= TOL_F32
+    s = min(D, 3)
+    S, gamma = np.arange(D - 1, D - 1 - s, -1).astype(np.uint8), signed_gamma(s)
+    want = oracle.dict_regress_selected(lr, coef, S, gamma, d, r, k, s, flags=oracle.IDX_GLOBAL)
+    got = host(sr.sr_dict_regress_selected(dev(lr), dev(coef), dev(S), dev(gamma), dev(d), r, k, s, sr.SR_IDX_GLOBAL))
+    assert max_abs_err(got, want) <= TOL_F32
+    # an unaligned view of the same planes (single-word copies) and the kept planes alone
+    room = torch.zeros(coef.size + 4, dtype=torch.float32, device="cuda")
+    view = room[1:1 + coef.size].view(coef.shape).copy_(dev(coef))
+    np.testing.assert_array_equal(host(sr.sr_dict_regress_dense(dev(lr), view, dev(d), r, k)), out)
+    kept = dev(np.ascontiguousarray(coef[:, S]))
+    np.testing.assert_array_equal(host(sr.sr_dict_regress_selected(dev(lr), kept, dev(S), dev(gamma), dev(d), r, k, s, sr.SR_IDX_GLOBAL | sr.SR_COEF_COMPACT)), got)
