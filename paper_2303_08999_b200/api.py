@@ -100,12 +100,29 @@ def status_string(status: int) -> str:
     return load_library().sr_status_string(status).decode()
 
 
+# Small calls are bound by this file, not by their kernels, so the per-call path asks torch for the raw handle of the
+# current stream (torch.cuda.current_stream() builds a Stream object around it: 3.2 us against 0.2).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_get_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    if _raw_stream is None or _get_device is None or not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_get_device())
 
 
 def _ptr(t):
     return None if t is None else t.data_ptr()
+
+
+def _out_like(lr: torch.Tensor, shape, dtype, out):
+    """`out` checked, or a new tensor on lr's device."""
+    if out is None:
+        return lr.new_empty(shape) if dtype is torch.float32 else torch.empty(shape, dtype=dtype, device=lr.device)
+    _dev(out, dtype, "out")
+    assert out.shape == shape
+    return out
 
 
 def _dev(t: torch.Tensor, dtype, what: str) -> torch.Tensor:
@@ -134,12 +151,11 @@ def _check(status: int, what: str):
 def _upsample(name: str, lr: torch.Tensor, scale: int, out: torch.Tensor | None) -> torch.Tensor:
     lr = _dev(lr, torch.float32, "lr")
     n, c, h, w = lr.shape
-    if out is None:
-        out = torch.empty((n, c, h * scale, w * scale), dtype=torch.float32, device=lr.device)
-    _dev(out, torch.float32, "out")
-    assert out.shape == (n, c, h * scale, w * scale)
+    out = _out_like(lr, (n, c, h * scale, w * scale), torch.float32, out)
     d = sr_dims(n, c, h, w, scale, 1, 1)
-    _check(getattr(load_library(), name)(_ptr(lr), _ptr(out), ctypes.byref(d), _stream()), name)
+    status = getattr(_lib or load_library(), name)(lr.data_ptr(), out.data_ptr(), ctypes.byref(d), _stream())
+    if status:
+        raise SrError(status, name)
     return out
 
 
@@ -157,15 +173,14 @@ def sr_dict_regress_dense(lr, coef, dict_, scale: int, k: int, flags: int = 0, o
     _dev(coef, coef.dtype, "coef")
     n, c, h, w = lr.shape
     D = dict_.shape[0]
-    assert dict_.shape == (D, k * k) and coef.shape == (n, D, h * scale, w * scale)
-    out_dtype = _out_dtype(flags)
-    if out is None:
-        out = torch.empty((n, c, h * scale, w * scale), dtype=out_dtype, device=lr.device)
-    _dev(out, out_dtype, "out")
-    assert out.shape == (n, c, h * scale, w * scale)
+    H, W = h * scale, w * scale
+    assert dict_.shape == (D, k * k) and coef.shape == (n, D, H, W)
+    out = _out_like(lr, (n, c, H, W), _out_dtype(flags), out)
     d = sr_dims(n, c, h, w, scale, k, D)
-    _check(load_library().sr_dict_regress_dense(_ptr(lr), _ptr(coef), code, _ptr(dict_), _ptr(out), ctypes.byref(d),
-                                                flags, _stream()), "sr_dict_regress_dense")
+    status = (_lib or load_library()).sr_dict_regress_dense(lr.data_ptr(), coef.data_ptr(), code, dict_.data_ptr(), out.data_ptr(),
+                                                            ctypes.byref(d), flags, _stream())
+    if status:
+        raise SrError(status, "sr_dict_regress_dense")
     return out
 
 
@@ -181,8 +196,9 @@ def sr_dict_select(coef, s: int, want_sel: bool = False, idx=None, sel=None):
     if sel is not None:
         _dev(sel, coef.dtype, "sel")
     d = sr_dims(n, 1, H, W, 1, 1, D)
-    _check(load_library().sr_dict_select(_ptr(coef), code, _ptr(idx), _ptr(sel), ctypes.byref(d), s, 0, _stream()),
-           "sr_dict_select")
+    status = (_lib or load_library()).sr_dict_select(coef.data_ptr(), code, idx.data_ptr(), _ptr(sel), ctypes.byref(d), s, 0, _stream())
+    if status:
+        raise SrError(status, "sr_dict_select")
     return (idx, sel) if sel is not None else idx
 
 
@@ -199,16 +215,14 @@ def sr_dict_regress_selected(lr, coef_or_sel, idx, gamma, dict_, scale: int, k: 
     D = dict_.shape[0]
     assert dict_.shape == (D, k * k)
     planes = s if (flags & SR_COEF_COMPACT) else D
-    assert coef_or_sel.shape == (n, planes, h * scale, w * scale)
-    out_dtype = _out_dtype(flags)
-    if out is None:
-        out = torch.empty((n, c, h * scale, w * scale), dtype=out_dtype, device=lr.device)
-    _dev(out, out_dtype, "out")
-    assert out.shape == (n, c, h * scale, w * scale)
+    H, W = h * scale, w * scale
+    assert coef_or_sel.shape == (n, planes, H, W)
+    out = _out_like(lr, (n, c, H, W), _out_dtype(flags), out)
     d = sr_dims(n, c, h, w, scale, k, D)
-    _check(load_library().sr_dict_regress_selected(_ptr(lr), _ptr(coef_or_sel), code, _ptr(idx), _ptr(gamma),
-                                                   _ptr(dict_), _ptr(out), ctypes.byref(d), s, flags, _stream()),
-           "sr_dict_regress_selected")
+    status = (_lib or load_library()).sr_dict_regress_selected(lr.data_ptr(), coef_or_sel.data_ptr(), code, _ptr(idx), _ptr(gamma),
+                                                               dict_.data_ptr(), out.data_ptr(), ctypes.byref(d), s, flags, _stream())
+    if status:
+        raise SrError(status, "sr_dict_regress_selected")
     return out
 
 
@@ -336,9 +350,9 @@ def sr_producer_regress(lr, feat, folded, scale: int, k: int, D: int, kc: int, f
         raise ValueError("feat must be [n][h][w][cin]")
     cin = feat.shape[3]
     if out is None:
-        out = torch.empty((n, c, h * scale, w * scale), dtype=_out_dtype(flags), device=lr.device)
+        out = _out_like(lr, (n, c, h * scale, w * scale), _out_dtype(flags), None)
     d = sr_dims(n, c, h, w, scale, k, D)
-    _check(load_library().sr_producer_regress(_ptr(lr), _ptr(feat), _ptr(folded), folded.numel(), _ptr(out), ctypes.byref(d), cin, kc,
+    _check((_lib or load_library()).sr_producer_regress(_ptr(lr), _ptr(feat), _ptr(folded), folded.numel(), _ptr(out), ctypes.byref(d), cin, kc,
                                               flags, _stream()), "sr_producer_regress")
     return out
 
