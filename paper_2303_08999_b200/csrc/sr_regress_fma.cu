@@ -6,6 +6,7 @@
 // (dictionary rows broadcast from shared memory), then y_c = F . B_c against an up-sampled tile with a
 // halo of p = (k-1)/2 that lives only in shared memory. Neither F nor the patch matrix B reaches HBM.
 #include "sr_common.cuh"
+#include "sr_regress_rows.cuh"
 #include "sr_regress_tile.cuh"
 
 namespace sr {
@@ -201,6 +202,7 @@ cudaError_t launch_regress_fma(int mode, const float* lr, const void* coef, int 
                                const float* gamma, const float* dict, float* out, const Problem& pb, cudaStream_t st)
 {
     if (regress_tile_supported(mode, coef_dtype, pb)) return launch_regress_tile(mode, lr, coef, idx, gamma, dict, out, pb, st);
+    if (regress_rows_supported(mode, coef_dtype, pb)) return launch_regress_rows(mode, lr, coef, idx, gamma, dict, out, pb, st);
     if (coef_dtype == SR_F16) return launch_k<__half>(mode, lr, coef, idx, gamma, dict, out, pb, st);
     return launch_k<float>(mode, lr, coef, idx, gamma, dict, out, pb, st);
 }

@@ -334,3 +334,47 @@ def test_register_tiled_fp32_dense_and_subset(case):
     np.testing.assert_array_equal(host(sr.sr_dict_regress_dense(dev(lr), view, dev(d), r, k)), out)
     kept = dev(np.ascontiguousarray(coef[:, S]))
     np.testing.assert_array_equal(host(sr.sr_dict_regress_selected(dev(lr), kept, dev(S), dev(gamma), dev(d), r, k, s, sr.SR_IDX_GLOBAL | sr.SR_COEF_COMPACT)), got)
+
+
+ROW_CASES = [  # k, n, c, h, w, scale, D: binary16 rows of any width; K-steps of 16 atoms and tiles of 64 x 8 on both sides of their edges
+    (5, 1, 3, 41, 43, 3, 72), (5, 2, 3, 9, 21, 3, 16), (5, 1, 1, 17, 65, 1, 17), (5, 1, 4, 5, 63, 1, 15), (3, 2, 3, 13, 33, 2, 1), (3, 1, 2, 27, 11, 4, 33),
+    (7, 1, 3, 19, 29, 3, 32), (7, 2, 1, 33, 67, 1, 40), (5, 1, 3, 3, 1, 5, 128), (5, 3, 3, 1, 1, 1, 256), (7, 1, 3, 30, 31, 2, 100), (5, 1, 3, 90, 101, 5, 24)]
+
+
+@pytest.mark.parametrize("case", ROW_CASES, ids=lambda c: "-".join(map(str, c)))
+@pytest.mark.parametrize("magnitude", [1.0, 2.0 ** 20, 2.0 ** -30])
+def test_binary16_rows_of_any_width(case, magnitude):
+    k, n, c, h, w, r, D = case
+    wl = sr_inputs.Workload("rows", n, c, h, w, r, D=D, k=k)
+    lr, d, coef = sr_inputs.make_inputs(wl)
+    d = (signed_asymmetric_dictionary(d, seed=k) * np.float32(magnitude)).astype(np.float32)
+    # the dictionary enters whole and sums are fp32: within the fp32 bound (D k^2 terms of at most 1.2 in all)
+    tol = TOL_F32 * magnitude
+    want = oracle.dict_regress_dense(lr, coef, d, r, k)
+    out = host(sr.sr_dict_regress_dense(dev(lr), dev(coef), dev(d), r, k))
+    assert max_abs_err(out, want) <= tol
+    # tensors that start in the upper half of a word, their last element alone in one
+    room = torch.zeros(coef.size + 8, dtype=torch.float16, device="cuda")
+    view = room[1:1 + coef.size].view(coef.shape).copy_(dev(coef))
+    np.testing.assert_array_equal(host(sr.sr_dict_regress_dense(dev(lr), view, dev(d), r, k)), out)
+    s = min(D, 9)                                             # nine: beyond the small-subset kernel
+    S, gamma = np.arange(D - 1, D - 1 - s, -1).astype(np.uint8), signed_gamma(s)
+    want = oracle.dict_regress_selected(lr, coef, S, gamma, d, r, k, s, flags=oracle.IDX_GLOBAL)
+    got = host(sr.sr_dict_regress_selected(dev(lr), view, dev(S), dev(gamma), dev(d), r, k, s, sr.SR_IDX_GLOBAL))
+    assert max_abs_err(got, want) <= tol
+    kept = dev(np.ascontiguousarray(coef[:, S]))
+    np.testing.assert_array_equal(host(sr.sr_dict_regress_selected(dev(lr), kept, dev(S), dev(gamma), dev(d), r, k, s, sr.SR_IDX_GLOBAL | sr.SR_COEF_COMPACT)), got)
+
+
+def test_binary16_rows_keep_a_non_finite_coefficient_to_its_pixel():
+    wl = sr_inputs.Workload("rows", 1, 3, 20, 27, 3, D=20, k=5)
+    lr, d, coef = sr_inputs.make_inputs(wl)
+    clean = host(sr.sr_dict_regress_dense(dev(lr), dev(coef), dev(d), 3, 5))
+    bad = coef.copy()
+    bad[0, 7, 30, 40] = np.inf
+    bad[0, 19, 31, 80] = np.nan
+    out = host(sr.sr_dict_regress_dense(dev(lr), dev(bad), dev(d), 3, 5))
+    hit = np.zeros(out.shape, bool)
+    hit[:, :, 30, 40] = hit[:, :, 31, 80] = True
+    np.testing.assert_array_equal(out[~hit], clean[~hit])
+    assert not np.isfinite(out[hit]).any()
