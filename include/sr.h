@@ -248,7 +248,9 @@ int sr_device_status(void* stream, int* out_status);
  * sr_dict_regress_dense / sr_dict_regress_selected with the same shape use it.  They synchronise `stream`, overwrite
  * `out`, and are meant to be called once per shape at start-up; inputs that are not larger than the L2 cache are timed
  * warm.  The per-pixel arithmetic does not depend on the tile shape, so results for one kernel are the same bits for
- * every shape.  *result (may be NULL) receives the choice.  sr_tune_reset forgets every recorded shape.
+ * every shape.  *result (may be NULL) receives the choice; kernel 0 has no launch shape, so where the host rules give a
+ * small frame to it, the call times it too and records nothing unless a searched shape is faster.  sr_tune_reset forgets
+ * every recorded shape.
  */
 typedef struct sr_tune_result {
     int32_t kernel;        /* 0 general FMA kernel, 1 first tensor-core layout, 2 second tensor-core layout, 3 subset
@@ -321,7 +323,7 @@ int64_t sr_set_wait_limit(int64_t cycles);
  * Test hook for the failure path, host-side injection: each of the next `launches` launches of the tensor-core
  * regression kernel leaves out one barrier arrival in its first thread block, so that one of its waits runs out
  * (set a small budget with sr_set_wait_limit first).  Nothing faults or spins without bound: the block gives up
- * as described above.  0 disarms.  Returns SR_OK, or SR_ERR_SHAPE for a negative count.  The paper has no counterpart.
+ * as described above.  0 disarms.  While armed, calls take a kernel that has such waits where one supports them.  Returns SR_OK, or SR_ERR_SHAPE for a negative count.  The paper has no counterpart.
  */
 int sr_test_lose_arrival(int launches);
 

@@ -9,6 +9,7 @@
 
 #include "sr_common.cuh"
 #include "sr_regress_listed.cuh"
+#include "sr_regress_rows.cuh"
 #include "sr_regress_subset.cuh"
 #include "sr_producer.cuh"
 #include "sr_regress_tc.cuh"
@@ -120,24 +121,59 @@ static bool bad_out_flags(uint32_t flags, const sr_dims* d)
     return ((flags & SR_OUT_F16) && (flags & SR_OUT_U8)) || ((flags & SR_LUMA_ONLY) && d->c != 3);
 }
 
+static long long hr_pixels(const Problem& pb) { return (long long)pb.n * pb.H * pb.W; }
+
+// Whether the frame is small enough for the row kernel (sr_regress_rows.cu) although the tensor-core layouts could take it:
+// it cuts a frame into 64 x 4 pieces where they need a 128 x 8 tile per CTA, but it works its atoms off four times slower,
+// so the limit falls with the number of atoms and taps. Device time, row kernel / better layout: 128 x 128, D = 16: k = 3
+// 6.5 / 9.3 us, k = 5 7.9 / 10.8, k = 7 9.2 / 11.8; D = 32: 7.7 / 9.6, 9.8 / 11.2, 11.2 / 12.4; D = 72, k = 5: 13.8 / 12.2.
+// The lines lie where the two meet (D = 16: k = 3 at 720p, k = 5 at 450 x 450, k = 7 at 300 x 300).
+static bool small_for_rows(const Problem& pb, int natoms)
+{
+    const long long px = hr_pixels(pb);
+    if (natoms <= 16) return px <= (pb.k == 3 ? 700000 : (pb.k == 5 ? 200000 : 80000));
+    if (natoms <= 32) return px <= (pb.k == 3 ? 100000 : (pb.k == 5 ? 80000 : 40000));
+    return false;
+}
+
 // Which tensor-core layout takes a dense launch. The second layout (sr_regress_tc.cu: channel-split epilogue, two CTAs
-// per SM, several rows per pipeline step) wins where the coefficient stream is light and the epilogue sets the pace:
-// few atoms, or 7 x 7 atoms with up to 32 of them; the first layout (sr_umma.cu) streams many atoms faster. Measured
-// on the 1080p sweep points (dense, D = 16 / 32 / 72 / 128; k = 3 / 5 / 7).
-static bool dense_prefers_second_layout(const Problem& pb) { return pb.D <= 16 || (pb.k == 7 && pb.D <= 32); }
+// per SM, several rows per pipeline step) has the smaller per-frame cost and the better epilogue for 7 x 7 atoms; the first
+// (sr_umma.cu) streams faster. 7 x 7: the second with up to 32 atoms (4K frame x2, D = 32: 315 against 383 us), and with any
+// number on frames below 600 000 pixels (128 x 128, D = 128: 15.7 / 18.5 us; 512 x 768: 46 / 51; 720p and above the first:
+// 4K, D = 72: 412 against 504). Up to 16 atoms of 5 x 5: the second between 300 000 and 1.5 million pixels (512 x 640:
+// 18.6 / 23.3; 720p: 32.8 / 36.5; 1080p: 60 / 57).
+static bool dense_prefers_second_layout(const Problem& pb)
+{
+    const long long px = hr_pixels(pb);
+    if (pb.k == 7) return pb.D <= 32 || px <= 600000;
+    return pb.k == 5 && pb.D <= 16 && px > 300000 && px <= 1500000;
+}
 
 // Which kernel takes a launch from index + value planes when both could. The gather kernel (sr_regress_listed.cu) pays
 // s * floor(k^2 / 4) 16-byte shared-memory gathers per pixel and nothing per atom of the dictionary; the first
 // tensor-core layout pays for clearing and filling a stage row of D coefficients per pixel and little per listed atom.
 // Measured on the 1080p sweep points and the 4K x2 batch (D = 16 / 32 / 72 / 128; k = 3 / 5 / 7; s = 4 / 8 / 16), both
 // kernels forced in turn: the gather kernel is 1.0 - 3.7 times faster wherever this returns true, and up to two times
-// slower at the far end (k = 7, s = 16, few atoms).
+// slower at the far end (k = 7, s = 16, few atoms). On frames that leave the first layout at most one 128 x 8 tile per SM
+// its time is flat and lower from about 52 gathers on (384 x 256, D = 72, k = 5: s = 8 15.3 / 17.4 us, s = 16 16.3 / 24.2).
+static int compact_gathers(const Problem& pb) { return pb.s * ((pb.k * pb.k + 3) / 4); }   // 16-byte units of dictionary per pixel
 static bool compact_prefers_listed(const Problem& pb)
 {
-    const int gathers = pb.s * ((pb.k * pb.k + 3) / 4);      // 16-byte units of dictionary per pixel
+    const int gathers = compact_gathers(pb);
+    if (pb.D <= 96 && gathers >= 52 && 2 * (long long)((pb.W + 127) / 128) * ((pb.H + 15) / 16) * pb.n <= sm_count()) return false;
     if (pb.D > 96 || gathers <= 52) return true;
     if (pb.D >= 64) return gathers <= 104 || (pb.r == 2 && gathers <= 112);
     return pb.r == 2 && gathers <= 56;
+}
+
+// Whether a small frame's index + value planes go to the general kernel, which replicates no dictionary and clears no
+// stage: its time is the work of one block per SM (device time, general / better of the others: 128 x 128, D = 72, k = 5,
+// s = 8: 9.0 / 15.0 us; 256 x 256: 12.8 / 15.1; 384 x 256: 16.7 / 15.3; s = 4 there 14.0 / 14.1; D = 32, k = 3, s = 16 there
+// 12.5 / 14.0).
+static bool compact_prefers_general(const Problem& pb)
+{
+    const long long px = hr_pixels(pb);
+    return px <= 100000 && px * compact_gathers(pb) <= 5200000;
 }
 
 // ---- which kernel runs a regression, and in which launch shape ----------------------------------------------------------
@@ -210,11 +246,16 @@ static bool kernel_supported(int kernel, const RegressArgs& a)
 // The host rules: small global subsets on the FMA-pipe subset kernel; per-pixel lists with their values on the gather
 // kernel; the second tensor-core layout for the other
 // global subsets and for dense launches with few atoms; the first layout for the rest it supports; else the general kernel.
-static int default_kernel(const RegressArgs& a)
+// `shaped`: only among the kernels whose launch shape can be searched (the general kernel has none). The same while a lost
+// arrival is armed: the general kernel has no wait that could run out.
+static int default_kernel(const RegressArgs& a, bool shaped = false)
 {
+    shaped = shaped || g_lose_arrival.load(std::memory_order_relaxed) > 0;
     const int forced = g_force_kernel.load(std::memory_order_relaxed);
     if (forced >= 0 && kernel_supported(forced, a)) return forced;
     if (kernel_supported(kKernelSubset, a)) return kKernelSubset;
+    if (!shaped && a.mode == kModeCompact && a.coef_dtype == SR_F16 && compact_prefers_general(a.pb)) return kKernelGeneral;
+    if (!shaped && small_for_rows(a.pb, a.pb.s) && regress_rows_supported(a.mode, a.coef_dtype, a.pb)) return kKernelGeneral;   // (dense: s = D)
     const bool first = kernel_supported(kKernelFirstLayout, a), second = kernel_supported(kKernelSecondLayout, a);
     if (kernel_supported(kKernelListed, a) && (!first || compact_prefers_listed(a.pb))) return kKernelListed;
     if (second && (a.mode == kModeGlobal || dense_prefers_second_layout(a.pb) || !first)) return kKernelSecondLayout;
@@ -312,7 +353,7 @@ static int tune_shape(const RegressArgs& a, int reps, sr_tune_result* res)
     if (cudaEventCreate(&e0) != cudaSuccess) return SR_ERR_CUDA;
     if (cudaEventCreate(&e1) != cudaSuccess) { cudaEventDestroy(e0); return SR_ERR_CUDA; }
     TuneChoice def;
-    def.kernel = default_kernel(a);
+    def.kernel = default_kernel(a, cands[0].kernel != kKernelGeneral);
     const float def_us = time_candidate(def, a, reps, e0, e1);
     int best = -1;
     float best_us = 0.f;
@@ -320,6 +361,10 @@ static int tune_shape(const RegressArgs& a, int reps, sr_tune_result* res)
         const float us = time_candidate(cands[i], a, reps, e0, e1);
         if (us > 0.f && (best < 0 || us < best_us)) { best = (int)i; best_us = us; }
     }
+    // a small frame that the host rules give to the general kernel stays there unless a searched shape beats it
+    TuneChoice small;
+    small.kernel = default_kernel(a);
+    const float small_us = small.kernel == def.kernel ? -1.f : time_candidate(small, a, reps, e0, e1);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (best < 0 || def_us < 0.f) return SR_ERR_CUDA;
@@ -327,7 +372,8 @@ static int tune_shape(const RegressArgs& a, int reps, sr_tune_result* res)
     if (def_us <= best_us) { pick = def; best_us = def_us; }        // the host rules' own choice stays unless something beat it
     {
         std::lock_guard<std::mutex> lock(g_tune_mu);
-        g_tune_table[tune_key(a.mode, a.coef_dtype, a.pb)] = pick;
+        if (small_us > 0.f && small_us <= best_us) g_tune_table.erase(tune_key(a.mode, a.coef_dtype, a.pb));
+        else g_tune_table[tune_key(a.mode, a.coef_dtype, a.pb)] = pick;
     }
     if (res) {
         res->kernel = pick.kernel;

@@ -404,9 +404,13 @@ template <int K> size_t plan_rows(RowParams& prm, const Problem& pb, int th)
 template <int K, int CTAS, bool GATHER>
 cudaError_t launch_g(RowParams& prm, const Problem& pb, cudaStream_t st)
 {
-    // two rows per warp and tile; one when that leaves blocks without a tile
-    size_t smem = plan_rows<K>(prm, pb, 2 * kWarps);
-    if (prm.g.num_tiles < sm_count() * CTAS) smem = plan_rows<K>(prm, pb, kWarps);
+    // rows per warp and tile: three where the taller tile leaves room for CTAS blocks and work for all of them (213 x 321
+    // x3: 62 us against 65 with two, 71 with one), else two, else one (123 x 129: 15.0 against 19.1)
+    size_t smem = 0;
+    for (int rows : {3, 2, 1}) {
+        smem = plan_rows<K>(prm, pb, rows * kWarps);
+        if (rows == 1 || (prm.g.num_tiles >= sm_count() * CTAS && (rows == 2 || CTAS * (smem + 2048) <= (size_t)227 * 1024))) break;
+    }
     if (smem > (size_t)kRowsSmemMax) return cudaErrorNotSupported;
     auto kern = regress_rows_kernel<K, CTAS, GATHER>;
     static bool configured[64] = {false};
