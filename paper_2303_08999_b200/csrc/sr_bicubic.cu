@@ -1,6 +1,6 @@
 // Stage 1 alone: bicubic up-sampling of every LR plane (Keys a = -0.75, half-pixel centres, edge clamp).
 // A thread produces a BS x BS block of HR pixels from one LR window, separably (bicubic_block_kernel): BS = 4 at scales
-// 1, 2 and 4, BS = 6 at scale 3, BS = r above. The direct 4 x 4 form (bicubic_kernel: one thread, four consecutive
+// 1, 2 and 4, BS = 6 or 3 at scale 3, BS = r above. The direct 4 x 4 form (bicubic_kernel: one thread, four consecutive
 // pixels of a row) remains for scales the block kernel is not instantiated for.
 // Vector stores when the row pitch allows it; the LR taps come through the read-only cache.
 #include "sr_common.cuh"
@@ -134,10 +134,11 @@ template <int R, int BS>
 static cudaError_t launch_block(const float* lr, float* hr, const Problem& pb, cudaStream_t st)
 {
     const int64_t bw = (pb.W + BS - 1) / BS, bh = (pb.H + BS - 1) / BS, planes = (int64_t)pb.n * pb.c;
-    // blocks per thread: as many (up to 8) as leave about twenty warps per SM (270 x 480 x4, threads per SM asked for:
-    // 256 8.0 us, 640 7.0, 1024 7.4, a block per thread 9.1; larger frames do not care below 1500)
+    // blocks per thread: as many as leave about twenty warps per SM (270 x 480 x4, threads per SM asked for: 256 8.0 us,
+    // 640 7.0, 1024 7.4, a block per thread 9.1), up to 4 (540 x 960 x4: 1 / 2 / 4 / 8 blocks 30.5 / 23.2 / 20.2 / 22.5 us;
+    // 705 x 1261 x3: 42.5 / 29.8 / 25.9 / 28.1; four frames 1080 x 1920 x2: 127 / 98 / 91 / 94)
     int64_t run = bw * bh * planes / ((int64_t)sm_count() * 640);
-    run = run < 1 ? 1 : (run > 8 ? 8 : run);
+    run = run < 1 ? 1 : (run > 4 ? 4 : run);
     const int64_t threads = bw * ((bh + run - 1) / run);
     const dim3 grid((unsigned)((threads + 127) / 128), (unsigned)(planes < 65535 ? planes : 65535));
     bicubic_block_kernel<R, BS><<<grid, 128, 0, st>>>(lr, hr, pb, (int)run);
@@ -150,7 +151,12 @@ cudaError_t launch_bicubic(const float* lr, float* hr, const Problem& pb, cudaSt
     switch (pb.r) {
     case 1: return launch_block<1, 4>(lr, hr, pb, st);
     case 2: return launch_block<2, 4>(lr, hr, pb, st);
-    case 3: return launch_block<3, 6>(lr, hr, pb, st);
+    case 3:
+        // 6 x 6 blocks store float2 but need an even width; rows of odd width and large frames take 3 x 3 blocks, whose
+        // smaller windows leave more warps (6 x 6 / 3 x 3, us: 180 x 320 3.9 / 4.6, 360 x 640 8.4 / 8.7, two planes
+        // 872 x 1736 30.0 / 28.5; odd widths 333 x 501 8.9 / 6.8, 705 x 1261 39.3 / 25.9)
+        if ((pb.W & 1) != 0 || (int64_t)pb.n * pb.c * pb.h * pb.w > 1000000) return launch_block<3, 3>(lr, hr, pb, st);
+        return launch_block<3, 6>(lr, hr, pb, st);
     case 4: return launch_block<4, 4>(lr, hr, pb, st);
     case 5: return launch_block<5, 5>(lr, hr, pb, st);
     case 6: return launch_block<6, 6>(lr, hr, pb, st);

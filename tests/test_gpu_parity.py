@@ -32,6 +32,11 @@ def test_bicubic(n, c, h, w, r):
     assert max_abs_err(got, want) <= 1e-6
 
 
+@pytest.mark.parametrize("n,c,h,w,r", [(2, 1, 720, 700, 3), (1, 3, 251, 401, 3), (1, 3, 271, 481, 4), (1, 2, 511, 515, 2)])
+def test_bicubic_runs_of_blocks(n, c, h, w, r):          # a thread walks several blocks; the last run is cut short
+    test_bicubic(n, c, h, w, r)
+
+
 # ------------------------------------------------------------------ dense
 
 DENSE_CASES = [
@@ -338,7 +343,10 @@ def test_register_tiled_fp32_dense_and_subset(case):
 
 ROW_CASES = [  # k, n, c, h, w, scale, D: binary16 rows of any width; K-steps of 16 atoms and tiles of 64 x 8 on both sides of their edges
     (5, 1, 3, 41, 43, 3, 72), (5, 2, 3, 9, 21, 3, 16), (5, 1, 1, 17, 65, 1, 17), (5, 1, 4, 5, 63, 1, 15), (3, 2, 3, 13, 33, 2, 1), (3, 1, 2, 27, 11, 4, 33),
-    (7, 1, 3, 19, 29, 3, 32), (7, 2, 1, 33, 67, 1, 40), (5, 1, 3, 3, 1, 5, 128), (5, 3, 3, 1, 1, 1, 256), (7, 1, 3, 30, 31, 2, 100), (5, 1, 3, 90, 101, 5, 24)]
+    (7, 1, 3, 19, 29, 3, 32), (7, 2, 1, 33, 67, 1, 40), (5, 1, 3, 3, 1, 5, 128), (5, 3, 3, 1, 1, 1, 256), (7, 1, 3, 30, 31, 2, 100), (5, 1, 3, 90, 101, 5, 24),
+    # from 32768 pixels the row kernel, below it the general one
+    (5, 2, 3, 41, 67, 3, 72), (5, 1, 1, 1, 32767, 1, 15), (5, 1, 1, 1, 32769, 1, 17), (3, 1, 4, 257, 129, 1, 33), (7, 1, 3, 63, 131, 2, 40), (7, 1, 2, 91, 91, 2, 128),
+    (3, 2, 3, 65, 67, 2, 1), (5, 1, 2, 33000, 1, 1, 16)]
 
 
 @pytest.mark.parametrize("case", ROW_CASES, ids=lambda c: "-".join(map(str, c)))
