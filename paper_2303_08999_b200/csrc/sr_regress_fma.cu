@@ -5,9 +5,10 @@
 // One thread per HR pixel, 32 x 8 pixel tiles. Per pixel: assemble the filter F = Phi_i D in registers
 // (dictionary rows broadcast from shared memory), then y_c = F . B_c against an up-sampled tile with a
 // halo of p = (k-1)/2 that lives only in shared memory. Neither F nor the patch matrix B reaches HBM.
-#include "sr_common.cuh"
+#include "sr_pick.cuh"
 #include "sr_regress_rows.cuh"
 #include "sr_regress_tile.cuh"
+#include <type_traits>
 
 namespace sr {
 
@@ -91,7 +92,28 @@ regress_fma_kernel(const float* __restrict__ lr, const CoefT* __restrict__ coef,
             const int64_t plane = compact ? ((int64_t)f * s + q) : ((int64_t)f * D + a);
             accumulate(a, g * load_coef(coef, plane * HW + pix));
         }
-    } else { // kModeFusedSelect: repeated scan for the next-largest key; any s, any D
+    } else if (s <= 16) { // kModeFusedSelect: the list in registers, its values fetched again (they are in L1 or L2 by now)
+        const CoefT* cp = coef + (int64_t)f * D * HW + pix;
+        uint32_t list[4] = {0, 0, 0, 0};                     // a byte per atom
+        auto pick = [&](auto tag) {
+            constexpr int S = decltype(tag)::value;
+            int atom[S];
+            pick_top<S, CoefT>(cp, HW, D, s, atom);
+#pragma unroll
+            for (int i = 0; i < S; ++i) list[i / 4] |= (uint32_t)atom[i] << (8 * (i % 4));
+        };
+        if (s <= 4) pick(std::integral_constant<int, 4>{});
+        else if (s <= 8) pick(std::integral_constant<int, 8>{});
+        else pick(std::integral_constant<int, 16>{});
+        for (int q = 0; q < s; ++q) {
+            const int a = (int)(list[0] & 255u);
+            list[0] = __funnelshift_r(list[0], list[1], 8);
+            list[1] = __funnelshift_r(list[1], list[2], 8);
+            list[2] = __funnelshift_r(list[2], list[3], 8);
+            list[3] >>= 8;
+            accumulate(a, load_coef(cp, (int64_t)a * HW));
+        }
+    } else { // longer lists: repeated scan for the next-largest key; any s, any D
         const CoefT* cp = coef + (int64_t)f * D * HW + pix;
         long long prev = 0x7FFFFFFFFFFFFFFFll;
         for (int q = 0; q < s; ++q) {

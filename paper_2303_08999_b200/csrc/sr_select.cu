@@ -2,7 +2,7 @@
 // Key of atom l = (bit pattern with the sign cleared) * 256 + (255 - l): one integer whose order is
 // exactly "larger magnitude first, then lower index"; keys of one pixel are distinct.
 //
-// Fast path (binary16 coefficients, s <= 16, even W): one thread owns two neighbouring pixels (one 4-byte load per
+// Fast path (binary16 coefficients, s <= 16, even H * W): one thread owns two neighbouring pixels (one 4-byte load per
 // plane, a full 128-byte line per warp), keeps their s best keys sorted in registers and merges every group of S
 // planes with branch-free sorting networks of integer max / min:
 //   sort the S new keys (19 compare-exchanges for S = 8), max against the reversed running list (S ops, gives a
@@ -11,7 +11,8 @@
 // The kernel is bound by the integer ALU rate or by HBM, whichever is slower for the shape.
 // With 16-byte aligned planes the block first stages its 256 pixels x D planes in shared memory (select_tilef_kernel)
 // and the threads read their words, and at the end the selected values, from there.
-#include "sr_common.cuh"
+// fp32 coefficients and planes of an odd number of pixels: one thread per pixel (sr_pick.cuh).
+#include "sr_pick.cuh"
 
 namespace sr {
 
@@ -28,62 +29,7 @@ __device__ __forceinline__ typename KeyOf<CoefT>::type make_key(CoefT v, int l)
     return (KeyT)(((KeyT)mag_bits(v) << 8) | (KeyT)(255 - l));
 }
 
-// ---- sorting networks on int keys (descending) -----------------------------------------------------------------------
-
-__device__ __forceinline__ void cx(int& a, int& b)    // afterwards a >= b
-{
-    const int hi = max(a, b), lo = min(a, b);
-    a = hi;
-    b = lo;
-}
-
-template <int S> __device__ __forceinline__ void sort_desc(int* k);
-
-template <> __device__ __forceinline__ void sort_desc<4>(int* k)
-{
-    cx(k[0], k[1]); cx(k[2], k[3]);
-    cx(k[0], k[2]); cx(k[1], k[3]);
-    cx(k[1], k[2]);
-}
-
-template <> __device__ __forceinline__ void sort_desc<8>(int* k)   // 19 exchanges
-{
-    cx(k[0], k[1]); cx(k[2], k[3]); cx(k[4], k[5]); cx(k[6], k[7]);
-    cx(k[0], k[2]); cx(k[1], k[3]); cx(k[4], k[6]); cx(k[5], k[7]);
-    cx(k[1], k[2]); cx(k[5], k[6]);
-    cx(k[0], k[4]); cx(k[1], k[5]); cx(k[2], k[6]); cx(k[3], k[7]);
-    cx(k[2], k[4]); cx(k[3], k[5]);
-    cx(k[1], k[2]); cx(k[3], k[4]); cx(k[5], k[6]);
-}
-
-// Sorts a bitonic sequence of S keys into descending order.
-template <int S> __device__ __forceinline__ void bitonic_merge_desc(int* k)
-{
-#pragma unroll
-    for (int d = S / 2; d >= 1; d >>= 1)
-#pragma unroll
-        for (int i = 0; i < S; ++i)
-            if ((i & d) == 0) cx(k[i], k[i + d]);
-}
-
-template <> __device__ __forceinline__ void sort_desc<16>(int* k)   // two sorted halves, then a bitonic merge
-{
-    sort_desc<8>(k);
-    sort_desc<8>(k + 8);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) { const int t = k[8 + i]; k[8 + i] = k[15 - i]; k[15 - i] = t; }   // second half ascending
-    bitonic_merge_desc<16>(k);
-}
-
-// top[] (sorted) <- the S best of top[] and grp[] (grp sorted descending)
-template <int S> __device__ __forceinline__ void merge_top(int* top, const int* grp)
-{
-#pragma unroll
-    for (int i = 0; i < S; ++i) top[i] = max(top[i], grp[S - 1 - i]);
-    bitonic_merge_desc<S>(top);
-}
-
-// Two pixels per thread, binary16, s <= S, W even.
+// Two pixels per thread, binary16, s <= S, H * W even (a pair may span two rows).
 template <int S>
 __global__ void __launch_bounds__(256)
 select_pair_kernel(const __half* __restrict__ coef, uint8_t* __restrict__ idx, __half* __restrict__ sel,
@@ -100,7 +46,7 @@ select_pair_kernel(const __half* __restrict__ coef, uint8_t* __restrict__ idx, _
 #pragma unroll
         for (int i = 0; i < S; ++i) ta[i] = tb[i] = -1;
         const uint32_t* wp = reinterpret_cast<const uint32_t*>(cp);      // one word = the pair's coefficients of a plane
-        const int64_t wstride = HW / 2;                                   // words between planes (W is even)
+        const int64_t wstride = HW / 2;                                   // words between planes (H * W is even)
         int l0 = 0;
         for (; l0 + S <= D; l0 += S) {                                   // whole groups: no per-key guards
             uint32_t w[S];
@@ -359,38 +305,27 @@ select_tilef_kernel(const __half* __restrict__ coef, uint8_t* __restrict__ idx, 
     }
 }
 
-// s <= SMAX: sorted list in registers, one branch-free insertion per atom (any dtype, any W).
-template <typename CoefT, int SMAX>
+// s <= S, any dtype, any size: one thread per pixel.
+// Blocks run in order over the planes, one wave after the other (see launch_pair).
+template <typename CoefT, int S>
 __global__ void __launch_bounds__(256)
-select_insert_kernel(const CoefT* __restrict__ coef, uint8_t* __restrict__ idx, CoefT* __restrict__ sel,
-                     const __grid_constant__ Problem pb)
+select_pick_kernel(const CoefT* __restrict__ coef, uint8_t* __restrict__ idx, CoefT* __restrict__ sel,
+                   const __grid_constant__ Problem pb)
 {
-    using KeyT = typename KeyOf<CoefT>::type;
     const int64_t HW = (int64_t)pb.H * pb.W;
     const int64_t total = (int64_t)pb.n * HW;
-    const int D = pb.D, s = pb.s;
+    const int s = pb.s;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
         const int64_t f = t / HW, pix = t - f * HW;
-        const CoefT* cp = coef + f * D * HW + pix;
-        KeyT top[SMAX];
+        const CoefT* cp = coef + f * pb.D * HW + pix;
+        int atom[S];
+        pick_top<S, CoefT>(cp, HW, pb.D, s, atom);
+        const int64_t o = f * s * HW + pix;
 #pragma unroll
-        for (int i = 0; i < SMAX; ++i) top[i] = (KeyT)-1;
-#pragma unroll 4
-        for (int l = 0; l < D; ++l) {
-            KeyT x = make_key<CoefT>(__ldg(cp + (int64_t)l * HW), l);
-#pragma unroll
-            for (int i = 0; i < SMAX; ++i) {
-                const KeyT hi = max(top[i], x);
-                x = min(top[i], x);
-                top[i] = hi;
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < SMAX; ++q) {
+        for (int q = 0; q < S; ++q) {
             if (q < s) {
-                const int a = 255 - (int)(top[q] & 255);
-                idx[(f * s + q) * HW + pix] = (uint8_t)a;
-                if (sel) sel[(f * s + q) * HW + pix] = __ldg(cp + (int64_t)a * HW);
+                idx[o + q * HW] = (uint8_t)atom[q];
+                if (sel) sel[o + q * HW] = __ldg(cp + (int64_t)atom[q] * HW);
             }
         }
     }
@@ -427,15 +362,14 @@ template <typename CoefT>
 cudaError_t launch_sel(const void* coef, uint8_t* idx, void* sel, const Problem& pb, cudaStream_t st)
 {
     const int64_t total = (int64_t)pb.n * pb.H * pb.W;
-    int64_t blocks = (total + 255) / 256;
-    const int64_t cap = (int64_t)sm_count() * 64;
-    if (blocks > cap) blocks = cap;
+    const int64_t all = (total + 255) / 256, cap = (int64_t)sm_count() * 64;
+    const unsigned ordered = (unsigned)(all < 0x7FFFFFFF ? all : 0x7FFFFFFF), blocks = (unsigned)(all < cap ? all : cap);
     const CoefT* c = (const CoefT*)coef;
     CoefT* sl = (CoefT*)sel;
-    if (pb.s <= 4) select_insert_kernel<CoefT, 4><<<(unsigned)blocks, 256, 0, st>>>(c, idx, sl, pb);
-    else if (pb.s <= 8) select_insert_kernel<CoefT, 8><<<(unsigned)blocks, 256, 0, st>>>(c, idx, sl, pb);
-    else if (pb.s <= 16) select_insert_kernel<CoefT, 16><<<(unsigned)blocks, 256, 0, st>>>(c, idx, sl, pb);
-    else select_scan_kernel<CoefT><<<(unsigned)blocks, 256, 0, st>>>(c, idx, sl, pb);
+    if (pb.s <= 4) select_pick_kernel<CoefT, 4><<<ordered, 256, 0, st>>>(c, idx, sl, pb);
+    else if (pb.s <= 8) select_pick_kernel<CoefT, 8><<<ordered, 256, 0, st>>>(c, idx, sl, pb);
+    else if (pb.s <= 16) select_pick_kernel<CoefT, 16><<<ordered, 256, 0, st>>>(c, idx, sl, pb);
+    else select_scan_kernel<CoefT><<<blocks, 256, 0, st>>>(c, idx, sl, pb);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -443,7 +377,7 @@ cudaError_t launch_sel(const void* coef, uint8_t* idx, void* sel, const Problem&
 // binary16 fast path: needs 4-byte aligned pixel pairs in every plane and in the outputs
 bool pair_path_ok(const void* coef, const uint8_t* idx, const void* sel, const Problem& pb)
 {
-    return pb.s <= 16 && (pb.W & 1) == 0 && (reinterpret_cast<uintptr_t>(coef) & 3) == 0 &&
+    return pb.s <= 16 && ((int64_t)pb.H * pb.W & 1) == 0 && (reinterpret_cast<uintptr_t>(coef) & 3) == 0 &&
            (reinterpret_cast<uintptr_t>(idx) & 1) == 0 && (reinterpret_cast<uintptr_t>(sel) & 3) == 0;
 }
 

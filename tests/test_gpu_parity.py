@@ -128,6 +128,30 @@ def test_select_bit_exact(dt, D, s):
         np.testing.assert_array_equal(host(sr.sr_dict_select(dev(coef), s)), want_idx)
 
 
+@pytest.mark.parametrize("dt", ["f16", "f32"])
+@pytest.mark.parametrize("n,h,w", [(1, 9, 23), (2, 5, 6), (1, 1, 1), (2, 2, 27)])
+@pytest.mark.parametrize("D,s", [(1, 1), (2, 2), (7, 4), (8, 4), (9, 5), (16, 8), (17, 9), (64, 8), (65, 16), (128, 15), (129, 8), (256, 16)])
+def test_select_any_width_with_magnitudes_that_differ_in_few_bits(dt, n, h, w, D, s):
+    rng = np.random.default_rng(D * 31 + s)
+    top = (n, D, h, w)
+    bits = rng.integers(0, 3, top) * 5 + rng.integers(0, 130, top) * (rng.random(top) < 0.5)      # exact ties and neighbours
+    base, kind = (np.float32(0.5).view(np.uint32), np.uint32) if dt == "f32" else (np.float16(0.5).view(np.uint16), np.uint16)
+    coef = (base + bits.astype(kind)).astype(kind).view(np.float32 if dt == "f32" else np.float16)
+    coef = coef * rng.choice([-1, 1], top).astype(coef.dtype) * (rng.random(top) < 0.8)           # signs, and some zeros
+    coef = np.ascontiguousarray(coef.astype(np.float32 if dt == "f32" else np.float16))
+    idx, sel = sr.sr_dict_select(dev(coef), s, want_sel=True)
+    want_idx, want_sel = oracle.dict_select(coef, s, want_sel=True)
+    np.testing.assert_array_equal(host(idx), want_idx)
+    np.testing.assert_array_equal(host(sel).astype(np.float64), want_sel)
+    # the selection made inside the regression: an atom that reads the centre alone, scaled by its index, tells the choice
+    lr, d = np.ones((n, 1, h, w), np.float32), np.zeros((D, 9), np.float32)
+    d[:, 4] = 1.0 + np.arange(D) / 8.0
+    got = host(sr.sr_dict_regress_selected(dev(lr), dev(coef), None, None, dev(d), 1, 3, s))
+    want = (want_sel * d[want_idx, 4]).sum(1)[:, None]
+    # s products of at most 0.53 x 33, summed in fp32
+    assert np.abs(got - want).max() <= 2.0 ** -23 * s * s * 18
+
+
 def test_select_signed_zero_and_extremes():
     coef = np.zeros((1, 8, 2, 8), np.float16)
     coef[0, 3] = -0.0
