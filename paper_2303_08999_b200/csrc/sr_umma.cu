@@ -56,17 +56,33 @@ namespace th8 {
 
 } // namespace
 
-// Tile height per mode: 16 rows wherever the shape still leaves the selective pipeline its eight stages (dense and
-// global-subset modes always; the in-kernel selection when the single U buffer it needs fits), else 8 rows.
+// Tile height. A CTA works off whole tiles, so a frame takes ceil(tiles / SMs) turns, and two turns of 8 rows cost f times
+// one of 16: more copies of the halo, twice the hand-overs. 8 rows wherever f * turns8 < 2 * turns16.
+// f, from the two heights timed on the same frames (8 / 16 rows, us, 544 x 640 (3 turns against 2), 720p (7 against 4), 4K
+// (55 against 28)):
+//   dense, eight 16-row stages or more: 1.2    (D = 32, k = 5: 22.2 / 24.5, 40.9 / 39.4, 269 / 227)
+//   dense, four to seven: 1.1                  (D = 72, k = 5, x4: 21.1 / 24.9, 37.5 / 40.0, 236 / 221; D = 96, x2: 24.9 / 28.8,
+//                                               44.9 / 49.0, 300 / 296)
+//   dense, fewer, where 8 rows double them: 0.85: three or two stages of 16 rows do not cover the copies' latency
+//                                              (D = 128, k = 5: 26.4 / 42.2, 50.1 / 79.8, 390 / 487)
+//   selection in the call, lists: 1.1          (D = 72, k = 5, s = 8: 36.9 / 44.3, 74.7 / 79.6, 1080p (14 against 7) 142.9 / 135.5)
+// The selective pipeline wants eight stages (compact values: four, nothing streams into them): 8 rows where 16 leave fewer.
 static bool tall_tiles(int mode, const void* coef, int coef_dtype, const Problem& pb)
 {
-    // frames whose 16-row tiles leave half the chip idle: a CTA's time is its rows, so halve them (128 x 128, D = 72, k = 5:
-    // dense 16.6 -> 12.2 us of device time, selection in the call 23.5 -> 15.4)
-    const long long tiles16 = (long long)((pb.W + 127) / 128) * ((pb.H + 15) / 16) * pb.n;
-    if (2 * tiles16 <= sm_count() && th8::supported(mode, coef, coef_dtype, pb)) return false;
-    if (!th8::is_selective(mode)) return true;
-    // (compact values: nothing streams into the stages, four are enough)
-    return th16::supported(mode, coef, coef_dtype, pb) && th16::stage_count(mode, pb) >= (mode == kModeCompact ? 4 : 8);
+    if (!th16::supported(mode, coef, coef_dtype, pb)) return false;
+    if (!th8::supported(mode, coef, coef_dtype, pb)) return true;
+    const long long columns = (long long)((pb.W + 127) / 128) * pb.n, sms = sm_count();
+    const long long turns16 = (columns * ((pb.H + 15) / 16) + sms - 1) / sms, turns8 = (columns * ((pb.H + 7) / 8) + sms - 1) / sms;
+    const int stages = th16::stage_count(mode, pb);
+    int percent = 110;                                      // f
+    if (th8::is_selective(mode)) {
+        if (stages < (mode == kModeCompact ? 4 : 8)) return false;
+    } else if (stages >= 8) {
+        percent = 120;
+    } else if (stages < 4) {
+        percent = th8::stage_count(mode, pb) >= 2 * stages ? 85 : 105;
+    }
+    return turns8 * percent >= 200 * turns16;
 }
 
 bool umma_supported(int mode, const void* coef, int coef_dtype, const Problem& pb)

@@ -241,6 +241,24 @@ def test_selected_with_ties(D, s, w):
     assert max_abs_err(got, want) <= TOL_F16
 
 
+# Frames whose tile counts lie on both sides of the tile-height and layout rules: 8-row tiles in one, two and three turns of
+# the SMs, 16-row tiles, the row kernel and the general kernel for few atoms and short lists.
+@pytest.mark.parametrize("n,h,w,r,D,k,s", [(1, 272, 320, 2, 20, 3, 4), (1, 150, 200, 2, 40, 5, 8), (2, 64, 64, 2, 16, 5, 16), (1, 31, 48, 4, 16, 3, 3),
+                                           (3, 37, 56, 2, 32, 7, 4), (1, 65, 112, 3, 128, 3, 8), (1, 117, 160, 3, 16, 5, 5)])
+def test_layout_rules_of_small_and_middling_frames(n, h, w, r, D, k, s):
+    wl = _wl(n, 1, h, w, r, D, k, "f16")
+    lr, d, coef = sr_inputs.make_inputs(wl)
+    d = signed_asymmetric_dictionary(d, seed=k)
+    want = oracle.dict_regress_dense(lr, coef, d, r, k)
+    assert max_abs_err(host(sr.sr_dict_regress_dense(dev(lr), dev(coef), dev(d), r, k)), want) <= TOL_F16
+    want = oracle.dict_regress_selected(lr, coef, None, None, d, r, k, s)
+    assert max_abs_err(host(sr.sr_dict_regress_selected(dev(lr), dev(coef), None, None, dev(d), r, k, s)), want) <= TOL_F16
+    idx, sel = sr.sr_dict_select(dev(coef), s, want_sel=True)
+    got = host(sr.sr_dict_regress_selected(dev(lr), sel, idx, None, dev(d), r, k, s, sr.SR_COEF_COMPACT))
+    assert max_abs_err(got, want) <= TOL_F16
+    assert sr.sr_device_status() == 0
+
+
 # ------------------------------------------------------------------ orientation and sign of the taps
 
 SIGNED_CASES = [
