@@ -219,7 +219,7 @@ typedef struct sr_search_opts {
  * (trace and steps_out may be NULL).  The printed listing's bisection is read as a bisection inside the last doubling
  * step with the feasible solution that keeps the most atoms taken when no lambda lands in the band.
  * `scratch`: device memory of at least sr_selection_search_scratch_bytes(D) bytes, 8-byte aligned.  fp64 throughout;
- * one warp, every sum in a fixed order: the same inputs give the same bits on every run.
+ * one block, every sum in a fixed order: the same inputs give the same bits on every run.
  */
 size_t sr_selection_search_scratch_bytes(int32_t D);
 int sr_selection_search(const double* G, const double* b, const double* hh, double nrows, int32_t D,
