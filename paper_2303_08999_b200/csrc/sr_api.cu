@@ -126,13 +126,14 @@ static long long hr_pixels(const Problem& pb) { return (long long)pb.n * pb.H * 
 // Whether the frame is small enough for the row kernel (sr_regress_rows.cu) although the tensor-core layouts could take it:
 // it cuts a frame into 64 x 4 pieces where they need a 128 x 8 tile per CTA, but it works its atoms off four times slower,
 // so the limit falls with the number of atoms and taps. Device time, row kernel / better layout: 128 x 128, D = 16: k = 3
-// 6.5 / 9.3 us, k = 5 7.9 / 10.8, k = 7 9.2 / 11.8; D = 32: 7.7 / 9.6, 9.8 / 11.2, 11.2 / 12.4; D = 72, k = 5: 13.8 / 12.2.
+// 6.5 / 9.3 us, k = 5 7.9 / 10.8, k = 7 9.2 / 11.8; D = 32: 7.7 / 9.6, 9.8 / 11.2, k = 7 11.8 / 11.1 (D = 24: 9.9 / 11.1);
+// D = 72, k = 5: 13.8 / 12.2. Below 32768 pixels the general kernel does the same work (launch_regress_fma).
 // The lines lie where the two meet (D = 16: k = 3 at 720p, k = 5 at 450 x 450, k = 7 at 300 x 300).
 static bool small_for_rows(const Problem& pb, int natoms)
 {
     const long long px = hr_pixels(pb);
     if (natoms <= 16) return px <= (pb.k == 3 ? 700000 : (pb.k == 5 ? 200000 : 80000));
-    if (natoms <= 32) return px <= (pb.k == 3 ? 100000 : (pb.k == 5 ? 80000 : 40000));
+    if (natoms <= 32) return px <= (pb.k == 3 ? 100000 : (pb.k == 5 ? 80000 : (natoms <= 24 ? 40000 : 0)));
     return false;
 }
 
