@@ -153,18 +153,23 @@ static bool dense_prefers_second_layout(const Problem& pb)
 // Which kernel takes a launch from index + value planes when both could. The gather kernel (sr_regress_listed.cu) pays
 // s * floor(k^2 / 4) 16-byte shared-memory gathers per pixel and nothing per atom of the dictionary; the first
 // tensor-core layout pays for clearing and filling a stage row of D coefficients per pixel and little per listed atom.
-// Measured on the 1080p sweep points and the 4K x2 batch (D = 16 / 32 / 72 / 128; k = 3 / 5 / 7; s = 4 / 8 / 16), both
-// kernels forced in turn: the gather kernel is 1.0 - 3.7 times faster wherever this returns true, and up to two times
-// slower at the far end (k = 7, s = 16, few atoms). On frames that leave the first layout at most one 128 x 8 tile per SM
-// its time is flat and lower from about 52 gathers on (384 x 256, D = 72, k = 5: s = 8 15.3 / 17.4 us, s = 16 16.3 / 24.2).
+// Both kernels forced in turn at 544 x 640, 720p, 1080p and 4K (gather kernel / first layout, us, 1080p unless said):
+//   above 80 atoms the first layout has stages for half its select warps: the gather kernel up to 112 gathers (D = 96: k = 5,
+//     s = 16 138 / 189; k = 7, s = 8 173 / 188; k = 7, s = 16, 208 gathers, 269 / 197);
+//   64 to 80 atoms: up to 64 gathers (D = 72, k = 5: s = 8 x4 86.6 / 84.8, 720p 45.7 / 51.8, 4K 350 / 379; s = 16, 112 gathers,
+//     142 / 104; k = 7, s = 8, 104 gathers, 164 / 131);
+//   fewer: up to 52 (k = 3, s = 16: D = 32 81.5 / 80.5, 720p 37.7 / 44.6), and up to 64 below 1.5 million pixels (D = 32, k = 5,
+//     s = 8: 86.7 / 79.4, 720p 45.6 / 49.4).
+// On frames that leave the first layout at most one 128 x 8 tile per SM its time is flat and lower from about 52 gathers on
+// (384 x 256, D = 72, k = 5: s = 8 15.3 / 17.4 us, s = 16 16.3 / 24.2).
 static int compact_gathers(const Problem& pb) { return pb.s * ((pb.k * pb.k + 3) / 4); }   // 16-byte units of dictionary per pixel
 static bool compact_prefers_listed(const Problem& pb)
 {
     const int gathers = compact_gathers(pb);
     if (pb.D <= 96 && gathers >= 52 && 2 * (long long)((pb.W + 127) / 128) * ((pb.H + 15) / 16) * pb.n <= sm_count()) return false;
-    if (pb.D > 96 || gathers <= 52) return true;
-    if (pb.D >= 64) return gathers <= 104 || (pb.r == 2 && gathers <= 112);
-    return pb.r == 2 && gathers <= 56;
+    if (pb.D > 80) return gathers <= 112;
+    if (pb.D >= 64) return gathers <= 64;
+    return gathers <= (hr_pixels(pb) < 1500000 ? 64 : 52);
 }
 
 // Whether a small frame's index + value planes go to the general kernel, which replicates no dictionary and clears no

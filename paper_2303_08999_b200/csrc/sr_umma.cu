@@ -66,7 +66,8 @@ namespace th8 {
 //   dense, fewer, where 8 rows double them: 0.85: three or two stages of 16 rows do not cover the copies' latency
 //                                              (D = 128, k = 5: 26.4 / 42.2, 50.1 / 79.8, 390 / 487)
 //   selection in the call, lists: 1.1          (D = 72, k = 5, s = 8: 36.9 / 44.3, 74.7 / 79.6, 1080p (14 against 7) 142.9 / 135.5)
-// The selective pipeline wants eight stages (compact values: four, nothing streams into them): 8 rows where 16 leave fewer.
+// The selective pipeline wants eight stages, two for each pair of select warps: 8 rows where 16 leave fewer (compact values:
+// only if 8 rows have them, else four will do; D = 72, k = 7, x2, s = 8, 1080p: 183 us with four, 147 with eight).
 static bool tall_tiles(int mode, const void* coef, int coef_dtype, const Problem& pb)
 {
     if (!th16::supported(mode, coef, coef_dtype, pb)) return false;
@@ -76,7 +77,7 @@ static bool tall_tiles(int mode, const void* coef, int coef_dtype, const Problem
     const int stages = th16::stage_count(mode, pb);
     int percent = 110;                                      // f
     if (th8::is_selective(mode)) {
-        if (stages < (mode == kModeCompact ? 4 : 8)) return false;
+        if (stages < 8 && (mode != kModeCompact || stages < 4 || th8::stage_count(mode, pb) >= 8)) return false;
     } else if (stages >= 8) {
         percent = 120;
     } else if (stages < 4) {
