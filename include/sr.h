@@ -214,7 +214,8 @@ typedef struct sr_search_opts {
  * sr_selection_search: Algorithm 1 on the Gram statistics (device pointers G [D][D], b [D], hh [1] in fp64, as
  * sr_selection_gram writes them; nrows = number of (pixel, channel) rows they were summed over: the 1/N of Eq. 7),
  * D <= 128.  Writes, all on the device: idx_out [D] the kept atoms in ascending order, gamma_out [D] their re-weights
- * (product over all steps), *count_out how many were kept (-1 when a re-fit met a singular matrix), and per step
+ * (product over all steps), *count_out how many were kept (-1 when a re-fit met a singular matrix, or when more
+ * atoms than a step may keep have a G[l][l] that is not positive: no lambda removes those), and per step
  * trace[t][0..5] = alpha_t, lambda used, atoms kept, loss after the beta step, loss after the re-fit, LASSO solves
  * (trace and steps_out may be NULL).  The printed listing's bisection is read as a bisection inside the last doubling
  * step with the feasible solution that keeps the most atoms taken when no lambda lands in the band.

@@ -723,6 +723,8 @@ int sr_ref_selection_search(const double* G_in, const double* b_in, double hh, i
             beta = cand;
             lam_hi = lambda;
             lambda = 2.0 * lambda;
+            /* atoms whose G_ll is not positive never move: no lambda is large enough once it stops growing */
+            if ((double)nnz > target && !(lambda > lam_hi)) return REF_ERR_UNSUPPORTED;
         }
         best = beta; best_nnz = nnz; best_lam = lam_hi; have = true;
         /* bisection inside the last doubling step */

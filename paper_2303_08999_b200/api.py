@@ -305,7 +305,7 @@ def sr_selection_search(G, b, hh, nrows: float, alpha: float, delta_alpha: float
                                    _ptr(trace), _ptr(steps), _ptr(scratch), nbytes, _stream()), "sr_selection_search")
     n = int(count.item())
     if n < 0:
-        raise SrError(SR_ERR_UNSUPPORTED, "sr_selection_search: a re-fit met a singular matrix")
+        raise SrError(SR_ERR_UNSUPPORTED, "sr_selection_search: a re-fit met a singular matrix, or too many atoms have no positive G[l][l]")
     return idx[:n], gamma[:n], trace[: int(steps.item())]
 
 

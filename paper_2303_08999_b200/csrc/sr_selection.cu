@@ -750,7 +750,11 @@ __global__ void __launch_bounds__(kSearchThreads, 1) selection_search_kernel(con
             nnz = count_nonzero(s, s.beta);
             lam_hi = lambda;
             lambda = __dmul_rn(2.0, lambda);
+            // Atoms whose G[l][l] is not positive keep beta = 1 at every lambda. When more of them than the target are
+            // left, no lambda is large enough: the search has failed once doubling no longer makes it larger.
+            if ((double)nnz > target && !(lambda > lam_hi)) { failed = true; break; }
         }
+        if (failed) break;
         copy(s.best, s.beta);
         int best_nnz = nnz;
         double best_lam = lam_hi;

@@ -9,6 +9,7 @@ import oracle
 import paper_2303_08999_b200 as sr
 import sr_inputs
 from gpu_util import TOL_F16, dev, host, signed_asymmetric_dictionary
+from test_oracle_pins_selection import DEAD
 
 pytestmark = pytest.mark.gpu
 
@@ -148,3 +149,11 @@ def test_search_bits_at_block_edges_and_extreme_scales(D, scale):
     np.testing.assert_array_equal(host(idx), want_idx)
     np.testing.assert_array_equal(host(trace), want_trace)
     np.testing.assert_array_equal(host(gamma), want_gamma.astype(np.float32))
+
+
+@pytest.mark.parametrize("diag", DEAD, ids=len)
+@pytest.mark.parametrize("lambda0", [1e-3, 5e-324, np.inf])
+def test_search_ends_when_no_lambda_removes_enough_atoms(diag, lambda0):
+    b = np.where(np.array(diag) > 0, 1.0, 0.0)
+    with pytest.raises(sr.SrError):
+        sr.sr_selection_search(dev(np.diag(diag)), dev(b), dev(np.array([5.0])), 10, 0.25, 0.25, 0.0, lambda0)

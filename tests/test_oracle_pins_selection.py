@@ -196,3 +196,16 @@ def test_selection_argument_errors():
         oracle.selection_search(G, b, 1.0, 10, 0.5, 0.0, 0.0, 1e-3)                # no progress per step
     with pytest.raises(ValueError):
         oracle.lasso_cd(G, b, 0.0, 0.1)                                            # no rows
+
+
+DEAD = [  # diagonals with atoms that no lambda removes: none of them live, more than a step may keep, not a number
+    [0.0] * 8, [0.0] * 6 + [1.0, 2.0], [-1.0] * 7 + [3.0], [np.nan] * 7 + [2.0], [0.0] * 100 + [1.0] * 28]
+
+
+@pytest.mark.parametrize("diag", DEAD, ids=len)
+@pytest.mark.parametrize("lambda0", [1e-3, 5e-324, np.inf])
+def test_search_ends_when_no_lambda_removes_enough_atoms(diag, lambda0):
+    G = np.diag(diag)
+    b = np.where(np.array(diag) > 0, 1.0, 0.0)
+    with pytest.raises(ValueError):
+        oracle.selection_search(G, b, 5.0, 10, 0.25, 0.25, 0.0, lambda0)
