@@ -245,21 +245,36 @@ __global__ void __launch_bounds__(32 * NS * GPC, CTAS) regress_tile_kernel(const
 
 constexpr int kTileSmemMax = 200 * 1024;
 
-template <int K, int NS, int GPC, int CTAS, int DEPTH, bool VEC>
-cudaError_t launch_v(TileParams& prm, const Problem& pb, cudaStream_t st)
+// Warps that share the taps, groups (rows) per block, blocks per SM and ring slots for atoms of side K.
+template <int K> struct Shape;
+template <> struct Shape<1> { static constexpr int NS = 1, GPC = 4, CTAS = 6, DEPTH = 8; };
+template <> struct Shape<3> { static constexpr int NS = 1, GPC = 4, CTAS = 4, DEPTH = 12; };
+template <> struct Shape<5> { static constexpr int NS = 1, GPC = 4, CTAS = 3, DEPTH = 8; };
+template <> struct Shape<7> { static constexpr int NS = 2, GPC = 2, CTAS = 3, DEPTH = 8; };
+template <> struct Shape<9> { static constexpr int NS = 4, GPC = 2, CTAS = 2, DEPTH = 8; };
+
+// Fills the tile geometry and the shared-memory offsets for natoms atoms; returns bytes.
+template <int K> size_t plan_tile(TileParams& prm, const Problem& pb)
 {
-    constexpr int P = (K - 1) / 2, NT = 32 * NS * GPC;
-    plan_geom(prm.g, pb, GPC, prm.lr);
+    using S = Shape<K>;
+    plan_geom(prm.g, pb, S::GPC, prm.lr);
     const Geom& g = prm.g;
     auto up4 = [](int v) { return (v + 3) & ~3; };
     prm.off_u = up4(prm.natoms * dict_pitch<K>() + 2 * prm.natoms);
-    prm.off_v = prm.off_u + up4(pb.c * g.uh * tile_uw(P));
+    prm.off_v = prm.off_u + up4(pb.c * g.uh * tile_uw((K - 1) / 2));
     prm.off_l = prm.off_v + up4(pb.c * g.uh * g.tcols);
     prm.off_red = prm.off_l + up4(pb.c * g.trows * g.tcols + 8);
-    prm.off_ring = prm.off_red + pb.c * PX * GPC * (NS - 1) * 32;
-    const size_t smem = (size_t)prm.off_ring * sizeof(float) + (size_t)NS * GPC * DEPTH * kStageBytes;
+    prm.off_ring = prm.off_red + pb.c * PX * S::GPC * (S::NS - 1) * 32;
+    return (size_t)prm.off_ring * sizeof(float) + (size_t)S::NS * S::GPC * S::DEPTH * kStageBytes;
+}
+
+template <int K, bool VEC>
+cudaError_t launch_v(TileParams& prm, const Problem& pb, cudaStream_t st)
+{
+    using S = Shape<K>;
+    const size_t smem = plan_tile<K>(prm, pb);
     if (smem > (size_t)kTileSmemMax) return cudaErrorNotSupported;
-    auto kern = regress_tile_kernel<K, NS, GPC, CTAS, DEPTH, VEC>;
+    auto kern = regress_tile_kernel<K, S::NS, S::GPC, S::CTAS, S::DEPTH, VEC>;
     static bool configured[64] = {false};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
@@ -270,16 +285,29 @@ cudaError_t launch_v(TileParams& prm, const Problem& pb, cudaStream_t st)
         if (e != cudaSuccess) return e;
         configured[dev] = true;
     }
-    kern<<<(unsigned)g.num_tiles, NT, smem, st>>>(prm);
+    kern<<<(unsigned)prm.g.num_tiles, 32 * S::NS * S::GPC, smem, st>>>(prm);
     count_launches(1);
     return cudaGetLastError();
 }
 
-template <int K, int NS, int GPC, int CTAS, int DEPTH>
+template <int K>
 cudaError_t launch_t(TileParams& prm, const Problem& pb, cudaStream_t st)
 {
-    if ((pb.W & 3) == 0 && (reinterpret_cast<uintptr_t>(prm.coef) & 15) == 0) return launch_v<K, NS, GPC, CTAS, DEPTH, true>(prm, pb, st);
-    return launch_v<K, NS, GPC, CTAS, DEPTH, false>(prm, pb, st);
+    if ((pb.W & 3) == 0 && (reinterpret_cast<uintptr_t>(prm.coef) & 15) == 0) return launch_v<K, true>(prm, pb, st);
+    return launch_v<K, false>(prm, pb, st);
+}
+
+size_t smem_bytes(const Problem& pb, int natoms)
+{
+    TileParams prm{};
+    prm.natoms = natoms;
+    switch (pb.k) {
+    case 1: return plan_tile<1>(prm, pb);
+    case 3: return plan_tile<3>(prm, pb);
+    case 5: return plan_tile<5>(prm, pb);
+    case 7: return plan_tile<7>(prm, pb);
+    default: return plan_tile<9>(prm, pb);
+    }
 }
 
 } // namespace
@@ -289,7 +317,8 @@ bool regress_tile_supported(int mode, int coef_dtype, const Problem& pb)
     if ((mode != kModeDense && mode != kModeGlobal) || coef_dtype != SR_F32 || pb.c > 4 || (pb.flags & SR_LUMA_ONLY)) return false;
     // Tiles of 512 pixels and three blocks per SM only pay once they fill the chip; the thread-per-pixel kernel is faster
     // on less than about one block per SM (64 x 64, x2, 5 x 5: 14.6 us against 18.4).
-    return (int64_t)pb.n * pb.H * pb.W >= (int64_t)sm_count() * 512;
+    if ((int64_t)pb.n * pb.H * pb.W < (int64_t)sm_count() * 512) return false;
+    return smem_bytes(pb, mode == kModeGlobal ? pb.s : pb.D) <= (size_t)kTileSmemMax;      // 9 x 9, c = 4, scale 1: up to 240 atoms
 }
 
 cudaError_t launch_regress_tile(int mode, const float* lr, const void* coef, const uint8_t* idx, const float* gamma, const float* dict,
@@ -307,11 +336,11 @@ cudaError_t launch_regress_tile(int mode, const float* lr, const void* coef, con
     }
     prm.out_vec = (pb.W & 3) == 0 && !(pb.flags & (SR_OUT_F16 | SR_OUT_U8)) && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
     switch (pb.k) {
-    case 1: return launch_t<1, 1, 4, 6, 8>(prm, pb, st);
-    case 3: return launch_t<3, 1, 4, 4, 12>(prm, pb, st);
-    case 5: return launch_t<5, 1, 4, 3, 8>(prm, pb, st);
-    case 7: return launch_t<7, 2, 2, 3, 8>(prm, pb, st);
-    case 9: return launch_t<9, 4, 2, 2, 8>(prm, pb, st);
+    case 1: return launch_t<1>(prm, pb, st);
+    case 3: return launch_t<3>(prm, pb, st);
+    case 5: return launch_t<5>(prm, pb, st);
+    case 7: return launch_t<7>(prm, pb, st);
+    case 9: return launch_t<9>(prm, pb, st);
     default: return cudaErrorNotSupported;
     }
 }

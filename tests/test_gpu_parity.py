@@ -383,6 +383,18 @@ def test_register_tiled_fp32_dense_and_subset(case):
     np.testing.assert_array_equal(host(sr.sr_dict_regress_selected(dev(lr), kept, dev(S), dev(gamma), dev(d), r, k, s, sr.SR_IDX_GLOBAL | sr.SR_COEF_COMPACT)), got)
 
 
+@pytest.mark.parametrize("D", [240, 241, 256])              # 240 atoms are the most that the register-tiled kernel's tables hold
+def test_fp32_9x9_four_channels_with_more_atoms_than_the_register_tiled_kernel_holds(D):
+    wl = sr_inputs.Workload("tile", 1, 4, 148, 512, 1, D=D, k=9, coef_dtype="f32")
+    lr, d, coef = sr_inputs.make_inputs(wl)
+    want = oracle.dict_regress_dense(lr, coef, d, 1, 9)
+    assert max_abs_err(host(sr.sr_dict_regress_dense(dev(lr), dev(coef), dev(d), 1, 9)), want) <= TOL_F32
+    s = D - 1
+    S, gamma = np.arange(1, D).astype(np.uint8), signed_gamma(s)
+    want = oracle.dict_regress_selected(lr, coef, S, gamma, d, 1, 9, s, flags=oracle.IDX_GLOBAL)
+    assert max_abs_err(host(sr.sr_dict_regress_selected(dev(lr), dev(coef), dev(S), dev(gamma), dev(d), 1, 9, s, sr.SR_IDX_GLOBAL)), want) <= TOL_F32
+
+
 ROW_CASES = [  # k, n, c, h, w, scale, D: binary16 rows of any width; K-steps of 16 atoms and tiles of 64 x 8 on both sides of their edges
     (5, 1, 3, 41, 43, 3, 72), (5, 2, 3, 9, 21, 3, 16), (5, 1, 1, 17, 65, 1, 17), (5, 1, 4, 5, 63, 1, 15), (3, 2, 3, 13, 33, 2, 1), (3, 1, 2, 27, 11, 4, 33),
     (7, 1, 3, 19, 29, 3, 32), (7, 2, 1, 33, 67, 1, 40), (5, 1, 3, 3, 1, 5, 128), (5, 3, 3, 1, 1, 1, 256), (7, 1, 3, 30, 31, 2, 100), (5, 1, 3, 90, 101, 5, 24),
