@@ -147,6 +147,8 @@ int sr_dict_select(const void* coef, int coef_dtype, uint8_t* idx, void* sel, co
  *   SR_IDX_GLOBAL:           a_q = idx[q], w_q = gamma[q] * coef[n][a_q][Y][X]  (gamma NULL = 1);
  *                            with SR_COEF_COMPACT, w_q = gamma[q] * coef_or_sel[n][q][Y][X]
  * SR_CLAMP01, SR_UPSAMPLE_BILINEAR and SR_OUT_F16 may be added to any of these.
+ * An lr value that is not finite reaches the pixels whose patches read it (through the sixteen taps of an up-sampled
+ * value) and no others, here and in the dense and producer-fused calls; with SR_IDX_GLOBAL lr must be finite.
  * With idx == NULL the coefficients must be finite (the selection multiplies dropped ones by zero).
  * Kept coefficients are used unchanged (no renormalisation).  The s indices of a pixel must be distinct (as
  * sr_dict_select writes them); repeated indices give an unspecified value for that pixel.  An idx value >= D

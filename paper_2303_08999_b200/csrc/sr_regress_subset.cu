@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(kThreads, 2) regress_subset_kernel(const __gri
                 prefetch_lr_window_of(g, p.lr, wn, sL, tid, kThreads);
             }
         }
-        if (h_lane < h_lanes) horizontal_pass<P>(g, wpad, w, uh, sV, sU, h_cg, h_lane, h_lanes);
+        if (h_lane < h_lanes) horizontal_pass<P, TW, false>(g, wpad, w, uh, sV, sU, h_cg, h_lane, h_lanes);
         __syncthreads();                                     // the U tile is complete
 
         const int px0 = w.x0 + 4 * lane;

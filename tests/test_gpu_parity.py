@@ -355,6 +355,62 @@ def test_dictionary_magnitude_range_of_the_tensor_core_path(scale, bound):
     assert max_abs_err(got, oracle.dict_regress_selected(lr, coef, None, None, dict_, 2, 5, 8)) <= bound
 
 
+# ------------------------------------------------------------------ LR pixels that are not finite
+
+# kernel (sr_test_force_kernel; -1 = host rules), mode, n, c, h, w, scale, D, k, coefficients: the kernels that make their
+# up-sampled tiles separably, each with more tiles than thread blocks where its tiles follow one another in a block
+NON_FINITE_LR = [
+    (1, "dense", 2, 3, 130, 320, 2, 32, 5, "f16"), (1, "dense", 2, 1, 400, 500, 1, 24, 3, "f16"), (1, "dense", 2, 1, 90, 136, 4, 72, 7, "f16"),
+    (1, "fused", 2, 3, 130, 320, 2, 32, 5, "f16"), (1, "compact", 1, 3, 96, 160, 3, 32, 5, "f16"),
+    (2, "dense", 2, 3, 130, 320, 2, 16, 5, "f16"), (4, "compact", 2, 3, 130, 320, 2, 32, 5, "f16"),
+    (-1, "dense", 2, 3, 130, 321, 2, 16, 5, "f16"), (-1, "dense", 2, 1, 300, 451, 1, 16, 3, "f16"), (-1, "dense", 1, 2, 101, 231, 3, 16, 7, "f16"),
+    (-1, "dense", 2, 3, 130, 320, 2, 16, 5, "f32"), (-1, "dense", 2, 1, 300, 451, 1, 8, 3, "f32"), (-1, "dense", 1, 1, 101, 230, 3, 8, 9, "f32"),
+    (-1, "fused", 2, 3, 40, 77, 2, 16, 5, "f16"), (-1, "producer", 2, 3, 100, 300, 2, 16, 5, "f16")]
+
+
+@pytest.mark.parametrize("case", NON_FINITE_LR, ids=lambda c: "-".join(map(str, c)))
+def test_a_non_finite_lr_pixel_reaches_only_the_pixels_that_read_it(case):
+    kernel, mode, n, c, h, w, r, D, k, dt = case
+    wl = sr_inputs.Workload("t", n, c, h, w, r, D=D, k=k, coef_dtype=dt)
+    lr, d, coef = sr_inputs.make_inputs(wl)
+    d, s, p = signed_asymmetric_dictionary(d, seed=k), 8, (k - 1) // 2
+    d[d == 0] = 0.25                                          # every tap reads its pixel
+    dco, ddi = dev(coef), dev(d)
+    if mode == "dense":
+        call = lambda x: sr.sr_dict_regress_dense(x, dco, ddi, r, k)
+    elif mode == "fused":
+        call = lambda x: sr.sr_dict_regress_selected(x, dco, None, None, ddi, r, k, s)
+    elif mode == "compact":
+        idx, sel = sr.sr_dict_select(dco, s, want_sel=True)
+        call = lambda x: sr.sr_dict_regress_selected(x, sel, idx, None, ddi, r, k, s, sr.SR_COEF_COMPACT)
+    else:
+        feat, wconv, bias = (dev(a) for a in sr_inputs.make_producer(wl, cin=32, kc=1))
+        folded = sr.sr_producer_fold(wconv, bias, ddi, r, k)
+        call = lambda x: sr.sr_producer_regress(x, feat, folded, r, k, D, 1)
+    sr.sr_test_force_kernel(kernel)
+    try:
+        clean = host(call(dev(lr)))
+        bad, hit = lr.copy(), np.zeros(clean.shape, bool)
+        H, W = h * r, w * r
+        rng = np.random.default_rng(k)
+        spots = [(0, 0, 0), (h - 1, w - 1, 0), (h // 2, 128 // r, 0), (h // 3, 64 // r - 1, n - 1), (h // 3, w - 1, n - 1)]
+        spots += [(int(rng.integers(h)), int(rng.integers(w)), int(rng.integers(n))) for _ in range(6)]
+        first = lambda Z: (2 * Z + 1 - r) // (2 * r) - 1      # first of the four taps of an HR coordinate
+        for j, (y, x, f) in enumerate(spots):
+            ch = j % c
+            bad[f, ch, y, x] = [np.nan, np.inf, -np.inf][j % 3]
+            rows = np.array([any(min(max(first(Z) + a, 0), h - 1) == y for a in range(4)) for Z in range(H)])
+            cols = np.array([any(min(max(first(Z) + a, 0), w - 1) == x for a in range(4)) for Z in range(W)])
+            near = lambda m, size: np.array([any(m[min(max(Z + a, 0), size - 1)] for a in range(-p, p + 1)) for Z in range(size)])
+            hit[f, ch] |= np.outer(near(rows, H), near(cols, W))
+        for _ in range(2):                                    # the second call meets blocks that have just worked on such a frame
+            out = host(call(dev(bad)))
+            np.testing.assert_array_equal(~np.isfinite(out), hit)
+            np.testing.assert_array_equal(out[~hit], clean[~hit])
+    finally:
+        sr.sr_test_force_kernel(-1)
+
+
 TILE_CASES = [  # k, c, h, w, scale, D: fp32 frames large enough for the register-tiled kernel, every atom size, both copy widths
     (1, 1, 260, 300, 1, 5), (3, 3, 130, 161, 2, 9), (5, 3, 101, 87, 3, 72), (5, 4, 70, 69, 4, 7), (7, 3, 100, 95, 3, 16), (9, 2, 80, 64, 4, 8),
     (5, 3, 97, 100, 3, 20), (5, 2, 280, 281, 1, 2)]
