@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(kNT, CTAS) regress_rows_kernel(const __grid_co
     uint32_t* ring = smem + p.off_ring + warp * (kRing * kStage);
     const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring);
     const int64_t frame_elems = (int64_t)p.planes * HW;
-    const uintptr_t end = reinterpret_cast<uintptr_t>(p.coef + p.coef_elems);
+    const uintptr_t begin = reinterpret_cast<uintptr_t>(p.coef), end = reinterpret_cast<uintptr_t>(p.coef + p.coef_elems);
 
     for (int l = tid; l < 16 * ksteps; l += kNT) {
         const int q = min(l, natoms - 1);
@@ -135,10 +135,10 @@ __global__ void __launch_bounds__(kNT, CTAS) regress_rows_kernel(const __grid_co
         if (ft < g.num_tiles) {
             const int64_t row = (int64_t)ff * frame_elems + (int64_t)(fy + fr) * W + fx;     // element in plane 0
             // 144 chunks, nine to a plane; a plane's first chunk may begin, its last end, with another row's elements. At
-            // the tensor's end only what exists is read.
+            // the tensor's two ends (its start may lie inside a chunk) only what exists is read.
             const int n = min(16, natoms - 16 * fk);
             const uint32_t dst = ring_s + fslot + 16 * lane;
-            if (!GATHER && row + (int64_t)(natoms - 1) * HW + 72 <= p.coef_elems) {
+            if (!GATHER && row >= 8 && row + (int64_t)(natoms - 1) * HW + 72 <= p.coef_elems) {
                 const uintptr_t base = reinterpret_cast<uintptr_t>(p.coef + row + (int64_t)(16 * fk) * HW);
 #pragma unroll
                 for (int j = 0; j < 5; ++j) {
@@ -154,7 +154,15 @@ __global__ void __launch_bounds__(kNT, CTAS) regress_rows_kernel(const __grid_co
                         const uintptr_t a0 = (base + 2 * off[q]) & ~(uintptr_t)15;
                         const int64_t left = (int64_t)(end - a0) - 16 * ch;
                         const uint32_t bytes = left >= 16 ? 16u : (left > 0 ? (uint32_t)left : 0u);
-                        cp16_part(dst + 512 * j, a0 + (bytes ? 16 * ch : 0), bytes);
+                        if (a0 + 16 * ch < begin) {          // the one chunk the tensor starts in: element by element
+                            for (int u = 0; u < 8; ++u) {
+                                const uintptr_t a = a0 + 2 * u;
+                                const uint16_t v = a >= begin && a < end ? __ldg(reinterpret_cast<const uint16_t*>(a)) : (uint16_t)0;
+                                asm volatile("st.shared.b16 [%0], %1;" ::"r"(dst + 512 * j + 2 * u), "h"(v) : "memory");
+                            }
+                        } else {
+                            cp16_part(dst + 512 * j, a0 + (bytes ? 16 * ch : 0), bytes);
+                        }
                     }
                 }
             }

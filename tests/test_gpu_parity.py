@@ -484,6 +484,23 @@ def test_binary16_rows_of_any_width(case, magnitude):
     np.testing.assert_array_equal(host(sr.sr_dict_regress_selected(dev(lr), kept, dev(S), dev(gamma), dev(d), r, k, s, sr.SR_IDX_GLOBAL | sr.SR_COEF_COMPACT)), got)
 
 
+@pytest.mark.parametrize("k,n,h,w,D", [(5, 1, 256, 201, 40), (7, 3, 130, 91, 24), (3, 1, 400, 257, 128)])
+def test_binary16_rows_that_start_at_any_half_of_a_chunk(k, n, h, w, D):
+    # the tensor's first chunk begins up to fourteen bytes in front of it; those bytes are not the tensor's
+    lr, d, coef = sr_inputs.make_inputs(sr_inputs.Workload("rows", n, 1, h, w, 1, D=D, k=k))
+    S = np.arange(D, dtype=np.uint8)
+    room = torch.zeros(coef.size + 16, dtype=torch.float16, device="cuda")
+    first = None
+    for start in range(8):
+        room.fill_(float("nan"))
+        view = room[start:start + coef.size].view(coef.shape).copy_(dev(coef))
+        got = host(sr.sr_dict_regress_dense(dev(lr), view, dev(d), 1, k))
+        first = got if first is None else first
+        np.testing.assert_array_equal(got, first)
+        np.testing.assert_array_equal(host(sr.sr_dict_regress_selected(dev(lr), view, dev(S), None, dev(d), 1, k, D, sr.SR_IDX_GLOBAL)), first)
+    assert max_abs_err(first, oracle.dict_regress_dense(lr, coef, d, 1, k)) <= TOL_F32
+
+
 def test_binary16_rows_keep_a_non_finite_coefficient_to_its_pixel():
     wl = sr_inputs.Workload("rows", 1, 3, 20, 27, 3, D=20, k=5)
     lr, d, coef = sr_inputs.make_inputs(wl)
