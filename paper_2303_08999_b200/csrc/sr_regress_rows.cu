@@ -391,6 +391,9 @@ __global__ void __launch_bounds__(kNT, CTAS) regress_rows_kernel(const __grid_co
 }
 
 constexpr int kRowsSmemMax = 224 * 1024;
+constexpr size_t kSmPool = 228 * 1024;                   // shared memory of an SM
+// what a block takes of it: its dynamic part, the kernel's own arrays (400 bytes) and the system's kilobyte, in units of 128
+constexpr size_t block_smem(size_t dynamic) { return (dynamic + 400 + 1024 + 127) / 128 * 128; }
 
 // Fills the shared-memory plan for tiles of th rows; returns bytes.
 template <int K> size_t plan_rows(RowParams& prm, const Problem& pb, int th)
@@ -413,11 +416,11 @@ template <int K, int CTAS, bool GATHER>
 cudaError_t launch_g(RowParams& prm, const Problem& pb, cudaStream_t st)
 {
     // rows per warp and tile: three where the taller tile leaves room for CTAS blocks and work for all of them (213 x 321
-    // x3: 62 us against 65 with two, 71 with one), else two, else one (123 x 129: 15.0 against 19.1)
+    // x3: 63.2 us against 63.8 with two, 71 with one), else two, else one (123 x 129: 15.0 against 19.1)
     size_t smem = 0;
     for (int rows : {3, 2, 1}) {
         smem = plan_rows<K>(prm, pb, rows * kWarps);
-        if (rows == 1 || (prm.g.num_tiles >= sm_count() * CTAS && (rows == 2 || CTAS * (smem + 2048) <= (size_t)227 * 1024))) break;
+        if (rows == 1 || (prm.g.num_tiles >= sm_count() * CTAS && (rows == 2 || CTAS * block_smem(smem) <= kSmPool))) break;
     }
     if (smem > (size_t)kRowsSmemMax) return cudaErrorNotSupported;
     auto kern = regress_rows_kernel<K, CTAS, GATHER>;
