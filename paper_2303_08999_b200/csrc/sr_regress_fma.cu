@@ -1,6 +1,6 @@
 // General regression kernel on the fp32 FMA pipe: every shape, fp32 or binary16 coefficients, all modes.
-// It is the path for small frames and the fallback for shapes and alignments the others do not take; dense fp32 frames
-// large enough go to the register-tiled kernel, dense binary16 frames of any width to the row kernel (launch_regress_fma).
+// It is the path for small and narrow frames and the fallback for shapes and alignments the others do not take; dense and
+// global-subset frames large enough go to the register-tiled kernel (fp32) or the row kernel (binary16; launch_regress_fma).
 //
 // One thread per HR pixel, 32 x 8 pixel tiles. Per pixel: assemble the filter F = Phi_i D in registers
 // (dictionary rows broadcast from shared memory), then y_c = F . B_c against an up-sampled tile with a
@@ -224,10 +224,7 @@ cudaError_t launch_regress_fma(int mode, const float* lr, const void* coef, int 
                                const float* gamma, const float* dict, float* out, const Problem& pb, cudaStream_t st)
 {
     if (regress_tile_supported(mode, coef_dtype, pb)) return launch_regress_tile(mode, lr, coef, idx, gamma, dict, out, pb, st);
-    // A few thousand pixels do not repay the row kernel's ring and dictionary fragments: the general kernel takes them
-    // (rows / general, us: 9207 px D = 72 k = 3 10.8 / 8.1, k = 5 13.6 / 11.8, D = 128 k = 7 26.5 / 23.8; 21412 px 11.0 /
-    // 8.2, 14.0 / 12.0, 27.4 / 24.2; 54720 px 12.3 / 11.3, 16.5 / 18.0, 31.2 / 41.9).
-    if ((int64_t)pb.n * pb.H * pb.W >= 32768 && regress_rows_supported(mode, coef_dtype, pb)) return launch_regress_rows(mode, lr, coef, idx, gamma, dict, out, pb, st);
+    if (regress_rows_supported(mode, coef_dtype, pb) && regress_rows_pay(mode, pb)) return launch_regress_rows(mode, lr, coef, idx, gamma, dict, out, pb, st);
     if (coef_dtype == SR_F16) return launch_k<__half>(mode, lr, coef, idx, gamma, dict, out, pb, st);
     return launch_k<float>(mode, lr, coef, idx, gamma, dict, out, pb, st);
 }

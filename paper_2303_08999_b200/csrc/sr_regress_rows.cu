@@ -412,16 +412,53 @@ template <int K> size_t plan_rows(RowParams& prm, const Problem& pb, int th)
     return (size_t)(prm.off_ring + kWarps * kRing * kStage) * 4;
 }
 
+// Blocks per SM the kernel is compiled for.
+template <int K> constexpr int blocks_per_sm() { return K == 3 ? 4 : (K == 5 ? 3 : 2); }
+
+// Tile height, geometry and shared memory of a launch; returns bytes (above kRowsSmemMax: the kernel cannot run).
+// Rows per warp and tile: three where the taller tile leaves room for all blocks and work for them (213 x 321 x3: 63.2 us
+// against 63.8 with two, 71 with one), else two, else one (123 x 129: 15.0 against 19.1).
+template <int K> size_t choose_rows(RowParams& prm, const Problem& pb)
+{
+    constexpr int CTAS = blocks_per_sm<K>();
+    for (int rows : {3, 2, 1}) {
+        const size_t smem = plan_rows<K>(prm, pb, rows * kWarps);
+        if (rows == 1 || (prm.g.num_tiles >= sm_count() * CTAS && (rows == 2 || CTAS * block_smem(smem) <= kSmPool))) return smem;
+    }
+    return 0;
+}
+
+// Estimated times of this kernel and of the thread-per-pixel kernel, us, fitted to both on 1700 frames of 33 000 to a million
+// pixels, 1 to 1203 pixels wide, 1 to 256 atoms (standard deviation 9 to 14 %).
+// A block of this kernel works in turns of one tile: x rows per warp in all. A row costs by K-step and by channel, and more
+// of both where other blocks share the SM; 64 columns wide whatever the frame's width. Before that the dictionary is laid
+// out, by K-step.
+// The other kernel covers the frame with blocks of 32 x 8 and costs by atom and by channel; its dictionary by atom.
+template <int K> struct Cost;
+template <> struct Cost<3> { static constexpr float layout = 0.63f, step = 0.61f, step_shared = 0.06f, channel = 0.02f, channel_shared = 0.36f, other_dict = 0.032f, other_atom = 0.036f, other_channel = 0.60f; };
+template <> struct Cost<5> { static constexpr float layout = 1.24f, step = 0.68f, step_shared = 0.20f, channel = 0.99f, channel_shared = 0.01f, other_dict = 0.056f, other_atom = 0.072f, other_channel = 0.83f; };
+template <> struct Cost<7> { static constexpr float layout = 2.24f, step = 0.97f, step_shared = 0.08f, channel = 0.33f, channel_shared = 0.28f, other_dict = 0.092f, other_atom = 0.139f, other_channel = 1.08f; };
+
+// Whether the kernel is expected to be the faster one by 5 % (on the frames above: 940 of 1800, with a
+// geometric mean of 0.75 of the other kernel's time and 43 that lose more than 6 %, 18 % at most; always: 1.02 and 720, 147 %).
+template <int K> bool rows_pay(RowParams& prm, const Problem& pb)
+{
+    const size_t smem = choose_rows<K>(prm, pb);
+    const int sms = sm_count(), rows = prm.g.th / kWarps, fit = (int)(kSmPool / block_smem(smem));
+    const int blocks = fit < blocks_per_sm<K>() ? fit : blocks_per_sm<K>();
+    const int turns = (prm.g.num_tiles + sms * blocks - 1) / (sms * blocks), tiles_per_sm = (prm.g.num_tiles + sms - 1) / sms;
+    const float x = (float)(turns * rows), shared = (float)(tiles_per_sm < blocks ? tiles_per_sm : blocks);
+    using C = Cost<K>;
+    const float mine = 4.3f + C::layout * prm.ksteps + x * (prm.ksteps * (C::step + C::step_shared * shared) + pb.c * (C::channel + C::channel_shared * shared));
+    const float covered = (float)((double)pb.n * ((pb.W + 31) / 32) * ((pb.H + 7) / 8) / sms);
+    const float other = 4.0f + C::other_dict * prm.natoms + covered * (C::other_atom * prm.natoms + C::other_channel * pb.c);
+    return mine < 0.95f * other;
+}
+
 template <int K, int CTAS, bool GATHER>
 cudaError_t launch_g(RowParams& prm, const Problem& pb, cudaStream_t st)
 {
-    // rows per warp and tile: three where the taller tile leaves room for CTAS blocks and work for all of them (213 x 321
-    // x3: 63.2 us against 63.8 with two, 71 with one), else two, else one (123 x 129: 15.0 against 19.1)
-    size_t smem = 0;
-    for (int rows : {3, 2, 1}) {
-        smem = plan_rows<K>(prm, pb, rows * kWarps);
-        if (rows == 1 || (prm.g.num_tiles >= sm_count() * CTAS && (rows == 2 || CTAS * block_smem(smem) <= kSmPool))) break;
-    }
+    const size_t smem = choose_rows<K>(prm, pb);
     if (smem > (size_t)kRowsSmemMax) return cudaErrorNotSupported;
     auto kern = regress_rows_kernel<K, CTAS, GATHER>;
     static bool configured[64] = {false};
@@ -440,9 +477,10 @@ cudaError_t launch_g(RowParams& prm, const Problem& pb, cudaStream_t st)
     return cudaGetLastError();
 }
 
-template <int K, int CTAS>
+template <int K>
 cudaError_t launch_k(RowParams& prm, const Problem& pb, cudaStream_t st)
 {
+    constexpr int CTAS = blocks_per_sm<K>();
     return prm.gather ? launch_g<K, CTAS, true>(prm, pb, st) : launch_g<K, CTAS, false>(prm, pb, st);
 }
 
@@ -456,6 +494,16 @@ bool regress_rows_supported(int mode, int coef_dtype, const Problem& pb)
     prm.natoms = mode == kModeGlobal ? pb.s : pb.D;
     const size_t smem = pb.k == 3 ? plan_rows<3>(prm, pb, 2 * kWarps) : (pb.k == 5 ? plan_rows<5>(prm, pb, 2 * kWarps) : plan_rows<7>(prm, pb, 2 * kWarps));
     return smem <= (size_t)kRowsSmemMax;
+}
+
+bool regress_rows_pay(int mode, const Problem& pb)
+{
+    // Fewer pixels do not repay the ring and the dictionary's fragments (rows / thread per pixel, us: 9207 px D = 72 k = 3 10.8
+    // / 8.1, k = 5 13.6 / 11.8, D = 128 k = 7 26.5 / 23.8; 21412 px 11.0 / 8.2, 14.0 / 12.0, 27.4 / 24.2).
+    if ((int64_t)pb.n * pb.H * pb.W < 32768) return false;
+    RowParams prm{};
+    prm.natoms = mode == kModeGlobal ? pb.s : pb.D;
+    return pb.k == 3 ? rows_pay<3>(prm, pb) : (pb.k == 5 ? rows_pay<5>(prm, pb) : rows_pay<7>(prm, pb));
 }
 
 cudaError_t launch_regress_rows(int mode, const float* lr, const void* coef, const uint8_t* idx, const float* gamma, const float* dict,
@@ -473,9 +521,9 @@ cudaError_t launch_regress_rows(int mode, const float* lr, const void* coef, con
     }
     prm.coef_elems = (int64_t)pb.n * prm.planes * pb.H * pb.W;
     switch (pb.k) {
-    case 3: return launch_k<3, 4>(prm, pb, st);
-    case 5: return launch_k<5, 3>(prm, pb, st);
-    case 7: return launch_k<7, 2>(prm, pb, st);
+    case 3: return launch_k<3>(prm, pb, st);
+    case 5: return launch_k<5>(prm, pb, st);
+    case 7: return launch_k<7>(prm, pb, st);
     default: return cudaErrorNotSupported;
     }
 }

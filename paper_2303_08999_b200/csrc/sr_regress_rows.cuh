@@ -9,6 +9,9 @@ namespace sr {
 // 7 x 7, up to four channels.
 bool regress_rows_supported(int mode, int coef_dtype, const Problem& pb);
 
+// Whether a call it takes is expected to be faster there than on the thread-per-pixel kernel.
+bool regress_rows_pay(int mode, const Problem& pb);
+
 cudaError_t launch_regress_rows(int mode, const float* lr, const void* coef, const uint8_t* idx, const float* gamma, const float* dict,
                                 float* out, const Problem& pb, cudaStream_t st);
 

@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(32 * NS * GPC, CTAS) regress_tile_kernel(const
     }
 }
 
-constexpr int kTileSmemMax = 200 * 1024;
+constexpr int kTileSmemMax = 227 * 1024 / 2 - 2048;      // two blocks on an SM (regress_tile_supported)
 
 // Warps that share the taps, groups (rows) per block, blocks per SM and ring slots for atoms of side K.
 template <int K> struct Shape;
@@ -318,7 +318,17 @@ bool regress_tile_supported(int mode, int coef_dtype, const Problem& pb)
     // Tiles of 512 pixels and three blocks per SM only pay once they fill the chip; the thread-per-pixel kernel is faster
     // on less than about one block per SM (64 x 64, x2, 5 x 5: 14.6 us against 18.4).
     if ((int64_t)pb.n * pb.H * pb.W < (int64_t)sm_count() * 512) return false;
-    return smem_bytes(pb, mode == kModeGlobal ? pb.s : pb.D) <= (size_t)kTileSmemMax;      // 9 x 9, c = 4, scale 1: up to 240 atoms
+    // A tile works on 128 columns however narrow the frame, the other kernel on 32 x 8 pixels. Both timed on 1470 frames of
+    // 1 to 1280 columns, 1 to 256 atoms. This kernel's time over the other's (geometric mean; up to 5 x 5, 7 x 7, 9 x 9), by the
+    // pixels its tiles cover over those the other covers: as many 0.70, 0.79, 0.84; 1.3 to 1.4 times 0.79, 0.98, 1.10; twice
+    // (64 columns) 1.07, 1.48, 1.54; four times (32 columns) 1.95, 3.0, 3.4.
+    const int rows = pb.k >= 7 ? 2 : 4, percent = pb.k <= 5 ? 140 : (pb.k == 7 ? 115 : 105);
+    const int64_t mine = (int64_t)((pb.W + 127) / 128) * 128 * ((pb.H + rows - 1) / rows * rows);
+    const int64_t other = (int64_t)((pb.W + 31) / 32) * 32 * ((pb.H + 7) / 8 * 8);
+    if (100 * mine > percent * other) return false;
+    // One block alone on an SM is not faster (7 x 7, 256 atoms, four channels: 283 us against 165; 9 x 9: 0.96 on average, 0.75
+    // with two).
+    return smem_bytes(pb, mode == kModeGlobal ? pb.s : pb.D) <= (size_t)kTileSmemMax;
 }
 
 cudaError_t launch_regress_tile(int mode, const float* lr, const void* coef, const uint8_t* idx, const float* gamma, const float* dict,

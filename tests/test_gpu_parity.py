@@ -413,7 +413,7 @@ def test_a_non_finite_lr_pixel_reaches_only_the_pixels_that_read_it(case):
 
 TILE_CASES = [  # k, c, h, w, scale, D: fp32 frames large enough for the register-tiled kernel, every atom size, both copy widths
     (1, 1, 260, 300, 1, 5), (3, 3, 130, 161, 2, 9), (5, 3, 101, 87, 3, 72), (5, 4, 70, 69, 4, 7), (7, 3, 100, 95, 3, 16), (9, 2, 80, 64, 4, 8),
-    (5, 3, 97, 100, 3, 20), (5, 2, 280, 281, 1, 2)]
+    (5, 3, 97, 100, 3, 20), (5, 2, 280, 281, 1, 2), (7, 3, 100, 125, 3, 16)]
 
 
 @pytest.mark.parametrize("case", TILE_CASES, ids=lambda c: "-".join(map(str, c)))
@@ -439,7 +439,7 @@ def test_register_tiled_fp32_dense_and_subset(case):
     np.testing.assert_array_equal(host(sr.sr_dict_regress_selected(dev(lr), kept, dev(S), dev(gamma), dev(d), r, k, s, sr.SR_IDX_GLOBAL | sr.SR_COEF_COMPACT)), got)
 
 
-@pytest.mark.parametrize("D", [240, 241, 256])              # 240 atoms are the most that the register-tiled kernel's tables hold
+@pytest.mark.parametrize("D", [240, 241, 256])
 def test_fp32_9x9_four_channels_with_more_atoms_than_the_register_tiled_kernel_holds(D):
     wl = sr_inputs.Workload("tile", 1, 4, 148, 512, 1, D=D, k=9, coef_dtype="f32")
     lr, d, coef = sr_inputs.make_inputs(wl)
@@ -449,6 +449,24 @@ def test_fp32_9x9_four_channels_with_more_atoms_than_the_register_tiled_kernel_h
     S, gamma = np.arange(1, D).astype(np.uint8), signed_gamma(s)
     want = oracle.dict_regress_selected(lr, coef, S, gamma, d, 1, 9, s, flags=oracle.IDX_GLOBAL)
     assert max_abs_err(host(sr.sr_dict_regress_selected(dev(lr), dev(coef), dev(S), dev(gamma), dev(d), 1, 9, s, sr.SR_IDX_GLOBAL)), want) <= TOL_F32
+
+
+# Batches of patches and frames a few columns wide: their tiles would be mostly empty, so the rules weigh what a tile covers
+NARROW = [(80, 32, 32, 1), (19, 32, 32, 2), (3, 300, 31, 3), (1, 2000, 20, 2), (300, 9, 5, 3)]
+
+
+@pytest.mark.parametrize("dt", ["f16", "f32"])
+@pytest.mark.parametrize("n,h,w,r", NARROW)
+@pytest.mark.parametrize("k,D", [(3, 5), (5, 24), (7, 17)])
+def test_batches_of_narrow_frames(dt, n, h, w, r, k, D):
+    lr, d, coef = sr_inputs.make_inputs(sr_inputs.Workload("narrow", n, 2, h, w, r, D=D, k=k, coef_dtype=dt))
+    d = signed_asymmetric_dictionary(d, seed=k)
+    tol = TOL_F32 if dt == "f32" else TOL_F16
+    assert max_abs_err(host(sr.sr_dict_regress_dense(dev(lr), dev(coef), dev(d), r, k)), oracle.dict_regress_dense(lr, coef, d, r, k)) <= tol
+    s = 3
+    S, gamma = np.arange(D - 1, D - 1 - s, -1).astype(np.uint8), signed_gamma(s)
+    want = oracle.dict_regress_selected(lr, coef, S, gamma, d, r, k, s, flags=oracle.IDX_GLOBAL)
+    assert max_abs_err(host(sr.sr_dict_regress_selected(dev(lr), dev(coef), dev(S), dev(gamma), dev(d), r, k, s, sr.SR_IDX_GLOBAL)), want) <= tol
 
 
 ROW_CASES = [  # k, n, c, h, w, scale, D: binary16 rows of any width; K-steps of 16 atoms and tiles of 64 x 8 on both sides of their edges
