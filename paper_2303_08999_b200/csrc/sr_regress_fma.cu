@@ -14,6 +14,10 @@ namespace sr {
 
 namespace {
 
+// Selection inside the call with lists beyond pick_top's sixteen: a kernel of its own, so that those networks' registers do not
+// cost it blocks (1 x 1 and 3 x 3 atoms: 64 registers instead of 48).
+constexpr int kModeFusedLong = 5;
+
 constexpr int TX = 32, TY = 8, CCHUNK = 4;
 
 template <int K> struct KK { static constexpr int value = K * K, padded = (K * K + 3) & ~3; };
@@ -64,7 +68,9 @@ regress_fma_kernel(const float* __restrict__ lr, const CoefT* __restrict__ coef,
     };
     if (MODE == kModeDense) {
         const CoefT* cp = coef + (int64_t)f * D * HW + pix;
-        constexpr int AHEAD = 12;                            // loads in flight: small frames wait for nothing else
+        // loads in flight: small frames wait for nothing else; 9 x 9 filters leave no registers for twelve (53 binary16 frames
+        // above 20 000 pixels: 2 % slower than with four on average, 14 % at most)
+        constexpr int AHEAD = K == 9 ? 4 : 12;
         int l0 = 0;
         for (; l0 + AHEAD <= D; l0 += AHEAD) {
             float v[AHEAD];
@@ -92,7 +98,7 @@ regress_fma_kernel(const float* __restrict__ lr, const CoefT* __restrict__ coef,
             const int64_t plane = compact ? ((int64_t)f * s + q) : ((int64_t)f * D + a);
             accumulate(a, g * load_coef(coef, plane * HW + pix));
         }
-    } else if (s <= 16) { // kModeFusedSelect: the list in registers, its values fetched again (from L1 or L2 by now); fp32 748 x 660 x3: 2809 -> 868 us
+    } else if (MODE == kModeFusedSelect) { // s <= 16: the list in registers, its values fetched again (from L1 or L2 by now); fp32 748 x 660 x3: 2809 -> 868 us
         const CoefT* cp = coef + (int64_t)f * D * HW + pix;
         uint32_t list[4] = {0, 0, 0, 0};                     // a byte per atom
         auto pick = [&](auto tag) {
@@ -113,7 +119,7 @@ regress_fma_kernel(const float* __restrict__ lr, const CoefT* __restrict__ coef,
             list[3] >>= 8;
             accumulate(a, load_coef(cp, (int64_t)a * HW));
         }
-    } else { // longer lists: repeated scan for the next-largest key; any s, any D
+    } else { // kModeFusedLong: repeated scan for the next-largest key; any s, any D
         const CoefT* cp = coef + (int64_t)f * D * HW + pix;
         long long prev = 0x7FFFFFFFFFFFFFFFll;
         for (int q = 0; q < s; ++q) {
@@ -201,7 +207,8 @@ cudaError_t launch_m(int mode, const float* lr, const void* coef, const uint8_t*
     case kModeIdx: return launch_t<K, CoefT, kModeIdx>(lr, coef, idx, gamma, dict, out, pb, st);
     case kModeCompact: return launch_t<K, CoefT, kModeCompact>(lr, coef, idx, gamma, dict, out, pb, st);
     case kModeGlobal: return launch_t<K, CoefT, kModeGlobal>(lr, coef, idx, gamma, dict, out, pb, st);
-    default: return launch_t<K, CoefT, kModeFusedSelect>(lr, coef, idx, gamma, dict, out, pb, st);
+    default: return pb.s <= 16 ? launch_t<K, CoefT, kModeFusedSelect>(lr, coef, idx, gamma, dict, out, pb, st)
+                               : launch_t<K, CoefT, kModeFusedLong>(lr, coef, idx, gamma, dict, out, pb, st);
     }
 }
 
