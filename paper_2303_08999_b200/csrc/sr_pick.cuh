@@ -5,10 +5,13 @@
 // A binary16 magnitude (15 bits) and an index fit one key. An fp32 magnitude does not: its lowest bits, as many as an index
 // below D needs (7 for D in 65 .. 128), give way to the index. Dropped bits can only matter between atoms whose kept bits
 // are the same, so the merge also keeps the best key that fell out, and a pixel in which two neighbours of the list, or the
-// last of it and the best that fell out, agree in all kept bits (a few pixels in a thousand) is picked again by exact
-// insertion on the full magnitudes.
-// Bound: the integer ALU (about 9 min / max per plane at S = 8) or the reads, 4 D bytes a pixel. Before, an insertion of
-// 64-bit keys, 48 operations per plane at S = 8, or s scans of the D planes where nothing was stored.
+// last of it and the best that fell out, agree in all kept bits is picked again by exact insertion on the full magnitudes.
+// Not where no coefficient of the pixel has any of the dropped bits (fp32 values widened from binary16): equal kept bits are
+// then equal magnitudes, and the index in the key has decided. Of Gaussian coefficients a few pixels in a thousand are
+// picked twice. Against the insertion kernel (sr_dict_select, 16 to 256 atoms; Gaussian, rectified, widened values): s <= 4
+// 0.65, 0.65, 0.61 of its time, longer lists 0.4, 0.5, 0.32.
+// Bound: the integer ALU (about 9 min / max per plane at S = 8) or the reads, 4 D bytes a pixel; an insertion of 64-bit keys
+// took 48 operations per plane at S = 8, s scans of the D planes where nothing was stored more.
 #pragma once
 #include "sr_common.cuh"
 
@@ -24,6 +27,9 @@ __device__ __forceinline__ void cx(int& a, int& b)    // afterwards a >= b
 }
 
 template <int S> __device__ __forceinline__ void sort_desc(int* k);
+
+template <> __device__ __forceinline__ void sort_desc<1>(int*) {}
+template <> __device__ __forceinline__ void sort_desc<2>(int* k) { cx(k[0], k[1]); }
 
 template <> __device__ __forceinline__ void sort_desc<4>(int* k)
 {
@@ -84,7 +90,11 @@ template <> __device__ __forceinline__ int pick_key<__half>(__half v, uint32_t, 
     return (int)__byte_perm(__half_as_ushort(v) & 0x7FFFu, 255u - (uint32_t)l, 0x7104);      // 0, magnitude (2 bytes), index
 }
 
-// Exact insertion: a magnitude enters below those that are not smaller, so equal ones stay in index order.
+__device__ __forceinline__ uint32_t pick_bits(float v) { return __float_as_uint(v); }
+__device__ __forceinline__ uint32_t pick_bits(__half) { return 0u; }
+
+// Exact insertion: a magnitude enters below those that are not smaller, so equal ones stay in index order. Eight planes are
+// loaded together: on a small frame the one warp that comes here would otherwise wait for each of them.
 template <int S, typename CoefT>
 __device__ __forceinline__ void pick_exact(const CoefT* __restrict__ cp, int64_t HW, int D, int (&atom)[S])
 {
@@ -92,13 +102,18 @@ __device__ __forceinline__ void pick_exact(const CoefT* __restrict__ cp, int64_t
 #pragma unroll
     for (int i = 0; i < S; ++i) { m[i] = -1; atom[i] = 0; }
 #pragma unroll 1
-    for (int l = 0; l < D; ++l, cp += HW) {
-        const int x = (int)mag_bits(__ldg(cp));
-        if (x > m[S - 1]) {
+    for (int l0 = 0; l0 < D; l0 += 8) {
+        int x[8];
 #pragma unroll
-            for (int i = S - 1; i >= 0; --i) {
-                const bool here = x > m[i], above = i > 0 && x > m[i > 0 ? i - 1 : 0];
-                if (here) { m[i] = above ? m[i > 0 ? i - 1 : 0] : x; atom[i] = above ? atom[i > 0 ? i - 1 : 0] : l; }
+        for (int u = 0; u < 8; ++u, cp += HW) x[u] = l0 + u < D ? (int)mag_bits(__ldg(cp)) : -1;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            if (x[u] > m[S - 1]) {
+#pragma unroll
+                for (int i = S - 1; i >= 0; --i) {
+                    const bool here = x[u] > m[i], above = i > 0 && x[u] > m[i > 0 ? i - 1 : 0];
+                    if (here) { m[i] = above ? m[i > 0 ? i - 1 : 0] : x[u]; atom[i] = above ? atom[i > 0 ? i - 1 : 0] : l0 + u; }
+                }
             }
         }
     }
@@ -112,6 +127,7 @@ __device__ __forceinline__ void pick_top(const CoefT* __restrict__ cp, int64_t H
     constexpr int G = S < 8 ? 8 : S;                         // planes loaded together, S of them merged at a time
     const uint32_t mask = whole ? 255u : pick_tag_mask(D);
     int top[S], out = -1;                                    // out: the best key that is in no list
+    uint32_t low = 0;                                        // every bit that any coefficient has
 #pragma unroll
     for (int i = 0; i < S; ++i) top[i] = -1;
     const CoefT* q = cp;
@@ -130,7 +146,10 @@ __device__ __forceinline__ void pick_top(const CoefT* __restrict__ cp, int64_t H
         for (int i = 0; i < G; ++i, q += HW) v[i] = __ldg(q);
         int g[G];
 #pragma unroll
-        for (int i = 0; i < G; ++i) g[i] = pick_key<CoefT>(v[i], mask, l0 + i);
+        for (int i = 0; i < G; ++i) {
+            g[i] = pick_key<CoefT>(v[i], mask, l0 + i);
+            if (!whole) low |= pick_bits(v[i]);
+        }
 #pragma unroll
         for (int i = 0; i < G; i += S) merge(g + i);
     }
@@ -139,12 +158,17 @@ __device__ __forceinline__ void pick_top(const CoefT* __restrict__ cp, int64_t H
 #pragma unroll
         for (int i = 0; i < G; ++i, q += HW) {
             g[i] = -1;
-            if (l0 + i < D) g[i] = pick_key<CoefT>(__ldg(q), mask, l0 + i);
+            if (l0 + i < D) {
+                const CoefT v = __ldg(q);
+                g[i] = pick_key<CoefT>(v, mask, l0 + i);
+                if (!whole) low |= pick_bits(v);
+            }
         }
 #pragma unroll
-        for (int i = 0; i < G; i += S) merge(g + i);
+        for (int i = 0; i < G; i += S)
+            if (l0 + i < D) merge(g + i);
     }
-    if (!whole) {
+    if (!whole && (low & mask) != 0) {
         bool tied = false;
 #pragma unroll
         for (int i = 0; i < S; ++i) {

@@ -108,7 +108,9 @@ regress_fma_kernel(const float* __restrict__ lr, const CoefT* __restrict__ coef,
 #pragma unroll
             for (int i = 0; i < S; ++i) list[i / 4] |= (uint32_t)atom[i] << (8 * (i % 4));
         };
-        if (s <= 4) pick(std::integral_constant<int, 4>{});
+        if (s == 1) pick(std::integral_constant<int, 1>{});
+        else if (s == 2) pick(std::integral_constant<int, 2>{});
+        else if (s <= 4) pick(std::integral_constant<int, 4>{});
         else if (s <= 8) pick(std::integral_constant<int, 8>{});
         else pick(std::integral_constant<int, 16>{});
         for (int q = 0; q < s; ++q) {

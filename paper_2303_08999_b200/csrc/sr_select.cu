@@ -366,7 +366,9 @@ cudaError_t launch_sel(const void* coef, uint8_t* idx, void* sel, const Problem&
     const unsigned ordered = (unsigned)(all < 0x7FFFFFFF ? all : 0x7FFFFFFF), blocks = (unsigned)(all < cap ? all : cap);
     const CoefT* c = (const CoefT*)coef;
     CoefT* sl = (CoefT*)sel;
-    if (pb.s <= 4) select_pick_kernel<CoefT, 4><<<ordered, 256, 0, st>>>(c, idx, sl, pb);
+    if (pb.s == 1) select_pick_kernel<CoefT, 1><<<ordered, 256, 0, st>>>(c, idx, sl, pb);
+    else if (pb.s == 2) select_pick_kernel<CoefT, 2><<<ordered, 256, 0, st>>>(c, idx, sl, pb);
+    else if (pb.s <= 4) select_pick_kernel<CoefT, 4><<<ordered, 256, 0, st>>>(c, idx, sl, pb);
     else if (pb.s <= 8) select_pick_kernel<CoefT, 8><<<ordered, 256, 0, st>>>(c, idx, sl, pb);
     else if (pb.s <= 16) select_pick_kernel<CoefT, 16><<<ordered, 256, 0, st>>>(c, idx, sl, pb);
     else select_scan_kernel<CoefT><<<blocks, 256, 0, st>>>(c, idx, sl, pb);

@@ -152,6 +152,29 @@ def test_select_any_width_with_magnitudes_that_differ_in_few_bits(dt, n, h, w, D
     assert np.abs(got - want).max() <= 2.0 ** -23 * s * s * 18
 
 
+@pytest.mark.parametrize("kind", ["widened", "rectified", "one tiny value"])
+@pytest.mark.parametrize("D,s", [(1, 1), (3, 1), (9, 1), (72, 1), (8, 2), (130, 2), (72, 3), (72, 8), (200, 16), (256, 17)])
+def test_fp32_selection_where_magnitudes_repeat(kind, D, s):
+    # repeated magnitudes whose dropped bits are all zero need no second look; one coefficient with such bits brings it back
+    rng = np.random.default_rng(D + s)
+    coef = rng.integers(-3, 4, (2, D, 7, 23)).astype(np.float16).astype(np.float32) * np.float32(0.125)
+    if kind == "rectified":
+        coef = np.maximum(rng.standard_normal(coef.shape), 0).astype(np.float32) * (rng.random(coef.shape) < 0.3)
+    elif kind == "one tiny value":                            # a magnitude below the key's lowest bit, behind equal zeros
+        coef[:, D - 1] = np.where(rng.random((2, 7, 23)) < 0.5, np.float32(1e-44), np.nextafter(np.float32(0.375), np.float32(1)))
+    coef = np.ascontiguousarray(coef.astype(np.float32))
+    idx, sel = sr.sr_dict_select(dev(coef), s, want_sel=True)
+    want_idx, want_sel = oracle.dict_select(coef, s, want_sel=True)
+    np.testing.assert_array_equal(host(idx), want_idx)
+    np.testing.assert_array_equal(host(sel).astype(np.float64), want_sel)
+    lr, d = np.ones((2, 1, 7, 23), np.float32), np.zeros((D, 9), np.float32)
+    d[:, 4] = 1.0 + np.arange(D) / 8.0
+    got = host(sr.sr_dict_regress_selected(dev(lr), dev(coef), None, None, dev(d), 1, 3, s))
+    want = (want_sel * d[want_idx, 4]).sum(1)[:, None]
+    # s products of at most 4 x 33, summed in fp32
+    assert np.abs(got - want).max() <= 2.0 ** -23 * s * s * 132
+
+
 def test_select_signed_zero_and_extremes():
     coef = np.zeros((1, 8, 2, 8), np.float16)
     coef[0, 3] = -0.0
