@@ -53,7 +53,7 @@ __host__ __device__ constexpr int phase_base(int p, int r)
 // window row loaded and filtered for every block).
 template <int R, int BS>
 __global__ void __launch_bounds__(128) bicubic_block_kernel(const float* __restrict__ lr, float* __restrict__ hr,
-                                                            const __grid_constant__ Problem pb, int run)
+                                                            const __grid_constant__ Problem pb, int run, unsigned flat)
 {
     static_assert(BS % R == 0, "a block starts on a multiple of the scale");
     constexpr int B0 = phase_base(0, R), STEP = BS / R;
@@ -61,7 +61,15 @@ __global__ void __launch_bounds__(128) bicubic_block_kernel(const float* __restr
     constexpr int VEC = BS % 4 == 0 ? 4 : (BS % 2 == 0 ? 2 : 1);                 // floats per store
     const int W = pb.W, H = pb.H, w = pb.w, h = pb.h;
     const unsigned bw = (unsigned)(W + BS - 1) / BS, bh = (unsigned)(H + BS - 1) / BS, runs = (bh + run - 1) / run;
-    const unsigned t = blockIdx.x * 128u + threadIdx.x;
+    // a block's threads share a plane, or (flat: threads per plane) thread after thread goes to plane after plane
+    const int64_t planes = (int64_t)pb.n * pb.c;
+    unsigned t = blockIdx.x * 128u + threadIdx.x;
+    int64_t plane = blockIdx.y, next = gridDim.y;
+    if (flat) {
+        plane = t / flat;
+        t -= (unsigned)plane * flat;
+        next = planes;
+    }
     const unsigned ry = t / bw, bx = t - ry * bw;
     if (ry >= runs) return;
     const bool vec = VEC > 1 && (W % VEC) == 0 && ((reinterpret_cast<uintptr_t>(hr) & (4 * VEC - 1)) == 0) && BS * (int)bx + BS <= W;
@@ -69,7 +77,7 @@ __global__ void __launch_bounds__(128) bicubic_block_kernel(const float* __restr
     int cx[NWIN];
 #pragma unroll
     for (int c = 0; c < NWIN; ++c) cx[c] = clampi(col0 + c, 0, w - 1);
-    for (int64_t plane = blockIdx.y; plane < (int64_t)pb.n * pb.c; plane += gridDim.y) {
+    for (; plane < planes; plane += next) {
         const float* src = lr + plane * (int64_t)h * w;
         float T[NWIN][BS];                                   // horizontal pass of the window's rows
         auto filter_row = [&](int j, int y) {                // LR row y (clamped) into window row j
@@ -138,10 +146,14 @@ static cudaError_t launch_block(const float* lr, float* hr, const Problem& pb, c
     // 640 7.0, 1024 7.4, a block per thread 9.1), up to 4 (540 x 960 x4: 1 / 2 / 4 / 8 blocks 30.5 / 23.2 / 20.2 / 22.5 us;
     // 705 x 1261 x3: 42.5 / 29.8 / 25.9 / 28.1; four frames 1080 x 1920 x2: 127 / 98 / 91 / 94)
     int64_t run = bw * bh * planes / ((int64_t)sm_count() * 640);
-    run = run < 1 ? 1 : (run > 4 ? 4 : run);
+    // one where a frame is less than four blocks wide: the lanes of a warp then take blocks one below the other
+    run = run < 1 || bw < 4 ? 1 : (run > 4 ? 4 : run);
     const int64_t threads = bw * ((bh + run - 1) / run);
-    const dim3 grid((unsigned)((threads + 127) / 128), (unsigned)(planes < 65535 ? planes : 65535));
-    bicubic_block_kernel<R, BS><<<grid, 128, 0, st>>>(lr, hr, pb, (int)run);
+    // planes of a few blocks of threads leave too much of the last one idle: their threads follow one another (batches of small
+    // frames and frames up to 16 columns wide: without this and the rule above up to 2.4 times the time of a block per thread)
+    const bool flat = planes > 1 && threads < 1024 && threads * planes < ((int64_t)1 << 31);
+    const dim3 grid((unsigned)(((flat ? threads * planes : threads) + 127) / 128), flat ? 1u : (unsigned)(planes < 65535 ? planes : 65535));
+    bicubic_block_kernel<R, BS><<<grid, 128, 0, st>>>(lr, hr, pb, (int)run, flat ? (unsigned)threads : 0u);
     count_launches(1);
     return cudaGetLastError();
 }

@@ -32,7 +32,8 @@ def test_bicubic(n, c, h, w, r):
     assert max_abs_err(got, want) <= 1e-6
 
 
-@pytest.mark.parametrize("n,c,h,w,r", [(2, 1, 720, 700, 3), (1, 3, 251, 401, 3), (1, 3, 271, 481, 4), (1, 2, 511, 515, 2)])
+@pytest.mark.parametrize("n,c,h,w,r", [(2, 1, 720, 700, 3), (1, 3, 251, 401, 3), (1, 3, 271, 481, 4), (1, 2, 511, 515, 2),
+                                       (300, 3, 9, 7, 3), (70, 2, 32, 32, 2), (40, 1, 2000, 1, 1), (3, 3, 700, 5, 2), (33, 3, 5, 2, 8)])
 def test_bicubic_runs_of_blocks(n, c, h, w, r):          # a thread walks several blocks; the last run is cut short
     test_bicubic(n, c, h, w, r)
 
