@@ -32,8 +32,8 @@ constexpr int kMaxSearchL = 128;
 // dealt over groups of threads. The LR windows of a producer's next chunk travel (cp.async) behind stage 2, its
 // coefficients and targets from the end of stage 2 to the next chunk's stage 2: sampled pixels are scattered, every
 // coefficient is a 32-byte sector of its own, and that latency has to be covered.
-// fp32 only ever sums up to 96 terms: then a thread adds its block to the CTA's fp64 sums, which stay in shared memory
-// until the CTA is done.
+// fp32 only ever sums the terms of 32 pixels, 96 at most: then a thread adds its block to the CTA's fp64 sums, which stay in
+// shared memory until the CTA is done.
 // Bound: the shared-memory pipe (about 60 % busy) and, beside it, the FMA pipe: a T x T block reads 2 T words for T^2
 // multiply-adds, sixteen clocks of either per warp and row at T = 8. 100 000 sampled pixels of a 1080p frame, D = 72,
 // k = 5, c = 3: 660 -> 176 us (before: an fp64 read-modify-write of the whole matrix in global memory per 32 pixels, one
@@ -862,10 +862,20 @@ cudaError_t launch_selection_gram(const float* lr, const void* coef, int coef_dt
     p.nw = (pb.k - 1 + pb.r - 1) / pb.r + 4;
     const int Dz = p.nb * T;
     auto up4 = [](int v) { return (v + 3) & ~3; };
-    // as many pixels per chunk as give at most 96 rows and fit; the divisors of 160 let a producer thread keep its pixel
+    p.groups = kGramRank / p.nblk;
+    if (p.groups > kGramMaxGroups) p.groups = kGramMaxGroups;
+    // No fp32 sum has more terms than 32 pixels give (grey images got 80 of them for a while: up to 20 units in the last place
+    // instead of 8).
+    const int terms = 32 * pb.c < kGramRows ? 32 * pb.c : kGramRows;
+    int64_t most = sm_count();                               // thread blocks
+    if (most > nslots) most = nslots;
+    // as many pixels per chunk as give at most 96 rows, keep to the terms and fit, but not fewer chunks than blocks as long as
+    // a chunk has more than eight pixels (1160 pixels, D = 16: 19.4 us against 27.2 with 80); the divisors of 160 let a producer thread keep its
+    // pixel
     int floats = 0;
     for (int px : {80, 40, 32, 20, 16, 8, 4}) {
-        if (px * pb.c > kGramRows) continue;
+        if (px * pb.c > kGramRows || px * pb.c > terms * p.groups) continue;
+        if (px > 8 && (p.count + px - 1) / px < most) continue;
         p.px = px;
         p.rows = px * pb.c;
         p.off_acc = up4(kk * Dz);
@@ -883,13 +893,10 @@ cudaError_t launch_selection_gram(const float* lr, const void* coef, int coef_dt
     const size_t smem = (size_t)floats * sizeof(float);
     auto magic = [](int d) { return (uint32_t)((0x100000000ull + d - 1) / d); };
     p.px_magic = magic(p.px); p.nw_magic = magic(p.nw); p.nb_magic = magic(p.nb); p.r_magic = magic(pb.r); p.rows_magic = magic(p.rows);
-    p.groups = kGramRank / p.nblk;
-    if (p.groups > kGramMaxGroups) p.groups = kGramMaxGroups;
     const int rows_per_group = (p.rows + p.groups - 1) / p.groups;
-    p.flush_every = kGramRows / rows_per_group > 1 ? kGramRows / rows_per_group : 1;
+    p.flush_every = terms / rows_per_group > 1 ? terms / rows_per_group : 1;
     const int64_t chunks = (p.count + p.px - 1) / p.px;
-    int64_t ctas = sm_count();
-    if (ctas > nslots) ctas = nslots;
+    int64_t ctas = most;
     if (ctas > chunks) ctas = chunks;
     if (ctas < 1) ctas = 1;
     cudaError_t e;

@@ -131,6 +131,20 @@ def test_gram_at_block_edges_and_odd_planes(D, k, r, h, w, dt, n, c, base):
     _gram_close(sr.sr_selection_gram(dev(lr), co, dev(d), dev(target), None, r, k), *oracle.selection_gram(lr, coef, d, target, None, r, k))
 
 
+@pytest.mark.parametrize("D", [16, 33, 72, 128])
+@pytest.mark.parametrize("n,h,w", [(1, 120, 100), (1, 9, 11)])
+def test_gram_adds_at_most_the_terms_of_32_pixels_in_fp32(D, n, h, w):
+    # responses that are all the same number, whose multiples have no room in fp32: m terms added one after the other are off by at
+    # most (m + 1) / 2 units of 2^-24, and with this number 80 terms are off by 20
+    v = np.float16(1.251953125)
+    lr, coef, d = np.ones((n, 1, h, w), np.float32), np.full((n, D, h, w), v, np.float16), np.ones((D, 1), np.float32)
+    target = np.full((n, 1, h, w), np.float32(v))
+    G, b, hh = (host(x) for x in sr.sr_selection_gram(dev(lr), dev(coef), dev(d), dev(target), None, 1, 1))
+    want = n * h * w * float(v) ** 2
+    for got in (G, b, hh):
+        assert np.abs(got - want).max() <= 16.5 * 2.0 ** -24 * want
+
+
 @pytest.mark.parametrize("D", [1, 7, 8, 9, 31, 33, 64, 65, 97, 128])
 @pytest.mark.parametrize("scale", [1.0, 2.0 ** -700, 2.0 ** 640])
 def test_search_bits_at_block_edges_and_extreme_scales(D, scale):
