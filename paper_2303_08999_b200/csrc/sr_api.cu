@@ -123,31 +123,47 @@ static bool bad_out_flags(uint32_t flags, const sr_dims* d)
 
 static long long hr_pixels(const Problem& pb) { return (long long)pb.n * pb.H * pb.W; }
 
-// Whether the frame is small enough for the row kernel (sr_regress_rows.cu) although the tensor-core layouts could take it:
-// it cuts a frame into 64 x 4 pieces where they need a 128 x 8 tile per CTA, but it works its atoms off four times slower,
-// so the limit falls with the number of atoms and taps. Device time, row kernel / better layout: 128 x 128, D = 16: k = 3
-// 6.5 / 9.3 us, k = 5 7.9 / 10.8, k = 7 9.2 / 11.8; D = 32: 7.7 / 9.6, 9.8 / 11.2, k = 7 11.8 / 11.1 (D = 24: 9.9 / 11.1);
-// D = 72, k = 5: 13.8 / 12.2. Below 32768 pixels the general kernel does the same work (launch_regress_fma).
-// The lines lie where the two meet (D = 16: k = 3 at 720p, k = 5 at 450 x 450, k = 7 at 300 x 300).
-static bool small_for_rows(const Problem& pb, int natoms)
-{
-    const long long px = hr_pixels(pb);
-    if (natoms <= 16) return px <= (pb.k == 3 ? 700000 : (pb.k == 5 ? 200000 : 80000));
-    if (natoms <= 32) return px <= (pb.k == 3 ? 100000 : (pb.k == 5 ? 80000 : (natoms <= 24 ? 40000 : 0)));
-    return false;
-}
+// Pixels that tiles of 128 columns cover.
+static long long covered_by_128(const Problem& pb) { return 128ll * ((pb.W + 127) / 128) * pb.H * pb.n; }
 
 // Which tensor-core layout takes a dense launch. The second layout (sr_regress_tc.cu: channel-split epilogue, two CTAs
-// per SM, several rows per pipeline step) has the smaller per-frame cost and the better epilogue for 7 x 7 atoms; the first
-// (sr_umma.cu) streams faster. 7 x 7: the second with up to 32 atoms (4K frame x2, D = 32: 315 against 383 us), and with any
-// number on frames below 600 000 pixels (128 x 128, D = 128: 15.7 / 18.5 us; 512 x 768: 46 / 51; 720p and above the first:
-// 4K, D = 72: 412 against 504). Up to 16 atoms of 5 x 5: the second between 300 000 and 1.5 million pixels (512 x 640:
-// 18.6 / 23.3; 720p: 32.8 / 36.5; 1080p: 60 / 57).
+// per SM, several rows per pipeline step) has the smaller per-frame cost and the better epilogue; the first (sr_umma.cu)
+// streams faster and is the better one at scale 1, whose up-sampled tiles cost most. Both timed on 3400 frames of 33 000
+// to nine million pixels, 16 to 4000 columns. Second / first, geometric means, by channels:
+//   scales 2 to 4, up to two: 3 x 3 (and 1 x 1) atoms, at most 16 of them 0.77 (0.85); 5 x 5, at most 32 0.72
+//   scales 2 to 4, three, at most 16 atoms: 3 x 3 1.10; 5 x 5 at scales 3 and 4 0.78; at scale 2 0.90 up to 1.6 million covered
+//     pixels, beyond them 0.84 where a seventh of the columns is empty, else 1.00 (1080p 60 / 57 us); 1 x 1 0.99 with empty ones
+//   7 x 7 at scales 2 to 4: at most 32 atoms 0.80; more 0.91 on small frames of several channels, else 1.20
+//   scale 1: three channels 1.42 to 1.65; one, 5 x 5, at most 32 atoms 0.85, up to 3 x 3 0.95; two, 5 x 5, at most 16 0.93
 static bool dense_prefers_second_layout(const Problem& pb)
 {
-    const long long px = hr_pixels(pb);
-    if (pb.k == 7) return pb.D <= 32 || px <= 600000;
-    return pb.k == 5 && pb.D <= 16 && px > 300000 && px <= 1500000;
+    const long long covered = covered_by_128(pb);
+    const bool empty_columns = 20 * hr_pixels(pb) < 17 * covered;
+    const int few = pb.k == 5 ? 32 : 16;
+    if (pb.r == 1) return pb.k <= 5 && ((pb.c == 1 && pb.D <= few) || (pb.c == 2 && pb.k == 5 && pb.D <= 16));
+    if (pb.k == 7) return pb.D <= 32 || (pb.c >= 2 && covered <= 250000);
+    if (pb.c <= 2) return pb.D <= few;
+    if (pb.D > 16) return false;
+    if (pb.k == 5) return covered > 200000 && (pb.r >= 3 || empty_columns || covered <= 1600000);
+    return pb.k == 1 && empty_columns;
+}
+
+// Whether a dense or global-subset launch of few atoms goes to the row or the thread-per-pixel kernel (launch_regress_fma
+// chooses) although the layouts could take it: they need a 128 x 8 tile per CTA, which small and narrow frames do not fill.
+// By the estimated times: those of sr_regress_rows.cu against the better layout's, fitted to the same 2300 frames up to 32
+// atoms within 9 to 10 % (per K-step of sixteen atoms, and by covered pixels with what a K-step, a channel and a channel's share
+// of the LR image add; four channels, which only the first layout takes, 1.2 times that).
+static bool small_for_layouts(int mode, const Problem& pb, int natoms)
+{
+    if (natoms > 32 || hr_pixels(pb) > 700000) return false;
+    struct Fit { float launch, step, px, px_step, px_channel, px_lr; };
+    constexpr Fit k3{8.03f, 0.24f, 0.59f, 0.31f, 0.14f, 0.56f}, k5{8.26f, 0.63f, 0.14f, 0.51f, 0.36f, 0.86f}, k7{7.25f, 1.31f, 1.45f, 0.33f, 0.10f, 1.31f};
+    const Fit& f = pb.k == 3 ? k3 : (pb.k == 5 ? k5 : k7);
+    const int steps = (natoms + 15) / 16;
+    const float px = 1e-5f * (float)covered_by_128(pb);
+    float layouts = f.launch + f.step * steps + px * (f.px + f.px_step * steps + pb.c * (f.px_channel + f.px_lr / pb.r));
+    if (pb.c > 3) layouts *= 1.2f;
+    return regress_rows_or_general_us(mode, pb) < 0.95f * layouts;
 }
 
 // Which kernel takes a launch from index + value planes when both could. The gather kernel (sr_regress_listed.cu) pays
@@ -261,7 +277,7 @@ static int default_kernel(const RegressArgs& a, bool shaped = false)
     if (forced >= 0 && kernel_supported(forced, a)) return forced;
     if (kernel_supported(kKernelSubset, a)) return kKernelSubset;
     if (!shaped && a.mode == kModeCompact && a.coef_dtype == SR_F16 && compact_prefers_general(a.pb)) return kKernelGeneral;
-    if (!shaped && small_for_rows(a.pb, a.pb.s) && regress_rows_supported(a.mode, a.coef_dtype, a.pb)) return kKernelGeneral;   // (dense: s = D)
+    if (!shaped && regress_rows_supported(a.mode, a.coef_dtype, a.pb) && small_for_layouts(a.mode, a.pb, a.pb.s)) return kKernelGeneral;   // (dense: s = D)
     const bool first = kernel_supported(kKernelFirstLayout, a), second = kernel_supported(kKernelSecondLayout, a);
     if (kernel_supported(kKernelListed, a) && (!first || compact_prefers_listed(a.pb))) return kKernelListed;
     if (second && (a.mode == kModeGlobal || dense_prefers_second_layout(a.pb) || !first)) return kKernelSecondLayout;

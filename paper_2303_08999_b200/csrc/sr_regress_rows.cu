@@ -15,6 +15,7 @@
 // Precision: the dictionary is scaled by a power of two that puts its largest tap near 2^14 and split into three binary16
 // numbers (33 bits below the largest tap: fp32 taps enter whole), products are exact, sixteen atoms are summed by the tensor
 // core and those sums are added in fp32.
+#include <math.h>
 #include <type_traits>
 
 #include "sr_regress_rows.cuh"
@@ -439,20 +440,36 @@ template <> struct Cost<3> { static constexpr float layout = 0.63f, step = 0.61f
 template <> struct Cost<5> { static constexpr float layout = 1.24f, step = 0.68f, step_shared = 0.20f, channel = 0.99f, channel_shared = 0.01f, other_dict = 0.056f, other_atom = 0.072f, other_channel = 0.83f; };
 template <> struct Cost<7> { static constexpr float layout = 2.24f, step = 0.97f, step_shared = 0.08f, channel = 0.33f, channel_shared = 0.28f, other_dict = 0.092f, other_atom = 0.139f, other_channel = 1.08f; };
 
-// Whether the kernel is expected to be the faster one by 5 % (on the frames above: 940 of 1800, with a
-// geometric mean of 0.75 of the other kernel's time and 43 that lose more than 6 %, 18 % at most; always: 1.02 and 720, 147 %).
-template <int K> bool rows_pay(RowParams& prm, const Problem& pb)
+// The two, us; this kernel's is infinite where it cannot run or has too few pixels to repay the ring and the dictionary's
+// fragments (rows / thread per pixel, us: 9207 px D = 72 k = 3 10.8 / 8.1, k = 5 13.6 / 11.8, D = 128 k = 7 26.5 / 23.8;
+// 21412 px 11.0 / 8.2, 14.0 / 12.0, 27.4 / 24.2).
+struct Estimate { float rows, other; };
+template <int K> Estimate estimate(RowParams& prm, const Problem& pb)
 {
     const size_t smem = choose_rows<K>(prm, pb);
     const int sms = sm_count(), rows = prm.g.th / kWarps, fit = (int)(kSmPool / block_smem(smem));
+    using C = Cost<K>;
+    const float covered = (float)((double)pb.n * ((pb.W + 31) / 32) * ((pb.H + 7) / 8) / sms);
+    Estimate e;
+    e.other = 4.0f + C::other_dict * prm.natoms + covered * (C::other_atom * prm.natoms + C::other_channel * pb.c);
+    e.rows = INFINITY;
+    if (smem > (size_t)kRowsSmemMax || (int64_t)pb.n * pb.H * pb.W < 32768) return e;
     const int blocks = fit < blocks_per_sm<K>() ? fit : blocks_per_sm<K>();
     const int turns = (prm.g.num_tiles + sms * blocks - 1) / (sms * blocks), tiles_per_sm = (prm.g.num_tiles + sms - 1) / sms;
     const float x = (float)(turns * rows), shared = (float)(tiles_per_sm < blocks ? tiles_per_sm : blocks);
-    using C = Cost<K>;
-    const float mine = 4.3f + C::layout * prm.ksteps + x * (prm.ksteps * (C::step + C::step_shared * shared) + pb.c * (C::channel + C::channel_shared * shared));
-    const float covered = (float)((double)pb.n * ((pb.W + 31) / 32) * ((pb.H + 7) / 8) / sms);
-    const float other = 4.0f + C::other_dict * prm.natoms + covered * (C::other_atom * prm.natoms + C::other_channel * pb.c);
-    return mine < 0.95f * other;
+    e.rows = 4.3f + C::layout * prm.ksteps + x * (prm.ksteps * (C::step + C::step_shared * shared) + pb.c * (C::channel + C::channel_shared * shared));
+    return e;
+}
+
+// Chosen where it is expected to be the faster one by 5 %. On the frames above that is 940 of 1800, with a geometric mean of
+// 0.75 of the other kernel's time and 43 that lose more than 6 %, 18 % at most; always: 1.02, 720 and 147 %.
+bool rows_win(const Estimate& e) { return e.rows < 0.95f * e.other; }
+
+Estimate estimate_of(int mode, const Problem& pb)
+{
+    RowParams prm{};
+    prm.natoms = mode == kModeGlobal ? pb.s : pb.D;
+    return pb.k == 3 ? estimate<3>(prm, pb) : (pb.k == 5 ? estimate<5>(prm, pb) : estimate<7>(prm, pb));
 }
 
 template <int K, int CTAS, bool GATHER>
@@ -496,14 +513,12 @@ bool regress_rows_supported(int mode, int coef_dtype, const Problem& pb)
     return smem <= (size_t)kRowsSmemMax;
 }
 
-bool regress_rows_pay(int mode, const Problem& pb)
+bool regress_rows_pay(int mode, const Problem& pb) { return rows_win(estimate_of(mode, pb)); }
+
+float regress_rows_or_general_us(int mode, const Problem& pb)
 {
-    // Fewer pixels do not repay the ring and the dictionary's fragments (rows / thread per pixel, us: 9207 px D = 72 k = 3 10.8
-    // / 8.1, k = 5 13.6 / 11.8, D = 128 k = 7 26.5 / 23.8; 21412 px 11.0 / 8.2, 14.0 / 12.0, 27.4 / 24.2).
-    if ((int64_t)pb.n * pb.H * pb.W < 32768) return false;
-    RowParams prm{};
-    prm.natoms = mode == kModeGlobal ? pb.s : pb.D;
-    return pb.k == 3 ? rows_pay<3>(prm, pb) : (pb.k == 5 ? rows_pay<5>(prm, pb) : rows_pay<7>(prm, pb));
+    const Estimate e = estimate_of(mode, pb);
+    return rows_win(e) ? e.rows : e.other;
 }
 
 cudaError_t launch_regress_rows(int mode, const float* lr, const void* coef, const uint8_t* idx, const float* gamma, const float* dict,

@@ -12,6 +12,9 @@ bool regress_rows_supported(int mode, int coef_dtype, const Problem& pb);
 // Whether a call it takes is expected to be faster there than on the thread-per-pixel kernel.
 bool regress_rows_pay(int mode, const Problem& pb);
 
+// The expected time of the faster of the two, us.
+float regress_rows_or_general_us(int mode, const Problem& pb);
+
 cudaError_t launch_regress_rows(int mode, const float* lr, const void* coef, const uint8_t* idx, const float* gamma, const float* dict,
                                 float* out, const Problem& pb, cudaStream_t st);
 
