@@ -191,11 +191,19 @@ static bool compact_prefers_listed(const Problem& pb)
 // Whether a small frame's index + value planes go to the general kernel, which replicates no dictionary and clears no
 // stage: its time is the work of one block per SM (device time, general / better of the others: 128 x 128, D = 72, k = 5,
 // s = 8: 9.0 / 15.0 us; 256 x 256: 12.8 / 15.1; 384 x 256: 16.7 / 15.3; s = 4 there 14.0 / 14.1; D = 32, k = 3, s = 16 there
-// 12.5 / 14.0).
+// 12.5 / 14.0). Its blocks cover 32 x 8 pixels (2400 x 40, s = 3: 17.0 / 13.4).
 static bool compact_prefers_general(const Problem& pb)
 {
-    const long long px = hr_pixels(pb);
+    const long long px = 256ll * ((pb.W + 31) / 32) * ((pb.H + 7) / 8) * pb.n;
     return px <= 100000 && px * compact_gathers(pb) <= 5200000;
+}
+
+// Whether index planes without values go to the general kernel: it gathers s coefficients a pixel where the first layout
+// streams all D through its stages, of which from about a hundred atoms on there are only four (84 frames of 96 atoms and
+// more within this line: the layout takes 1.03 to 4 times as long, 2.5 on average).
+static bool idx_prefers_general(const Problem& pb)
+{
+    return pb.D >= 96 && hr_pixels(pb) * pb.s * pb.k * pb.k <= 5000000;
 }
 
 // ---- which kernel runs a regression, and in which launch shape ----------------------------------------------------------
@@ -277,6 +285,7 @@ static int default_kernel(const RegressArgs& a, bool shaped = false)
     if (forced >= 0 && kernel_supported(forced, a)) return forced;
     if (kernel_supported(kKernelSubset, a)) return kKernelSubset;
     if (!shaped && a.mode == kModeCompact && a.coef_dtype == SR_F16 && compact_prefers_general(a.pb)) return kKernelGeneral;
+    if (!shaped && a.mode == kModeIdx && idx_prefers_general(a.pb)) return kKernelGeneral;
     if (!shaped && regress_rows_supported(a.mode, a.coef_dtype, a.pb) && small_for_layouts(a.mode, a.pb, a.pb.s)) return kKernelGeneral;   // (dense: s = D)
     const bool first = kernel_supported(kKernelFirstLayout, a), second = kernel_supported(kKernelSecondLayout, a);
     if (kernel_supported(kKernelListed, a) && (!first || compact_prefers_listed(a.pb))) return kKernelListed;
