@@ -155,7 +155,9 @@ static bool dense_prefers_second_layout(const Problem& pb)
 // of the LR image add; four channels, which only the first layout takes, 1.2 times that).
 static bool small_for_layouts(int mode, const Problem& pb, int natoms)
 {
-    if (natoms > 32 || hr_pixels(pb) > 700000) return false;
+    // (beyond 700 000 pixels the layouts' columns are full, or one of the two has the smaller tiles; with four channels there is
+    // only the first: 300 frames 1618 x 16, one atom of 5 x 5: 3077 us against 1348)
+    if (natoms > 32 || (pb.c <= 3 && hr_pixels(pb) > 700000)) return false;
     struct Fit { float launch, step, px, px_step, px_channel, px_lr; };
     constexpr Fit k3{8.03f, 0.24f, 0.59f, 0.31f, 0.14f, 0.56f}, k5{8.26f, 0.63f, 0.14f, 0.51f, 0.36f, 0.86f}, k7{7.25f, 1.31f, 1.45f, 0.33f, 0.10f, 1.31f};
     const Fit& f = pb.k == 3 ? k3 : (pb.k == 5 ? k5 : k7);
