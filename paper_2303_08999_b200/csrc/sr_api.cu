@@ -278,11 +278,9 @@ static bool kernel_supported(int kernel, const RegressArgs& a)
 // The host rules: small global subsets on the FMA-pipe subset kernel; per-pixel lists with their values on the gather
 // kernel; the second tensor-core layout for the other
 // global subsets and for dense launches with few atoms; the first layout for the rest it supports; else the general kernel.
-// `shaped`: only among the kernels whose launch shape can be searched (the general kernel has none). The same while a lost
-// arrival is armed: the general kernel has no wait that could run out.
+// `shaped`: the layouts, subset and gather kernels before the general one, however small the frame.
 static int default_kernel(const RegressArgs& a, bool shaped = false)
 {
-    shaped = shaped || g_lose_arrival.load(std::memory_order_relaxed) > 0;
     const int forced = g_force_kernel.load(std::memory_order_relaxed);
     if (forced >= 0 && kernel_supported(forced, a)) return forced;
     if (kernel_supported(kKernelSubset, a)) return kKernelSubset;
@@ -344,7 +342,7 @@ static cudaError_t run_regress(const RegressArgs& a)
     TuneChoice c;
     if (tune_lookup(tune_key(a.mode, a.coef_dtype, a.pb), c) && kernel_supported(c.kernel, a)) return run_kernel(c, a);
     c = TuneChoice{};
-    c.kernel = default_kernel(a);
+    c.kernel = default_kernel(a, g_lose_arrival.load(std::memory_order_relaxed) > 0);      // (the general kernel has no wait to lose an arrival of)
     return run_kernel(c, a);
 }
 

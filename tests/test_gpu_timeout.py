@@ -39,8 +39,10 @@ def _calls():
         "index_planes": lambda: sr.sr_dict_regress_selected(dlr, dco, idx, None, ddi, 2, 5, 8),
         # pinned to the first tensor-core layout: the host rules give this shape to the gather kernel, which has no waits
         "compact": lambda: _on_kernel(1, lambda: sr.sr_dict_regress_selected(dlr, sel, idx, None, ddi, 2, 5, 8, sr.SR_COEF_COMPACT)),
-        "global_subset": lambda: sr.sr_dict_regress_selected(dlr, dco, S, None, ddi, 2, 5, 12, sr.SR_IDX_GLOBAL),
-        "dense_few_atoms": lambda: sr.sr_dict_regress_dense(dlr, dco[:, :16].contiguous(), ddi[:16].contiguous(), 2, 5),
+        # pinned to the second layout: the host rules give frames as small as this to the general kernel, which has no waits,
+        # so that the calls before and after would not meet the tensor memory and barriers of the one that failed
+        "global_subset": lambda: _on_kernel(2, lambda: sr.sr_dict_regress_selected(dlr, dco, S, None, ddi, 2, 5, 12, sr.SR_IDX_GLOBAL)),
+        "dense_few_atoms": lambda: _on_kernel(2, lambda: sr.sr_dict_regress_dense(dlr, dco[:, :16].contiguous(), ddi[:16].contiguous(), 2, 5)),
     }
 
 
