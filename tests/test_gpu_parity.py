@@ -543,6 +543,31 @@ def test_binary16_rows_that_start_at_any_half_of_a_chunk(k, n, h, w, D):
     assert max_abs_err(first, oracle.dict_regress_dense(lr, coef, d, 1, k)) <= TOL_F32
 
 
+@pytest.mark.parametrize("k,D", [(3, 72), (5, 53), (7, 33)])
+@pytest.mark.parametrize("flags", [0, sr.SR_CLAMP01 | sr.SR_OUT_U8])
+def test_row_kernel_with_coefficients_that_are_not_finite(k, D, flags):
+    # beside the edges of a 64-pixel column and of a row, in the first, the last and an inner atom: the same infinities and NaN
+    # as the sum has, in that pixel alone
+    lr, d, coef = sr_inputs.make_inputs(sr_inputs.Workload("rows", 2, 3, 97, 85, 2, D=D, k=k))
+    d = signed_asymmetric_dictionary(d, seed=k)
+    d[D - 1] = np.abs(d[D - 1]) + 0.01                        # with finite taps of one sign: an infinity, not NaN
+    args = (dev(d), 2, k, flags)
+    clean = host(sr.sr_dict_regress_dense(dev(lr), dev(coef), *args))
+    bad, hit = coef.copy(), np.zeros(clean.shape, bool)
+    for j, (f, y, x) in enumerate([(0, 0, 0), (0, 30, 63), (0, 30, 64), (0, 31, 65), (1, 100, 169), (1, 101, 0), (1, 193, 169), (0, 7, 127), (1, 8, 128), (0, 60, 150), (0, 61, 150)]):
+        bad[f, [D - 1, 0, D // 2][j % 3], y, x] = [np.inf, -np.inf, np.nan, np.inf][j % 4]
+        hit[f, :, y, x] = True
+    out = host(sr.sr_dict_regress_dense(dev(lr), dev(bad), *args))
+    np.testing.assert_array_equal(out[~hit], clean[~hit])
+    want = oracle.dict_regress_dense(lr, bad, d, 2, k, flags=flags & 1)[hit]
+    if flags == 0:
+        np.testing.assert_array_equal(np.isnan(out[hit]), np.isnan(want))
+        np.testing.assert_array_equal(out[hit][~np.isnan(want)], want[~np.isnan(want)].astype(np.float32))
+        assert np.isinf(want).any() and np.isnan(want).any()
+    else:                                                     # NaN is stored as 0, as by the other kernels
+        np.testing.assert_array_equal(out[hit], np.where(np.isnan(want), 0, np.clip(want, 0, 1) * 255))
+
+
 def test_binary16_rows_keep_a_non_finite_coefficient_to_its_pixel():
     wl = sr_inputs.Workload("rows", 1, 3, 20, 27, 3, D=20, k=5)
     lr, d, coef = sr_inputs.make_inputs(wl)
