@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(kNT, CTAS) regress_rows_kernel(const __grid_co
     if (lane == 0) sMax[warp] = m;
     __syncthreads();
     m = fmaxf(fmaxf(sMax[0], sMax[1]), fmaxf(sMax[2], sMax[3]));
-    const int se = m > 0.f ? max(-100, min(100, 14 + 127 - (int)(__float_as_uint(m) >> 23))) : 0;
+    const int se = m > 0.f ? max(-113, min(126, 14 + 127 - (int)(__float_as_uint(m) >> 23))) : 0;      // (both powers are normal numbers)
     const float scale = __uint_as_float((uint32_t)(127 + se) << 23), unscale = __uint_as_float((uint32_t)(127 - se) << 23);
     for (int i = tid; i < ksteps * NT * 32; i += kNT) {
         const int ln = i & 31, n = (i >> 5) % NT, ks = (i >> 5) / NT;

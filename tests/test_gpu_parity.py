@@ -568,6 +568,16 @@ def test_row_kernel_with_coefficients_that_are_not_finite(k, D, flags):
         np.testing.assert_array_equal(out[hit], np.where(np.isnan(want), 0, np.clip(want, 0, 1) * 255))
 
 
+@pytest.mark.parametrize("magnitude", [2.0 ** 120, 2.0 ** -122])
+def test_row_kernel_at_the_ends_of_the_dictionary_range(magnitude):
+    lr, d, coef = sr_inputs.make_inputs(sr_inputs.Workload("rows", 1, 3, 97, 65, 3, D=48, k=5))
+    d = (signed_asymmetric_dictionary(d, seed=5) * np.float32(magnitude)).astype(np.float32)
+    got = host(sr.sr_dict_regress_dense(dev(lr), dev(coef), dev(d), 3, 5)).astype(np.float64) / magnitude
+    want = oracle.dict_regress_dense(lr, coef, d, 3, 5) / magnitude
+    # (2^-122: results below 2^-126 keep 2^-149, here 2^-27)
+    assert np.abs(got - want).max() <= TOL_F32
+
+
 def test_binary16_rows_keep_a_non_finite_coefficient_to_its_pixel():
     wl = sr_inputs.Workload("rows", 1, 3, 20, 27, 3, D=20, k=5)
     lr, d, coef = sr_inputs.make_inputs(wl)
