@@ -72,6 +72,27 @@ def test_dense(case, clamp):
     assert max_abs_err(got, want) <= tol_for(coef)
 
 
+@pytest.mark.parametrize("kernel", [1, 2])                   # first, second tensor-core layout
+@pytest.mark.parametrize("case", [(1, 3, 24, 40, 2, 16, 3), (2, 1, 33, 48, 2, 8, 5), (1, 2, 20, 72, 3, 17, 5), (1, 3, 24, 40, 2, 32, 7), (1, 3, 20, 32, 1, 16, 1),
+                                  (2, 3, 9, 34, 4, 1, 5), (1, 1, 40, 56, 1, 33, 3), (1, 2, 17, 40, 4, 24, 7)], ids=lambda c: "-".join(map(str, c)))
+def test_both_layouts_on_small_frames_of_few_atoms(kernel, case):
+    # the host rules give such frames to the general kernel; what the layouts do with them stays tested
+    n, c, h, w, r, D, k = case
+    lr, d, coef = sr_inputs.make_inputs(_wl(n, c, h, w, r, D, k, "f16"))
+    d = signed_asymmetric_dictionary(d, seed=k) if k > 1 else np.random.default_rng(1).uniform(-1, 1, d.shape).astype(np.float32)
+    s = min(D, 12)
+    S, gamma = np.arange(D - 1, D - 1 - s, -1).astype(np.uint8), signed_gamma(s)
+    sr.sr_test_force_kernel(kernel)
+    try:
+        dense = host(sr.sr_dict_regress_dense(dev(lr), dev(coef), dev(d), r, k))
+        subset = host(sr.sr_dict_regress_selected(dev(lr), dev(coef), dev(S), dev(gamma), dev(d), r, k, s, sr.SR_IDX_GLOBAL))
+    finally:
+        sr.sr_test_force_kernel(-1)
+    assert sr.sr_device_status() == 0
+    assert max_abs_err(dense, oracle.dict_regress_dense(lr, coef, d, r, k)) <= TOL_F16
+    assert max_abs_err(subset, oracle.dict_regress_selected(lr, coef, S, gamma, d, r, k, s, flags=oracle.IDX_GLOBAL)) <= TOL_F16
+
+
 def test_dense_is_deterministic_and_leaves_inputs_alone():
     lr, dict_, coef = sr_inputs.make_inputs(_wl(2, 3, 33, 50, 4, 72, 5, "f16"))
     dlr, dco, ddi = dev(lr), dev(coef), dev(dict_)
@@ -496,7 +517,7 @@ def test_batches_of_narrow_frames(dt, n, h, w, r, k, D):
 ROW_CASES = [  # k, n, c, h, w, scale, D: binary16 rows of any width; K-steps of 16 atoms and tiles of 64 x 8 on both sides of their edges
     (5, 1, 3, 41, 43, 3, 72), (5, 2, 3, 9, 21, 3, 16), (5, 1, 1, 17, 65, 1, 17), (5, 1, 4, 5, 63, 1, 15), (3, 2, 3, 13, 33, 2, 1), (3, 1, 2, 27, 11, 4, 33),
     (7, 1, 3, 19, 29, 3, 32), (7, 2, 1, 33, 67, 1, 40), (5, 1, 3, 3, 1, 5, 128), (5, 3, 3, 1, 1, 1, 256), (7, 1, 3, 30, 31, 2, 100), (5, 1, 3, 90, 101, 5, 24),
-    # from 32768 pixels the row kernel, below it the general one
+    # both sides of the 32768 pixels from which the row kernel is considered (ROW_KERNEL_CASES are the ones that run it)
     (5, 2, 3, 41, 67, 3, 72), (5, 1, 1, 1, 32767, 1, 15), (5, 1, 1, 1, 32769, 1, 17), (3, 1, 4, 257, 129, 1, 33), (7, 1, 3, 63, 131, 2, 40), (7, 1, 2, 91, 91, 2, 128),
     (3, 2, 3, 65, 67, 2, 1), (5, 1, 2, 33000, 1, 1, 16)]
 
@@ -526,7 +547,7 @@ def test_binary16_rows_of_any_width(case, magnitude):
     np.testing.assert_array_equal(host(sr.sr_dict_regress_selected(dev(lr), kept, dev(S), dev(gamma), dev(d), r, k, s, sr.SR_IDX_GLOBAL | sr.SR_COEF_COMPACT)), got)
 
 
-@pytest.mark.parametrize("k,n,h,w,D", [(5, 1, 256, 201, 40), (7, 3, 130, 91, 24), (3, 1, 400, 257, 128)])
+@pytest.mark.parametrize("k,n,h,w,D", [(5, 2, 301, 257, 48), (7, 2, 211, 97, 16), (3, 1, 400, 257, 128)])
 def test_binary16_rows_that_start_at_any_half_of_a_chunk(k, n, h, w, D):
     # the tensor's first chunk begins up to fourteen bytes in front of it; those bytes are not the tensor's
     lr, d, coef = sr_inputs.make_inputs(sr_inputs.Workload("rows", n, 1, h, w, 1, D=D, k=k))
@@ -541,6 +562,33 @@ def test_binary16_rows_that_start_at_any_half_of_a_chunk(k, n, h, w, D):
         np.testing.assert_array_equal(got, first)
         np.testing.assert_array_equal(host(sr.sr_dict_regress_selected(dev(lr), view, dev(S), None, dev(d), 1, k, D, sr.SR_IDX_GLOBAL)), first)
     assert max_abs_err(first, oracle.dict_regress_dense(lr, coef, d, 1, k)) <= TOL_F32
+
+
+# k, n, c, h, w, scale, D: frames that the rules give to the row kernel (by its estimated time; none of those above is large or
+# has atoms enough). K-steps and 64-pixel columns on both sides of their edges, one to four channels, one to three rows a
+# warp; the last four with more tiles than blocks, so that a block works on several (k = 3, 5, 7, two and five K-steps)
+ROW_KERNEL_CASES = [
+    (5, 2, 4, 211, 129, 1, 16), (5, 1, 2, 161, 43, 3, 31), (5, 2, 3, 97, 43, 3, 33), (5, 1, 3, 97, 65, 3, 48), (5, 2, 1, 129, 85, 2, 49),
+    (5, 2, 2, 97, 65, 2, 256), (3, 2, 3, 97, 85, 2, 48), (3, 2, 1, 129, 43, 3, 65), (3, 2, 4, 97, 85, 2, 200), (7, 2, 3, 97, 65, 3, 3),
+    (7, 2, 1, 211, 97, 1, 16), (7, 2, 4, 85, 85, 2, 17), (7, 2, 3, 161, 161, 1, 33), (7, 1, 2, 201, 97, 2, 100),
+    (3, 1, 3, 160, 401, 3, 72), (7, 1, 2, 151, 151, 3, 40), (5, 1, 3, 213, 321, 3, 72), (5, 2, 3, 201, 321, 1, 24)]
+
+
+@pytest.mark.parametrize("case", ROW_KERNEL_CASES, ids=lambda c: "-".join(map(str, c)))
+def test_row_kernel_dense_and_gathered(case):
+    k, n, c, h, w, r, D = case
+    lr, d, coef = sr_inputs.make_inputs(sr_inputs.Workload("rows", n, c, h, w, r, D=D, k=k))
+    d = signed_asymmetric_dictionary(d, seed=k)
+    out = host(sr.sr_dict_regress_dense(dev(lr), dev(coef), dev(d), r, k))
+    assert max_abs_err(out, oracle.dict_regress_dense(lr, coef, d, r, k)) <= TOL_F32
+    # more than three K-steps where there are as many atoms
+    s = min(D, 61) - (D > 20)
+    S, gamma = np.arange(D - 1, D - 1 - s, -1).astype(np.uint8), signed_gamma(s)
+    want = oracle.dict_regress_selected(lr, coef, S, gamma, d, r, k, s, flags=oracle.IDX_GLOBAL)
+    # (signed weights up to 1.5 on up to 60 atoms of up to 1 / D each)
+    assert max_abs_err(host(sr.sr_dict_regress_selected(dev(lr), dev(coef), dev(S), dev(gamma), dev(d), r, k, s, sr.SR_IDX_GLOBAL)), want) <= 2 * TOL_F32
+    kept = dev(np.ascontiguousarray(coef[:, S]))
+    assert max_abs_err(host(sr.sr_dict_regress_selected(dev(lr), kept, dev(S), dev(gamma), dev(d), r, k, s, sr.SR_IDX_GLOBAL | sr.SR_COEF_COMPACT)), want) <= 2 * TOL_F32
 
 
 @pytest.mark.parametrize("k,D", [(3, 72), (5, 53), (7, 33)])
@@ -578,7 +626,7 @@ def test_row_kernel_at_the_ends_of_the_dictionary_range(magnitude):
     assert np.abs(got - want).max() <= TOL_F32
 
 
-def test_binary16_rows_keep_a_non_finite_coefficient_to_its_pixel():
+def test_binary16_rows_keep_a_non_finite_coefficient_to_its_pixel():       # (a small frame: the general kernel)
     wl = sr_inputs.Workload("rows", 1, 3, 20, 27, 3, D=20, k=5)
     lr, d, coef = sr_inputs.make_inputs(wl)
     clean = host(sr.sr_dict_regress_dense(dev(lr), dev(coef), dev(d), 3, 5))
