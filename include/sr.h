@@ -172,7 +172,7 @@ int sr_dict_regress_selected(const float* lr, const void* coef_or_sel, int coef_
  *     G[l][m] = sum z_l z_m,   b[l] = sum z_l target,   *hh = sum target^2      (device fp64: G [D][D], b [D], hh [1])
  * summed over the pixels listed in `samples` (device int64 flat [n][H][W] indices, nsamples of them; the paper samples
  * its LASSO features too) or over every pixel when samples == NULL, all c channels of each.  Indices outside the
- * tensor are skipped.  flags: SR_UPSAMPLE_BILINEAR or 0.  fp32 arithmetic per 32 pixels, fp64 accumulation; the result
+ * tensor are skipped.  flags: SR_UPSAMPLE_BILINEAR or 0.  fp32 sums of at most 32 pixels, fp64 accumulation; the result
  * does not depend on the order in which thread blocks run.
  * `scratch` is device memory of at least sr_selection_gram_scratch_bytes(d) bytes, 8-byte aligned; the call
  * overwrites it, and two calls that share it must not overlap.  Returns SR_ERR_SHAPE when it is too small.
@@ -192,9 +192,9 @@ int sr_selection_gram(const float* lr, const void* coef, int coef_dtype, const f
  * SR_ERR_TOO_LARGE and launches nothing.  The call allocates nothing and frees nothing.  The first call on a device
  * looks up the array's device address (cudaGetSymbolAddress, with that device current) and sets the kernel's
  * shared-memory limit; make that first call before any stream capture begins.  The array is shared by all calls on a
- * device and keeps the previous call's contents; every block clears its part before use, so back-to-back calls on one
+ * device and keeps the previous call's contents; every block overwrites its part, so back-to-back calls on one
  * stream are fine, but two calls that can overlap on the GPU (different streams or host threads) race on it and give
- * wrong sums.  With 32 blocks instead of two per multiprocessor it is slower than sr_selection_gram on large inputs.
+ * wrong sums.  With 32 blocks instead of one per multiprocessor it is slower than sr_selection_gram on large inputs.
  * A convenience of this library; the paper has no counterpart.
  */
 int sr_selection_gram_static(const float* lr, const void* coef, int coef_dtype, const float* dict, const float* target,
@@ -221,7 +221,8 @@ typedef struct sr_search_opts {
  * trace[t][0..5] = alpha_t, lambda used, atoms kept, loss after the beta step, loss after the re-fit, LASSO solves
  * (trace and steps_out may be NULL).  The printed listing's bisection is read as a bisection inside the last doubling
  * step with the feasible solution that keeps the most atoms taken when no lambda lands in the band.
- * `scratch`: device memory of at least sr_selection_search_scratch_bytes(D) bytes, 8-byte aligned.  fp64 throughout;
+ * `scratch`: device memory of at least sr_selection_search_scratch_bytes(D) bytes, 8-byte aligned: asked for and checked as
+ * before, although the factorisation it was for now stays on the chip and nothing is written to it.  fp64 throughout;
  * one block, every sum in a fixed order: the same inputs give the same bits on every run.
  */
 size_t sr_selection_search_scratch_bytes(int32_t D);
@@ -326,7 +327,8 @@ int64_t sr_set_wait_limit(int64_t cycles);
  * Test hook for the failure path, host-side injection: each of the next `launches` launches of the tensor-core
  * regression kernel leaves out one barrier arrival in its first thread block, so that one of its waits runs out
  * (set a small budget with sr_set_wait_limit first).  Nothing faults or spins without bound: the block gives up
- * as described above.  0 disarms.  While armed, calls take a kernel that has such waits where one supports them.  Returns SR_OK, or SR_ERR_SHAPE for a negative count.  The paper has no counterpart.
+ * as described above.  0 disarms.  While armed, calls take a kernel that has such waits where one supports them.
+ * Returns SR_OK, or SR_ERR_SHAPE for a negative count.  The paper has no counterpart.
  */
 int sr_test_lose_arrival(int launches);
 

@@ -838,7 +838,7 @@ __global__ void __launch_bounds__(kSearchThreads, 1) selection_search_kernel(con
 
 } // namespace
 
-int selection_gram_slots() { return 2 * sm_count(); }
+int selection_gram_slots() { return sm_count(); }
 
 size_t selection_gram_slot_bytes(int D)
 {
@@ -923,8 +923,8 @@ cudaError_t launch_selection_gram(const float* lr, const void* coef, int coef_dt
 // selection_gram_kernel live in the array below instead of in memory the caller passes: kStaticGramSlots slots for at
 // most kStaticGramMaxD atoms, 32 x (80 x 80 + 80 + 8) doubles = 1 660 928 bytes that every device which loads the
 // library holds until the process exits. The array is shared by all calls and keeps what the last call left in it:
-// every CTA clears its own slot before it adds to it, and two calls whose kernels could run at the same time (two
-// streams, two host threads) must not both use this entry point, or they would sum into each other's slots.
+// every CTA overwrites what is read of its slot, once, at its end, and two calls whose kernels could run at the same time
+// (two streams, two host threads) must not both use this entry point, or one would read the other's slots.
 constexpr int kStaticGramSlots = 32;
 constexpr int kStaticGramMaxD = 80;
 static __device__ __align__(256) double g_gram_static_slots[kStaticGramSlots * (kStaticGramMaxD * kStaticGramMaxD + kStaticGramMaxD + 8)];

@@ -19,7 +19,8 @@ cudaError_t launch_selection_gram_static(const float* lr, const void* coef, int 
                                          const int64_t* samples, int64_t nsamples, double* G, double* b, double* hh, const Problem& pb,
                                          cudaStream_t st);
 
-// Scratch the search call asks of its caller: room for the matrix of its factorisation (which now stays in shared memory).
+// Scratch the search call asks of its caller: room for the matrix of its factorisation (which stays in shared memory; the size
+// is part of the interface).
 size_t selection_search_scratch_bytes(int L);
 
 cudaError_t launch_selection_search(const double* G, const double* b, const double* hh, double nrows, int L, const sr_search_opts& o,

@@ -40,8 +40,8 @@ namespace {
 
 using namespace ptx;
 
-// The kernel is instantiated for two tile heights: 16 rows (less halo work per pixel) and 8 rows, for selective
-// launches whose U tile would otherwise leave fewer than eight coefficient stages.
+// The kernel is instantiated for two tile heights: 16 rows (less halo work per pixel) and 8 rows, where they take fewer
+// turns of the SMs or leave the pipeline the stages that 16 do not (tall_tiles).
 namespace th16 {
 #define SR_UMMA_TH 16
 #include "sr_umma_impl.inc"
