@@ -252,9 +252,9 @@ int sr_device_status(void* stream, int* out_status);
  * sr_dict_regress_dense / sr_dict_regress_selected with the same shape use it.  They synchronise `stream`, overwrite
  * `out`, and are meant to be called once per shape at start-up; inputs that are not larger than the L2 cache are timed
  * warm.  The per-pixel arithmetic does not depend on the tile shape, so results for one kernel are the same bits for
- * every shape.  *result (may be NULL) receives the choice.  Kernel 0 has no launch shape to search; where the host rules
- * give a small frame to it, it is timed as the untuned choice and stays unless a searched shape is faster.  sr_tune_reset
- * forgets every recorded shape.
+ * every shape.  *result (may be NULL) receives the choice; kernel 0 has no launch shape, so where the host rules give a
+ * small frame to it, the call times it too and records nothing unless a searched shape is faster.  sr_tune_reset forgets
+ * every recorded shape.
  */
 typedef struct sr_tune_result {
     int32_t kernel;        /* 0 general FMA kernel, 1 first tensor-core layout, 2 second tensor-core layout, 3 subset

@@ -384,7 +384,7 @@ static int tune_shape(const RegressArgs& a, int reps, sr_tune_result* res)
     if (cudaEventCreate(&e0) != cudaSuccess) return SR_ERR_CUDA;
     if (cudaEventCreate(&e1) != cudaSuccess) { cudaEventDestroy(e0); return SR_ERR_CUDA; }
     TuneChoice def;
-    def.kernel = default_kernel(a);
+    def.kernel = default_kernel(a, cands[0].kernel != kKernelGeneral);
     const float def_us = time_candidate(def, a, reps, e0, e1);
     int best = -1;
     float best_us = 0.f;
@@ -392,6 +392,10 @@ static int tune_shape(const RegressArgs& a, int reps, sr_tune_result* res)
         const float us = time_candidate(cands[i], a, reps, e0, e1);
         if (us > 0.f && (best < 0 || us < best_us)) { best = (int)i; best_us = us; }
     }
+    // a small frame that the host rules give to the general kernel stays there unless a searched shape beats it
+    TuneChoice small;
+    small.kernel = default_kernel(a);
+    const float small_us = small.kernel == def.kernel ? -1.f : time_candidate(small, a, reps, e0, e1);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (best < 0 || def_us < 0.f) return SR_ERR_CUDA;
@@ -399,7 +403,8 @@ static int tune_shape(const RegressArgs& a, int reps, sr_tune_result* res)
     if (def_us <= best_us) { pick = def; best_us = def_us; }        // the host rules' own choice stays unless something beat it
     {
         std::lock_guard<std::mutex> lock(g_tune_mu);
-        g_tune_table[tune_key(a.mode, a.coef_dtype, a.pb)] = pick;
+        if (small_us > 0.f && small_us <= best_us) g_tune_table.erase(tune_key(a.mode, a.coef_dtype, a.pb));
+        else g_tune_table[tune_key(a.mode, a.coef_dtype, a.pb)] = pick;
     }
     if (res) {
         res->kernel = pick.kernel;
