@@ -252,9 +252,10 @@ int sr_device_status(void* stream, int* out_status);
  * sr_dict_regress_dense / sr_dict_regress_selected with the same shape use it.  They synchronise `stream`, overwrite
  * `out`, and are meant to be called once per shape at start-up; inputs that are not larger than the L2 cache are timed
  * warm.  The per-pixel arithmetic does not depend on the tile shape, so results for one kernel are the same bits for
- * every shape.  *result (may be NULL) receives the choice; kernel 0 has no launch shape, so where the host rules give a
- * small frame to it, the call times it too and records nothing unless a searched shape is faster.  sr_tune_reset forgets
- * every recorded shape.
+ * every shape.  *result (may be NULL) receives the outcome of the search.  Kernel 0 has no launch shape and is not
+ * searched: where the host rules give a small frame to it, it is timed beside the search, and when it is the fastest,
+ * nothing is recorded and later calls keep running it, while *result still describes the search among the other kernels.
+ * sr_tune_reset forgets every recorded shape.
  */
 typedef struct sr_tune_result {
     int32_t kernel;        /* 0 general FMA kernel, 1 first tensor-core layout, 2 second tensor-core layout, 3 subset
@@ -262,8 +263,9 @@ typedef struct sr_tune_result {
     int32_t tile_rows;     /* tile height (kernels 2, 3 and 4; 0 otherwise)                                            */
     int32_t rows_per_step; /* tile rows per pipeline step (kernel 2; 0 otherwise)                                      */
     int32_t candidates;    /* launch shapes that were legal and timed                                                   */
-    float best_us;         /* time per launch of the recorded shape                                                     */
-    float default_us;      /* time per launch of the shape the host rules pick without tuning                           */
+    float best_us;         /* time per launch of the fastest of them (recorded unless kernel 0 is faster, see above)    */
+    float default_us;      /* time per launch of the shape the host rules pick among kernels 1 to 4 (kernel 0 if none
+                              of those takes the call)                                                                */
 } sr_tune_result;
 int sr_tune_dense(const float* lr, const void* coef, int coef_dtype, const float* dict, float* out, const sr_dims* d,
                   uint32_t flags, int reps, void* stream, sr_tune_result* result);

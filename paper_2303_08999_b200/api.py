@@ -363,7 +363,8 @@ def _tune_dict(res: sr_tune_result) -> dict:
 
 
 def sr_tune_dense(lr, coef, dict_, scale: int, k: int, flags: int = 0, reps: int = 5) -> dict:
-    """Tile-shape search for sr_dict_regress_dense on these buffers; later calls with the same shape use the result."""
+    """Tile-shape search for sr_dict_regress_dense on these buffers; later calls with the same shape use the result, unless
+    the general kernel, which has no shape to search, is faster than every searched one (a small frame)."""
     lr, dict_ = _dev(lr, torch.float32, "lr"), _dev(dict_, torch.float32, "dict")
     code = _coef_code(coef)
     n, c, h, w = lr.shape

@@ -392,7 +392,8 @@ static int tune_shape(const RegressArgs& a, int reps, sr_tune_result* res)
         const float us = time_candidate(cands[i], a, reps, e0, e1);
         if (us > 0.f && (best < 0 || us < best_us)) { best = (int)i; best_us = us; }
     }
-    // a small frame that the host rules give to the general kernel stays there unless a searched shape beats it
+    // a small frame that the host rules give to the general kernel stays there unless a searched shape beats it; the result
+    // describes the search all the same
     TuneChoice small;
     small.kernel = default_kernel(a);
     const float small_us = small.kernel == def.kernel ? -1.f : time_candidate(small, a, reps, e0, e1);

@@ -37,6 +37,25 @@ def test_dense_search_keeps_the_result_and_never_loses_to_the_host_rules(D, k, r
     assert sr.sr_device_status() == 0
 
 
+@pytest.mark.parametrize("h,w,c", [(24, 40, 3), (48, 64, 1), (100, 160, 3)])
+def test_calls_after_a_search_on_a_small_frame(h, w, c):
+    # frames that the host rules give to the general kernel: later calls run the reported shape, or the general kernel as before
+    wl = sr_inputs.Workload("t", 1, c, h, w, 2, D=16, k=3, coef_dtype="f16")
+    lr, d, coef = sr_inputs.make_inputs(wl)
+    dlr, dco, ddi = dev(lr), dev(coef), dev(signed_asymmetric_dictionary(d))
+    before = host(sr.sr_dict_regress_dense(dlr, dco, ddi, 2, 3))
+    res = sr.sr_tune_dense(dlr, dco, ddi, 2, 3, reps=5)
+    after = host(sr.sr_dict_regress_dense(dlr, dco, ddi, 2, 3))
+    assert res["candidates"] > 1 and res["best_us"] <= res["default_us"] * 1.0001
+    sr.sr_tune_reset()
+    sr.sr_test_force_kernel({"first tensor-core layout": 1, "second tensor-core layout": 2}[res["kernel"]])
+    try:
+        reported = host(sr.sr_dict_regress_dense(dlr, dco, ddi, 2, 3))
+    finally:
+        sr.sr_test_force_kernel(-1)
+    assert np.array_equal(after, before) or np.array_equal(after, reported)
+
+
 @pytest.mark.parametrize("s", [8, 12])
 def test_global_subset_search(s):
     wl = sr_inputs.Workload("t", 1, 3, 48, 64, 4, D=72, k=5, coef_dtype="f16")
