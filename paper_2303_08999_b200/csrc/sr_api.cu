@@ -132,7 +132,7 @@ static long long covered_by_128(const Problem& pb) { return 128ll * ((pb.W + 127
 // to nine million pixels, 16 to 4000 columns. Second / first, geometric means, by channels:
 //   scales 2 to 4, up to two: 3 x 3 (and 1 x 1) atoms, at most 16 of them 0.77 (0.85); 5 x 5, at most 32 0.72
 //   scales 2 to 4, three, at most 16 atoms: 3 x 3 1.10; 5 x 5 at scales 3 and 4 0.78; at scale 2 0.90 up to 1.6 million covered
-//     pixels, beyond them 0.84 where a seventh of the columns is empty, else 1.00 (1080p 60 / 57 us); 1 x 1 0.99 with empty ones
+//     pixels, beyond them 0.84 where a seventh of the columns is empty, else 1.00 (1080p 60 / 57 us)
 //   7 x 7 at scales 2 to 4: at most 32 atoms 0.80; more 0.91 on small frames of several channels, else 1.20
 //   scale 1: three channels 1.42 to 1.65; one, 5 x 5, at most 32 atoms 0.85, up to 3 x 3 0.95; two, 5 x 5, at most 16 0.93
 static bool dense_prefers_second_layout(const Problem& pb)
@@ -143,16 +143,14 @@ static bool dense_prefers_second_layout(const Problem& pb)
     if (pb.r == 1) return pb.k <= 5 && ((pb.c == 1 && pb.D <= few) || (pb.c == 2 && pb.k == 5 && pb.D <= 16));
     if (pb.k == 7) return pb.D <= 32 || (pb.c >= 2 && covered <= 250000);
     if (pb.c <= 2) return pb.D <= few;
-    if (pb.D > 16) return false;
-    if (pb.k == 5) return covered > 200000 && (pb.r >= 3 || empty_columns || covered <= 1600000);
-    return pb.k == 1 && empty_columns;
+    return pb.k == 5 && pb.D <= 16 && covered > 200000 && (pb.r >= 3 || empty_columns || covered <= 1600000);
 }
 
 // Whether a dense or global-subset launch of few atoms goes to the row or the thread-per-pixel kernel (launch_regress_fma
 // chooses) although the layouts could take it: they need a 128 x 8 tile per CTA, which small and narrow frames do not fill.
 // By the estimated times: those of sr_regress_rows.cu against the better layout's, fitted to the same 2300 frames up to 32
 // atoms within 9 to 10 % (per K-step of sixteen atoms, and by covered pixels with what a K-step, a channel and a channel's share
-// of the LR image add; four channels, which only the first layout takes, 1.2 times that).
+// of the LR image add; four channels, which only the first layout takes, 1.2 to 1.5 times that).
 static bool small_for_layouts(int mode, const Problem& pb, int natoms)
 {
     // (beyond 700 000 pixels the layouts' columns are full, or one of the two has the smaller tiles; with four channels there is
@@ -164,8 +162,8 @@ static bool small_for_layouts(int mode, const Problem& pb, int natoms)
     const int steps = (natoms + 15) / 16;
     const float px = 1e-5f * (float)covered_by_128(pb);
     float layouts = f.launch + f.step * steps + px * (f.px + f.px_step * steps + pb.c * (f.px_channel + f.px_lr / pb.r));
-    if (pb.c > 3) layouts *= 1.2f;
-    return regress_rows_or_general_us(mode, pb) < 0.95f * layouts;
+    if (pb.c > 3) layouts *= pb.k == 3 ? 1.2f : (pb.k == 5 ? 1.3f : 1.5f);
+    return regress_rows_or_general_us(mode, pb) < layouts;
 }
 
 // Which kernel takes a launch from index + value planes when both could. The gather kernel (sr_regress_listed.cu) pays
@@ -286,7 +284,7 @@ static int default_kernel(const RegressArgs& a, bool shaped = false)
     if (kernel_supported(kKernelSubset, a)) return kKernelSubset;
     if (!shaped && a.mode == kModeCompact && a.coef_dtype == SR_F16 && compact_prefers_general(a.pb)) return kKernelGeneral;
     if (!shaped && a.mode == kModeIdx && idx_prefers_general(a.pb)) return kKernelGeneral;
-    if (!shaped && regress_rows_supported(a.mode, a.coef_dtype, a.pb) && small_for_layouts(a.mode, a.pb, a.pb.s)) return kKernelGeneral;   // (dense: s = D)
+    if (!shaped && regress_rows_form(a.mode, a.coef_dtype, a.pb) && small_for_layouts(a.mode, a.pb, a.pb.s)) return kKernelGeneral;   // (dense: s = D)
     const bool first = kernel_supported(kKernelFirstLayout, a), second = kernel_supported(kKernelSecondLayout, a);
     if (kernel_supported(kKernelListed, a) && (!first || compact_prefers_listed(a.pb))) return kKernelListed;
     if (second && (a.mode == kModeGlobal || dense_prefers_second_layout(a.pb) || !first)) return kKernelSecondLayout;

@@ -464,47 +464,37 @@ template <int K> size_t choose_rows(RowParams& prm, const Problem& pb)
     return 0;
 }
 
-// Estimated times of this kernel and of the thread-per-pixel kernel, us, fitted to both on 1700 frames of 33 000 to a million
-// pixels, 1 to 1203 pixels wide, 1 to 256 atoms (standard deviation 9 to 14 %).
-// A block of this kernel works in turns of one tile: x rows per warp in all. A row costs by K-step and by channel, and more
-// of both where other blocks share the SM; 64 columns wide whatever the frame's width. Before that the dictionary is laid
-// out, by K-step.
-// The other kernel covers the frame with blocks of 32 x 8 and costs by atom and by channel; its dictionary by atom.
+// The kernel's expected time, us. A block works in turns of one tile, x rows per warp in all, 64 columns wide whatever the
+// frame's width. Before that the dictionary is laid out, by K-step. A row costs by K-step, by channel, and by channel over the
+// scale (the LR image's part of the up-sampled tile), and more of each where other blocks share the SM. Fitted to 2550 of the
+// frames that regress_general_us is fitted to (standard deviation 10 to 11 %).
 template <int K> struct Cost;
-template <> struct Cost<3> { static constexpr float layout = 0.63f, step = 0.61f, step_shared = 0.06f, channel = 0.02f, channel_shared = 0.36f, other_dict = 0.032f, other_atom = 0.036f, other_channel = 0.60f; };
-template <> struct Cost<5> { static constexpr float layout = 1.24f, step = 0.68f, step_shared = 0.20f, channel = 0.99f, channel_shared = 0.01f, other_dict = 0.056f, other_atom = 0.072f, other_channel = 0.83f; };
-template <> struct Cost<7> { static constexpr float layout = 2.24f, step = 0.97f, step_shared = 0.08f, channel = 0.33f, channel_shared = 0.28f, other_dict = 0.092f, other_atom = 0.139f, other_channel = 1.08f; };
+template <> struct Cost<3> { static constexpr float launch = 4.38f, layout = 0.45f, step = 0.35f, step_shared = 0.22f, channel = 0.39f, channel_shared = 0.f, lr = 0.15f, lr_shared = 0.18f; };
+template <> struct Cost<5> { static constexpr float launch = 4.65f, layout = 0.88f, step = 1.25f, step_shared = 0.01f, channel = 0.05f, channel_shared = 0.14f, lr = 0.58f, lr_shared = 0.f; };
+template <> struct Cost<7> { static constexpr float launch = 4.48f, layout = 2.01f, step = 1.14f, step_shared = 0.f, channel = 0.07f, channel_shared = 0.24f, lr = 0.05f, lr_shared = 0.14f; };
 
-// The two, us; this kernel's is infinite where it cannot run or has too few pixels to repay the ring and the dictionary's
-// fragments (rows / thread per pixel, us: 9207 px D = 72 k = 3 10.8 / 8.1, k = 5 13.6 / 11.8, D = 128 k = 7 26.5 / 23.8;
-// 21412 px 11.0 / 8.2, 14.0 / 12.0, 27.4 / 24.2).
-struct Estimate { float rows, other; };
-template <int K> Estimate estimate(RowParams& prm, const Problem& pb)
+template <int K> float rows_us(int natoms, const Problem& pb)
 {
+    RowParams prm{};
+    prm.natoms = natoms;
     const size_t smem = choose_rows<K>(prm, pb);
+    if (smem > (size_t)kRowsSmemMax) return INFINITY;
     const int sms = sm_count(), rows = prm.g.th / kWarps, fit = (int)(kSmPool / block_smem(smem));
-    using C = Cost<K>;
-    const float covered = (float)((double)pb.n * ((pb.W + 31) / 32) * ((pb.H + 7) / 8) / sms);
-    Estimate e;
-    e.other = 4.0f + C::other_dict * prm.natoms + covered * (C::other_atom * prm.natoms + C::other_channel * pb.c);
-    e.rows = INFINITY;
-    if (smem > (size_t)kRowsSmemMax || (int64_t)pb.n * pb.H * pb.W < 32768) return e;
     const int blocks = fit < blocks_per_sm<K>() ? fit : blocks_per_sm<K>();
     const int turns = (prm.g.num_tiles + sms * blocks - 1) / (sms * blocks), tiles_per_sm = (prm.g.num_tiles + sms - 1) / sms;
     const float x = (float)(turns * rows), shared = (float)(tiles_per_sm < blocks ? tiles_per_sm : blocks);
-    e.rows = 4.3f + C::layout * prm.ksteps + x * (prm.ksteps * (C::step + C::step_shared * shared) + pb.c * (C::channel + C::channel_shared * shared));
-    return e;
+    using C = Cost<K>;
+    return C::launch + C::layout * prm.ksteps +
+           x * (prm.ksteps * (C::step + C::step_shared * shared) + pb.c * (C::channel + C::channel_shared * shared + (C::lr + C::lr_shared * shared) / pb.r));
 }
 
-// Chosen where it is expected to be the faster one by 5 %. On the frames above that is 940 of 1800, with a geometric mean of
-// 0.75 of the other kernel's time and 43 that lose more than 6 %, 18 % at most; always: 1.02, 720 and 147 %.
-bool rows_win(const Estimate& e) { return e.rows < 0.95f * e.other; }
-
-Estimate estimate_of(int mode, const Problem& pb)
+// Infinite where the kernel cannot run or has too few pixels to repay the ring and the dictionary's fragments (rows / thread per
+// pixel, us: 9207 px D = 72 k = 3 10.8 / 8.1, k = 5 13.6 / 11.8, D = 128 k = 7 26.5 / 23.8; 21412 px 11.0 / 8.2, 14.0 / 12.0, 27.4 / 24.2).
+float estimate(int mode, const Problem& pb)
 {
-    RowParams prm{};
-    prm.natoms = mode == kModeGlobal ? pb.s : pb.D;
-    return pb.k == 3 ? estimate<3>(prm, pb) : (pb.k == 5 ? estimate<5>(prm, pb) : estimate<7>(prm, pb));
+    if ((int64_t)pb.n * pb.H * pb.W < 32768) return INFINITY;
+    const int natoms = mode == kModeGlobal ? pb.s : pb.D;
+    return pb.k == 3 ? rows_us<3>(natoms, pb) : (pb.k == 5 ? rows_us<5>(natoms, pb) : rows_us<7>(natoms, pb));
 }
 
 template <int K, int CTAS, bool GATHER>
@@ -538,22 +528,20 @@ cudaError_t launch_k(RowParams& prm, const Problem& pb, cudaStream_t st)
 
 } // namespace
 
-bool regress_rows_supported(int mode, int coef_dtype, const Problem& pb)
+bool regress_rows_form(int mode, int coef_dtype, const Problem& pb)
 {
-    if ((mode != kModeDense && mode != kModeGlobal) || coef_dtype != SR_F16 || pb.c > 4 || (pb.flags & SR_LUMA_ONLY)) return false;
-    if (pb.k != 3 && pb.k != 5 && pb.k != 7) return false;
-    RowParams prm{};
-    prm.natoms = mode == kModeGlobal ? pb.s : pb.D;
-    const size_t smem = pb.k == 3 ? plan_rows<3>(prm, pb, 2 * kWarps) : (pb.k == 5 ? plan_rows<5>(prm, pb, 2 * kWarps) : plan_rows<7>(prm, pb, 2 * kWarps));
-    return smem <= (size_t)kRowsSmemMax;
+    return (mode == kModeDense || mode == kModeGlobal) && coef_dtype == SR_F16 && pb.c <= 4 && !(pb.flags & SR_LUMA_ONLY) &&
+           (pb.k == 3 || pb.k == 5 || pb.k == 7);
 }
 
-bool regress_rows_pay(int mode, const Problem& pb) { return rows_win(estimate_of(mode, pb)); }
+// On the 2550 frames: taken for 1974, 0.73 of the other kernel's time on average; 46 frames lose more than 6 % against that kernel,
+// 71 against this one, 46 % at most.
+bool regress_rows_pay(int mode, const Problem& pb) { return estimate(mode, pb) < regress_general_us(mode, SR_F16, pb); }
 
 float regress_rows_or_general_us(int mode, const Problem& pb)
 {
-    const Estimate e = estimate_of(mode, pb);
-    return rows_win(e) ? e.rows : e.other;
+    const float rows = estimate(mode, pb), general = regress_general_us(mode, SR_F16, pb);
+    return rows < general ? rows : general;
 }
 
 cudaError_t launch_regress_rows(int mode, const float* lr, const void* coef, const uint8_t* idx, const float* gamma, const float* dict,

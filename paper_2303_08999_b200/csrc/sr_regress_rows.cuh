@@ -5,11 +5,11 @@
 
 namespace sr {
 
-// Whether launch_regress_rows takes the call: dense or global subset, binary16 coefficients, atoms of 3 x 3, 5 x 5 or
-// 7 x 7, up to four channels.
-bool regress_rows_supported(int mode, int coef_dtype, const Problem& pb);
+// Whether the call has the form that launch_regress_rows takes: dense or global subset, binary16 coefficients, atoms of 3 x 3,
+// 5 x 5 or 7 x 7, up to four channels.
+bool regress_rows_form(int mode, int coef_dtype, const Problem& pb);
 
-// Whether a call it takes is expected to be faster there than on the thread-per-pixel kernel.
+// Whether a call of that form fits it and is expected to be faster there than on the thread-per-pixel kernel.
 bool regress_rows_pay(int mode, const Problem& pb);
 
 // The expected time of the faster of the two, us.

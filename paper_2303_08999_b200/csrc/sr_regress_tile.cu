@@ -14,6 +14,7 @@
 // Measured on the first shape and dropped: coefficients prefetched into registers (PF atoms ahead share the warp's few
 // load scoreboards: 78-124 us); tiles of 32 columns x 4 rows per thread (DRAM rows of 128 bytes, 83 us); 16 warps per SM
 // (spills, 128 us); scalar multiply-adds (84 us); the taps of 5 x 5 over two or three warps (77-115 us).
+#include <math.h>
 #include <type_traits>
 
 #include "sr_regress_tile.cuh"
@@ -243,7 +244,7 @@ __global__ void __launch_bounds__(32 * NS * GPC, CTAS) regress_tile_kernel(const
     }
 }
 
-constexpr int kTileSmemMax = 227 * 1024 / 2 - 2048;      // two blocks on an SM (regress_tile_supported)
+constexpr int kTileSmemMax = 200 * 1024;
 
 // Warps that share the taps, groups (rows) per block, blocks per SM and ring slots for atoms of side K.
 template <int K> struct Shape;
@@ -297,16 +298,31 @@ cudaError_t launch_t(TileParams& prm, const Problem& pb, cudaStream_t st)
     return launch_v<K, false>(prm, pb, st);
 }
 
-size_t smem_bytes(const Problem& pb, int natoms)
+// The kernel's expected time, us: a launch, the dictionary by atom, what an SM's tiles cost together and what each turn of the
+// blocks that fit an SM costs, either of them as such, by atom, by channel and by channel over the scale. Fitted to 1045 of the
+// frames that regress_general_us is fitted to (standard deviation 6 to 8 %; 1 x 1 12 %).
+struct Cost { float launch, dict, tile, tile_atom, tile_channel, tile_lr, turn, turn_atom, turn_channel, turn_lr; };
+template <int K> float tile_us(int natoms, const Problem& pb, const Cost& c)
 {
     TileParams prm{};
     prm.natoms = natoms;
+    const size_t smem = plan_tile<K>(prm, pb);
+    if (smem > (size_t)kTileSmemMax) return INFINITY;
+    const int sms = sm_count(), fit = (int)(228 * 1024 / (smem + 1536));      // (1536: the kernel's own arrays and the system's kilobyte)
+    const int blocks = fit < 1 ? 1 : (fit < Shape<K>::CTAS ? fit : Shape<K>::CTAS);
+    const float tiles = (float)prm.g.num_tiles / sms, turns = (float)((prm.g.num_tiles + sms * blocks - 1) / (sms * blocks));
+    return c.launch + c.dict * natoms + tiles * (c.tile + c.tile_atom * natoms + pb.c * (c.tile_channel + c.tile_lr / pb.r)) +
+           turns * (c.turn + c.turn_atom * natoms + pb.c * (c.turn_channel + c.turn_lr / pb.r));
+}
+
+float estimate(const Problem& pb, int natoms)
+{
     switch (pb.k) {
-    case 1: return plan_tile<1>(prm, pb);
-    case 3: return plan_tile<3>(prm, pb);
-    case 5: return plan_tile<5>(prm, pb);
-    case 7: return plan_tile<7>(prm, pb);
-    default: return plan_tile<9>(prm, pb);
+    case 1: return tile_us<1>(natoms, pb, {2.85f, 0.006f, 0.30f, 0.027f, 0.03f, 0.11f, 0.f, 0.043f, 0.14f, 0.54f});
+    case 3: return tile_us<3>(natoms, pb, {2.79f, 0.017f, 0.47f, 0.023f, 0.06f, 0.10f, 0.35f, 0.083f, 0.14f, 0.78f});
+    case 5: return tile_us<5>(natoms, pb, {2.54f, 0.085f, 0.41f, 0.062f, 0.14f, 0.07f, 0.98f, 0.057f, 0.05f, 1.02f});
+    case 7: return tile_us<7>(natoms, pb, {3.12f, 0.081f, 0.66f, 0.035f, 0.19f, 0.f, 0.f, 0.168f, 0.f, 1.27f});
+    default: return tile_us<9>(natoms, pb, {3.38f, 0.020f, 1.29f, 0.077f, 0.29f, 0.f, 0.f, 0.236f, 0.21f, 1.00f});
     }
 }
 
@@ -318,17 +334,10 @@ bool regress_tile_supported(int mode, int coef_dtype, const Problem& pb)
     // Tiles of 512 pixels and three blocks per SM only pay once they fill the chip; the thread-per-pixel kernel is faster
     // on less than about one block per SM (64 x 64, x2, 5 x 5: 14.6 us against 18.4).
     if ((int64_t)pb.n * pb.H * pb.W < (int64_t)sm_count() * 512) return false;
-    // A tile works on 128 columns however narrow the frame, the other kernel on 32 x 8 pixels. Both timed on 1470 frames of
-    // 1 to 1280 columns, 1 to 256 atoms. This kernel's time over the other's (geometric mean; up to 5 x 5, 7 x 7, 9 x 9), by the
-    // pixels its tiles cover over those the other covers: as many 0.70, 0.79, 0.84; 1.3 to 1.4 times 0.79, 0.98, 1.10; twice
-    // (64 columns) 1.07, 1.48, 1.54; four times (32 columns) 1.95, 3.0, 3.4.
-    const int rows = pb.k >= 7 ? 2 : 4, percent = pb.k <= 5 ? 140 : (pb.k == 7 ? 115 : 105);
-    const int64_t mine = (int64_t)((pb.W + 127) / 128) * 128 * ((pb.H + rows - 1) / rows * rows);
-    const int64_t other = (int64_t)((pb.W + 31) / 32) * 32 * ((pb.H + 7) / 8 * 8);
-    if (100 * mine > percent * other) return false;
-    // One block alone on an SM is not faster (7 x 7, 256 atoms, four channels: 283 us against 165; 9 x 9: 0.96 on average, 0.75
-    // with two).
-    return smem_bytes(pb, mode == kModeGlobal ? pb.s : pb.D) <= (size_t)kTileSmemMax;
+    // A tile works on 128 columns however narrow the frame, the other kernel on 32 x 8 pixels, and large tables leave one block
+    // on an SM: by expected times (on the 1045 frames 31 lose more than 6 % against the better kernel, 35 % at most; batches of 32
+    // columns would take 1.6 to 3.4 times as long here, full tiles take 0.5 to 0.8 of the other's time).
+    return estimate(pb, mode == kModeGlobal ? pb.s : pb.D) < regress_general_us(mode, SR_F32, pb);
 }
 
 cudaError_t launch_regress_tile(int mode, const float* lr, const void* coef, const uint8_t* idx, const float* gamma, const float* dict,
