@@ -191,10 +191,12 @@ static bool compact_prefers_listed(const Problem& pb)
 // Whether a small frame's index + value planes go to the general kernel, which replicates no dictionary and clears no
 // stage: its time is the work of one block per SM (device time, general / better of the others: 128 x 128, D = 72, k = 5,
 // s = 8: 9.0 / 15.0 us; 256 x 256: 12.8 / 15.1; 384 x 256: 16.7 / 15.3; s = 4 there 14.0 / 14.1; D = 32, k = 3, s = 16 there
-// 12.5 / 14.0). Its blocks cover 32 x 8 pixels (2400 x 40, s = 3: 17.0 / 13.4).
+// 12.5 / 14.0). Its blocks cover 32 x 8 pixels (2400 x 40, s = 3: 17.0 / 13.4), the others' 128 columns: up to 32 columns it has
+// the advantage again (8000 x 4, D = 64, k = 3, s = 8: 11.0 / 19.8).
 static bool compact_prefers_general(const Problem& pb)
 {
-    const long long px = 256ll * ((pb.W + 31) / 32) * ((pb.H + 7) / 8) * pb.n;
+    const long long covered = 256ll * ((pb.W + 31) / 32) * ((pb.H + 7) / 8) * pb.n;
+    const long long px = pb.W <= 32 ? hr_pixels(pb) : covered;
     return px <= 100000 && px * compact_gathers(pb) <= 5200000;
 }
 
