@@ -8,15 +8,20 @@
 //        F_{W,beta} = Phi diag(beta) D), G = Z^T Z, b = Z^T h, hh = h^T h for the target image h. Patches, responses and
 //        a register-tiled fp32 rank update, summed in fp64; every CTA leaves its sums in a slot of scratch memory and a
 //        second kernel adds the slots in a fixed order (no atomics: results are reproducible).
-//  selection_search_kernel   Algorithm 1 on G, b, hh in fp64 by ONE thread block: LASSO by cyclic coordinate descent
+//  selection_search_kernel   Algorithm 1 on G, b, hh in fp64 by one cluster of thread blocks: LASSO by cyclic coordinate descent
 //        (Eq. 7), lambda doubling and bisection to || beta ||_0 ~ alpha_t L, least-squares re-fit of gamma on the
 //        support (Eq. 9, Cholesky), gamma folded into G and b, next alpha_t. Every element-wise update and every sum runs
 //        in the same order as a sequential program, with separate multiplies and adds (no contraction), so the result
 //        does not depend on the parallelisation.
+#include <cooperative_groups.h>
+#include <type_traits>
+
 #include "sr_common.cuh"
 #include "sr_selection.cuh"
 
 namespace sr {
+
+namespace cg = cooperative_groups;
 
 namespace {
 
@@ -469,22 +474,30 @@ cudaError_t launch_gram_k(const GramParams& p, int T, int ctas, size_t smem, cud
     return T == 4 ? launch_gram_kt<K, 4>(p, ctas, smem, st) : launch_gram_kt<K, 8>(p, ctas, smem, st);
 }
 
-// ---- Algorithm 1 in one thread block -----------------------------------------------------------------------------------
+// ---- Algorithm 1 in one cluster of thread blocks ------------------------------------------------------------------------
 //
 // The sweeps of coordinate descent are one serial chain in fp64: coordinate l's step needs the residual that coordinate
 // l - 1's step left. One warp walks it; four warps share what is parallel (residuals, factorisation, re-scaling).
 // The active atoms are kept compacted (index 0 .. na - 1, order of the atoms), so no step ever looks at a dropped one.
 //
-// What bounds a sweep is the latency of that chain, so everything else is kept off it. Coordinates go in blocks of
-// eight: all lanes hold the block's eight residuals, make its eight steps redundantly and apply each step to the
-// residuals that follow in the block; the residuals of all atoms (lane, lane + 32, ...) get the eight steps afterwards,
-// in the same order, behind the next steps. A step is then ten dependent fp64 operations: two additions to the
-// thresholded numerator, five for the quotient, one for the step, a product and a sum to the next residual; no shuffle,
-// no shared-memory load and no branch among them. Every rounding is that of the sequential program, so the results are
-// the same bits.
-// 72 atoms down to 8 in four steps (about 90 solves, 90 000 steps): 46.0 -> 9.3 ms against one warp that kept residuals and
-// coefficients in shared memory and divided inside the chain.
+// What bounds a sweep is the latency of that chain, so everything else is kept off it. Lane m holds the residuals of
+// coordinates m, m + 32, ...; all lanes make every step redundantly. The residual a step needs reaches them by a shuffle that
+// leaves two steps earlier, and gets the last step's change in every lane: no shuffle and no load stands between two
+// steps. A step is then six dependent fp64 operations: two additions to the thresholded numerator, one
+// multiply-add for the quotient, one addition for the step, a product and a sum to the next residual. Every rounding is that
+// of the sequential program, so the results are the same bits.
+//
+// The bisection's solves all start from the same coefficients until one of them is kept. So each round solves the whole
+// tree of the next five mid points, one per warp of a cluster of eight blocks (a warp per scheduler: nobody slows the
+// chains down), and then walks it as the sequential program would. The blocks run everything else alike.
+// 72 atoms down to 8 in four steps (about 90 solves, 90 000 steps, 33 000 of them in bisections): 8.7 -> 6.0 ms against one block
+// with eleven operations to a step, a bisection's solves one after the other (46 ms with one warp that divided inside the chain).
+// Left are some 165 clocks a step: about 60 instructions of one warp, fp64 at two clocks each, around a chain of 75.
 constexpr int kSearchThreads = 128;
+constexpr int kSearchWarps = kSearchThreads / 32;
+constexpr int kSearchCtas = 8;                     // blocks of the cluster
+constexpr int kTreeLevels = 5;                     // 31 of the 32 warps have a node
+static_assert((1 << kTreeLevels) - 1 <= kSearchCtas * kSearchWarps, "a warp per node");
 constexpr int kCdBlock = 8;
 
 struct SearchParams {
@@ -502,14 +515,18 @@ struct SearchParams {
 };
 
 struct SearchState {
-    double* G;            // [L8][Lp], active atoms only; columns na .. na8 - 1 are zero
+    double* G;            // [L8][Lp], active atoms only; rows and columns na .. na8 - 1 are zero
     double* A;            // packed lower triangle
-    double *b, *beta, *r, *best, *cand, *gtot, *tmp, *prod;
-    double *diag, *rcp, *frz;   // G[l][l], 1 / G[l][l], and 0 or (atoms whose G[l][l] is not positive: never moved) infinity
+    double *b, *beta, *r, *best, *gtot, *tmp, *prod;
+    double *diag, *rcp, *rcl, *frz;  // G[l][l], 1 / G[l][l] rounded and what the rounding left of it, and 0 or (atoms whose G[l][l] is not
+                                     // positive: never moved) infinity
+    double* sub;          // G[l + 1][l]; of the last coordinate G[0][na8 - 1]
+    double* solve;        // [warps][2][L8]: a warp's coefficients, old and new ones of a sweep
     int *S, *orig;        // support; compact index -> atom
     int L8, Lp, na, na8, tid, lane;
     double nrows;
     bool safe;            // every positive G[l][l] lies in [2^-300, 2^300]
+    bool frozen;          // some G[l][l] is not positive
 };
 
 __host__ __device__ constexpr int search_l8(int L) { return (L + kCdBlock - 1) / kCdBlock * kCdBlock; }
@@ -526,95 +543,167 @@ __device__ int count_nonzero(const SearchState& s, const double* beta)   // ever
 __device__ void prepare_active(SearchState& s)
 {
     s.na8 = search_l8(s.na);
-    int bad = 0;
+    int bad = 0, dead = 0;
     for (int l = s.tid; l < s.L8; l += kSearchThreads) {
         const double g = l < s.na ? s.G[l * s.Lp + l] : 0.0;
         const bool live = g > 0.0;
+        const double y = live ? __drcp_rn(g) : 0.0;
         s.diag[l] = g;
-        s.rcp[l] = live ? __drcp_rn(g) : 0.0;
+        s.rcp[l] = y;
+        s.rcl[l] = live ? __dmul_rn(__fma_rn(-g, y, 1.0), y) : 0.0;
         s.frz[l] = live ? 0.0 : __longlong_as_double(0x7FF0000000000000ll);
         if (live && !(g >= 0x1p-300 && g <= 0x1p300)) bad = 1;
-        if (l >= s.na) s.beta[l] = s.cand[l] = s.best[l] = s.r[l] = 0.0;
-        for (int m = s.na; m < s.na8; ++m) s.G[l * s.Lp + m] = 0.0;
+        if (l < s.na && !live) dead = 1;
+        if (l >= s.na) s.beta[l] = s.best[l] = s.r[l] = 0.0;
+        for (int m = l < s.na ? s.na : 0; m < s.na8; ++m) s.G[l * s.Lp + m] = 0.0;
     }
     s.safe = !__syncthreads_or(bad);
+    s.frozen = __syncthreads_or(dead);
+    for (int l = s.tid; l < s.na8; l += kSearchThreads) s.sub[l] = s.G[(l + 1 < s.na8 ? l + 1 : 0) * s.Lp + l];
+    __syncthreads();
 }
 
-// num / g rounded to nearest. FAST: y = 1 / g rounded to nearest; an estimate is corrected twice by its exact remainder
-// (Markstein, IBM J. Res. Dev. 34 (1990): if q is one of the two neighbours of the quotient, y the rounded reciprocal
-// and the remainder exact, then q + remainder * y rounds to the rounded quotient; the first correction makes the
-// estimate such a neighbour). The caller has excluded operands that could under- or overflow on the way.
-template <bool FAST> __device__ __forceinline__ double cd_quotient(double num, double g, double y)
+// The plain form: one warp, sweeps over the active atoms until no coefficient moves by more than tol, quotients by division.
+// beta in place; rr: residuals of the coordinates lane, lane + 32, ... Returns the sweeps made; *settled says whether the last one
+// moved nothing.
+__device__ __noinline__ int cd_sweeps_plain(const SearchState& s, double thr, double (&rr)[4], double* beta, double tol, int max_sweeps, bool* settled)
 {
-    if (!FAST) return __ddiv_rn(num, g);
-    double q = __dmul_rn(num, y);
-    q = __fma_rn(__fma_rn(-g, q, num), y, q);
-    return __fma_rn(__fma_rn(-g, q, num), y, q);
+    const int Lp = s.Lp;
+    const double* row[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) row[k] = s.G + min(s.lane + 32 * k, s.L8 - 1) * Lp;
+    int sweep = 0;
+    *settled = false;
+    while (sweep < max_sweeps && !*settled) {
+        double moved = 0.0;
+#pragma unroll 1
+        for (int l = 0; l < s.na; ++l) {
+            double rk = rr[0];
+#pragma unroll
+            for (int k = 1; k < 4; ++k) rk = l >= 32 * k ? rr[k] : rk;
+            const double g = s.diag[l], be = beta[l], fz = s.frz[l];
+            const double rho = __dadd_rn(__shfl_sync(0xffffffffu, rk, l & 31), __dmul_rn(g, be));
+            const double nb = fabs(rho) > __dadd_rn(thr, fz) ? __ddiv_rn(__dadd_rn(rho, -copysign(thr, rho)), g) : (fz > 0.0 ? be : 0.0);
+            const double d = __dadd_rn(nb, -be);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) rr[k] = __dadd_rn(rr[k], -__dmul_rn(d, row[k][l]));
+            moved = fmax(moved, fabs(d));
+            __syncwarp();
+            if (s.lane == 0) beta[l] = nb;
+            __syncwarp();
+        }
+        ++sweep;
+        *settled = moved <= tol;
+    }
+    return sweep;
 }
 
-// Warp 0: sweeps over the active atoms until no coefficient moves by more than tol. Residuals in and out through s.r.
-// Returns the sweeps made, negative when it stopped because a step was too large for the fast quotient's range.
-template <int NK, bool FAST>
-__device__ __noinline__ int cd_sweeps(const SearchState& s, double thr, double* beta, double tol, int max_sweeps)
+__device__ __forceinline__ double with_sign_of(double magnitude, double x)   // magnitude >= 0
 {
-    const int Lp = s.Lp, na8 = s.na8;
+    return __hiloint2double((__double2hiint(x) & 0x80000000) | __double2hiint(magnitude), __double2loint(magnitude));
+}
+
+// One warp; coefficients in buf[0 .. L8), scratch behind them; residuals from s.r. Returns where the coefficients ended up.
+//
+// The quotient num / g, rounded to nearest, is made as q = num y + t with y the rounded reciprocal and t = num (1/g - y), which is known
+// no later than num. That is the rounded quotient but where the quotient lies within about 2^-50 units in the last place of the
+// middle of two numbers. So every q is checked, off the chain: with the remainder of q, q + remainder y rounds to the
+// rounded quotient if q is one of the quotient's two neighbours (Markstein, IBM J. Res. Dev. 34 (1990)), and it differs from q if q is further
+// off (or if anything over- or underflowed). A sweep with a q that fails is made again in the plain form, from the coefficients
+// and residuals it started with.
+template <int NK, bool FROZEN>
+__device__ __noinline__ double* cd_sweeps(const SearchState& s, double thr, double* buf, double tol, int max_sweeps)
+{
+    const int na8 = s.na8;
     double rr[NK];
     const double* row[NK];
 #pragma unroll
     for (int k = 0; k < NK; ++k) {
         const int m = s.lane + 32 * k;
         rr[k] = m < na8 ? s.r[m] : 0.0;
-        row[k] = s.G + min(m, s.L8 - 1) * Lp;
+        row[k] = s.G + min(m, s.L8 - 1) * s.Lp;
     }
-    int sweep = 0;
-    bool too_large = false;
-    while (sweep < max_sweeps && !too_large) {
-        double moved = 0.0;
+    double *cur = buf, *nxt = buf + s.L8;
+    double r0 = s.r[0], r1 = s.r[1];                         // residuals of this step's coordinate and, without the last step, the next one's
+#pragma unroll 1
+    for (int sweep = 0; sweep < max_sweeps; ++sweep) {
+        double was[NK];
+#pragma unroll
+        for (int k = 0; k < NK; ++k) was[k] = rr[k];
+        bool moved = false, bad = false;
 #pragma unroll 1
         for (int l0 = 0; l0 < na8; l0 += kCdBlock) {
-            double rk = rr[0];
+            auto load = [](double (&to)[kCdBlock], const double* from) {
 #pragma unroll
-            for (int k = 1; k < NK; ++k) rk = l0 >= 32 * k ? rr[k] : rk;
-            double rb[kCdBlock], d[kCdBlock], nb[kCdBlock];
-#pragma unroll
-            for (int i = 0; i < kCdBlock; ++i) rb[i] = __shfl_sync(0xffffffffu, rk, (l0 & 31) + i);
-            const double* Gb = s.G + l0 * Lp + l0;
+                for (int i = 0; i < kCdBlock; i += 2) {
+                    const double2 v = *reinterpret_cast<const double2*>(from + i);
+                    to[i] = v.x;
+                    to[i + 1] = v.y;
+                }
+            };
+            double g[kCdBlock], y[kCdBlock], yl[kCdBlock], be[kCdBlock], sub[kCdBlock], nb[kCdBlock];
+            load(g, s.diag + l0);
+            load(be, cur + l0);
+            load(y, s.rcp + l0);
+            load(yl, s.rcl + l0);
+            load(sub, s.sub + l0);
+            const int next = l0 + kCdBlock < na8 ? l0 + kCdBlock : 0;
 #pragma unroll
             for (int i = 0; i < kCdBlock; ++i) {
-                const double g = s.diag[l0 + i], be = beta[l0 + i], fz = s.frz[l0 + i];
-                const double rho = __dadd_rn(rb[i], __dmul_rn(g, be));
-                const double q = cd_quotient<FAST>(__dadd_rn(rho, -copysign(thr, rho)), g, s.rcp[l0 + i]);
-                nb[i] = fabs(rho) > __dadd_rn(thr, fz) ? q : (fz > 0.0 ? be : 0.0);
-                d[i] = __dadd_rn(nb[i], -be);
+                const double rho = __dadd_rn(r0, __dmul_rn(g[i], be[i]));
+                const double num = __dadd_rn(rho, -with_sign_of(thr, rho));
+                const double tl = __dmul_rn(thr, yl[i]);
+                const double t = __fma_rn(rho, yl[i], __hiloint2double((__double2hiint(rho) & 0x80000000) ^ 0x80000000 ^ __double2hiint(tl), __double2loint(tl)));
+                const double q = __fma_rn(num, y[i], t);
+                bool in = fabs(rho) > thr;
+                double out = 0.0;
+                if (FROZEN) {
+                    const bool held = s.frz[l0 + i] > 0.0;
+                    in = in & !held;
+                    out = held ? be[i] : 0.0;
+                }
+                const double d = in ? __dadd_rn(q, -be[i]) : __dadd_rn(out, -be[i]);
+                r0 = __dadd_rn(r1, -__dmul_rn(d, sub[i]));
+                nb[i] = in ? q : out;
+                const double again = __fma_rn(__fma_rn(-g[i], q, num), y[i], q);
+                bad = bad | (in & !(again == q));
+                moved = moved | (fabs(d) > tol);
 #pragma unroll
-                for (int j = i + 1; j < kCdBlock; ++j) rb[j] = __dadd_rn(rb[j], -__dmul_rn(d[i], Gb[j * Lp + i]));
-                moved = fmax(moved, fabs(d[i]));
+                for (int k = 0; k < NK; ++k) rr[k] = __dadd_rn(rr[k], -__dmul_rn(d, row[k][l0 + i]));
+                const int after = i + 2 < kCdBlock ? l0 + i + 2 : next + i + 2 - kCdBlock;
+                double v = rr[0];
+#pragma unroll
+                for (int k = 1; k < NK; ++k) v = after >= 32 * k ? rr[k] : v;
+                r1 = __shfl_sync(0xffffffffu, v, after & 31);
             }
-#pragma unroll
-            for (int i = 0; i < kCdBlock; ++i)
-#pragma unroll
-                for (int k = 0; k < NK; ++k) rr[k] = __dadd_rn(rr[k], -__dmul_rn(d[i], row[k][l0 + i]));
-            __syncwarp();
             if (s.lane == 0) {
 #pragma unroll
-                for (int i = 0; i < kCdBlock; ++i) beta[l0 + i] = nb[i];
+                for (int i = 0; i < kCdBlock; i += 2) *reinterpret_cast<double2*>(nxt + l0 + i) = make_double2(nb[i], nb[i + 1]);
             }
-            __syncwarp();
         }
-        ++sweep;
-        if (moved <= tol) break;
-        if (FAST && !(moved < 0x1p200)) too_large = true;
-    }
+        __syncwarp();
+        if (bad) {                                           // the same in every lane
+            double again[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-    for (int k = 0; k < NK; ++k)
-        if (s.lane + 32 * k < na8) s.r[s.lane + 32 * k] = rr[k];
-    __syncwarp();
-    return too_large ? -sweep : sweep;
+            for (int k = 0; k < NK; ++k) again[k] = was[k];
+            for (int l = s.lane; l < na8; l += 32) nxt[l] = cur[l];
+            __syncwarp();
+            bool settled;
+            cd_sweeps_plain(s, thr, again, nxt, tol, 1, &settled);
+#pragma unroll
+            for (int k = 0; k < NK; ++k) rr[k] = again[k];
+            r0 = __shfl_sync(0xffffffffu, rr[0], 0);
+            r1 = __shfl_sync(0xffffffffu, rr[0], 1);
+            moved = !settled;
+        }
+        double* swap = cur; cur = nxt; nxt = swap;
+        if (!moved && tol == tol) break;
+    }
+    return cur;
 }
 
-// Eq. 7 by cyclic coordinate descent; beta in / out. Same operation order as a sequential loop over the atoms. All
-// threads; starts after a barrier that made beta visible and ends in one.
-__device__ void lasso_cd(const SearchState& s, double lambda, double* beta, double tol, int max_sweeps)
+// s.r = b - G beta; all threads, ends in a barrier.
+__device__ void residuals(const SearchState& s, const double* beta)
 {
     for (int l = s.tid; l < s.na; l += kSearchThreads) {
         double acc = 0.0;
@@ -623,20 +712,29 @@ __device__ void lasso_cd(const SearchState& s, double lambda, double* beta, doub
         s.r[l] = __dadd_rn(s.b[l], -acc);
     }
     __syncthreads();
-    if (s.tid < 32) {
-        const double thr = __dmul_rn(__dmul_rn(0.5, lambda), s.nrows);
-        int done = 0;
-        if (s.safe && thr >= 0x1p-300 && thr <= 0x1p300) {
-            if (s.na8 <= 32) done = cd_sweeps<1, true>(s, thr, beta, tol, max_sweeps);
-            else if (s.na8 <= 64) done = cd_sweeps<2, true>(s, thr, beta, tol, max_sweeps);
-            else if (s.na8 <= 96) done = cd_sweeps<3, true>(s, thr, beta, tol, max_sweeps);
-            else done = cd_sweeps<4, true>(s, thr, beta, tol, max_sweeps);
-            if (done < 0 && -done < max_sweeps) cd_sweeps<4, false>(s, thr, beta, tol, max_sweeps + done);
-        } else {
-            cd_sweeps<4, false>(s, thr, beta, tol, max_sweeps);
-        }
+}
+
+// Eq. 7 by cyclic coordinate descent from `start`, whose residuals are in s.r, by one warp in its own buffers. Same operation
+// order as a sequential loop over the atoms. Returns the coefficients.
+__device__ double* lasso_cd(const SearchState& s, double lambda, const double* start, double tol, int max_sweeps)
+{
+    double* buf = s.solve + (s.tid >> 5) * 2 * s.L8;
+    for (int l = s.lane; l < s.na8; l += 32) { buf[l] = start[l]; buf[s.L8 + l] = 0.0; }
+    __syncwarp();
+    const double thr = __dmul_rn(__dmul_rn(0.5, lambda), s.nrows);
+    if (s.safe && thr >= 0x1p-300 && thr <= 0x1p300) {
+        if (s.frozen) return cd_sweeps<4, true>(s, thr, buf, tol, max_sweeps);
+        if (s.na8 <= 32) return cd_sweeps<1, false>(s, thr, buf, tol, max_sweeps);
+        if (s.na8 <= 64) return cd_sweeps<2, false>(s, thr, buf, tol, max_sweeps);
+        if (s.na8 <= 96) return cd_sweeps<3, false>(s, thr, buf, tol, max_sweeps);
+        return cd_sweeps<4, false>(s, thr, buf, tol, max_sweeps);
     }
-    __syncthreads();
+    double rr[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) rr[k] = s.lane + 32 * k < s.na ? s.r[s.lane + 32 * k] : 0.0;
+    bool settled;
+    cd_sweeps_plain(s, thr, rr, buf, tol, max_sweeps, &settled);
+    return buf;
 }
 
 // All threads; every thread returns the loss. Starts after a barrier that made beta visible.
@@ -709,17 +807,24 @@ __device__ bool refit_gamma(const SearchState& s, int ns)
     return true;
 }
 
-__global__ void __launch_bounds__(kSearchThreads, 1) selection_search_kernel(const __grid_constant__ SearchParams p)
+__global__ void __cluster_dims__(kSearchCtas, 1, 1) __launch_bounds__(kSearchThreads, 1)
+selection_search_kernel(const __grid_constant__ SearchParams p)
 {
     extern __shared__ __align__(16) double ssm[];
+    __shared__ int sCount[kSearchWarps], sAt[kSearchWarps];   // this block's nodes: coefficients that are not zero, and where they are
+    __shared__ int sTree[kSearchCtas * kSearchWarps][2];      // the same of all blocks
+    cg::cluster_group cluster = cg::this_cluster();
+    const int cta = (int)cluster.block_rank();
     SearchState s;
     const int L = p.L;
     s.L8 = search_l8(L); s.Lp = s.L8 + 1; s.tid = threadIdx.x; s.lane = threadIdx.x & 31; s.nrows = p.nrows;
     s.na = L;
     double* v = ssm;
-    s.diag = v; v += s.L8; s.rcp = v; v += s.L8; s.frz = v; v += s.L8;
-    s.b = v; v += s.L8; s.beta = v; v += s.L8; s.r = v; v += s.L8; s.best = v; v += s.L8; s.cand = v; v += s.L8;
+    s.diag = v; v += s.L8; s.rcp = v; v += s.L8; s.rcl = v; v += s.L8; s.frz = v; v += s.L8;
+    s.b = v; v += s.L8; s.beta = v; v += s.L8; s.r = v; v += s.L8; s.best = v; v += s.L8;
     s.gtot = v; v += s.L8; s.tmp = v; v += s.L8; s.prod = v; v += s.L8;
+    s.sub = v; v += s.L8;
+    s.solve = v; v += kSearchWarps * 2 * s.L8;
     s.G = v; v += s.L8 * s.Lp;
     s.A = v; v += L * (L + 1) / 2;
     s.S = reinterpret_cast<int*>(v);
@@ -745,7 +850,12 @@ __global__ void __launch_bounds__(kSearchThreads, 1) selection_search_kernel(con
         double lam_hi = lambda;
         // doubling
         while ((double)nnz > target) {
-            lasso_cd(s, lambda, s.beta, p.tol, p.max_sweeps);
+            residuals(s, s.beta);
+            if (tid < 32) {
+                const double* now = lasso_cd(s, lambda, s.beta, p.tol, p.max_sweeps);
+                for (int l = s.lane; l < s.na; l += 32) s.beta[l] = now[l];
+            }
+            __syncthreads();
             ++solves;
             nnz = count_nonzero(s, s.beta);
             lam_hi = lambda;
@@ -758,25 +868,53 @@ __global__ void __launch_bounds__(kSearchThreads, 1) selection_search_kernel(con
         copy(s.best, s.beta);
         int best_nnz = nnz;
         double best_lam = lam_hi;
-        // bisection inside the last doubling step
+        // bisection inside the last doubling step: warp w of the cluster solves node w + 1 of the tree of mid points below
+        // [left, right] (children of node i: 2 i, the lower half, and 2 i + 1), then every block walks down that tree. The walk ends
+        // where the coefficients that all of it started from are replaced.
         double left = __dmul_rn(0.5, lam_hi), right = lam_hi;
         int it = 0;
+        bool stale = true;                                     // s.r does not belong to s.best
         while (fabs(__dadd_rn(target, -(double)nnz)) > band && it < p.max_bisect) {
-            const double mid = __dmul_rn(0.5, __dadd_rn(left, right));
-            copy(s.cand, s.best);
-            lasso_cd(s, mid, s.cand, p.tol, p.max_sweeps);
-            ++solves;
-            ++it;
-            nnz = count_nonzero(s, s.cand);
-            const bool in_band_feasible = fabs(__dadd_rn(target, -(double)nnz)) <= band && (double)nnz <= target;
-            if (((double)nnz <= target && nnz > best_nnz) || in_band_feasible) {
-                copy(s.best, s.cand);
-                best_nnz = nnz;
-                best_lam = mid;
+            if (stale) residuals(s, s.best);
+            stale = false;
+            const int node = cta * kSearchWarps + (tid >> 5) + 1, level = 31 - __clz(node);
+            if (level < kTreeLevels && it + level < p.max_bisect) {
+                double lo = left, hi = right, mid = __dmul_rn(0.5, __dadd_rn(lo, hi));
+                for (int u = level - 1; u >= 0; --u) {
+                    if ((node >> u) & 1) lo = mid;
+                    else hi = mid;
+                    mid = __dmul_rn(0.5, __dadd_rn(lo, hi));
+                }
+                const double* now = lasso_cd(s, mid, s.best, p.tol, p.max_sweeps);
+                const int count = count_nonzero(s, now);
+                if (s.lane == 0) { sCount[tid >> 5] = count; sAt[tid >> 5] = (int)(now - s.solve); }
             }
-            if ((double)nnz < target) right = mid;
-            else if ((double)nnz > target) left = mid;
+            cluster.sync();
+            if (tid < kSearchCtas * kSearchWarps) {
+                sTree[tid][0] = cluster.map_shared_rank(sCount, tid / kSearchWarps)[tid % kSearchWarps];
+                sTree[tid][1] = cluster.map_shared_rank(sAt, tid / kSearchWarps)[tid % kSearchWarps];
+            }
             __syncthreads();
+            int at = 1;
+            while (at < (1 << kTreeLevels) && fabs(__dadd_rn(target, -(double)nnz)) > band && it < p.max_bisect) {
+                const double mid = __dmul_rn(0.5, __dadd_rn(left, right));
+                ++solves;
+                ++it;
+                nnz = sTree[at - 1][0];
+                const bool in_band_feasible = fabs(__dadd_rn(target, -(double)nnz)) <= band && (double)nnz <= target;
+                if (((double)nnz <= target && nnz > best_nnz) || in_band_feasible) {
+                    const double* from = cluster.map_shared_rank(s.solve, (at - 1) / kSearchWarps) + sTree[at - 1][1];
+                    for (int l = tid; l < s.na; l += kSearchThreads) s.best[l] = from[l];
+                    best_nnz = nnz;
+                    best_lam = mid;
+                    stale = true;
+                }
+                if ((double)nnz < target) { right = mid; at = 2 * at; }
+                else if ((double)nnz > target) { left = mid; at = 2 * at + 1; }
+                else break;                                    // the interval stays: the same mid point again
+                if (stale) break;
+            }
+            cluster.sync();                                    // everybody has read the nodes
         }
         copy(s.beta, s.best);
         lambda = best_lam;
@@ -821,13 +959,14 @@ __global__ void __launch_bounds__(kSearchThreads, 1) selection_search_kernel(con
         __syncthreads();
         prepare_active(s);
         const double loss_gamma = selection_loss(s, hh, s.beta);
-        if (p.trace && tid == 0) {
+        if (p.trace && cta == 0 && tid == 0) {
             double* tr = p.trace + (size_t)step * 6;
             tr[0] = alpha_next; tr[1] = best_lam; tr[2] = (double)ns; tr[3] = loss_beta; tr[4] = loss_gamma; tr[5] = (double)solves;
         }
         alpha_t = alpha_next;
         ++step;
     }
+    if (cta != 0) return;
     if (!failed)
         for (int l = tid; l < s.na; l += kSearchThreads) { p.idx_out[l] = (uint8_t)s.orig[l]; p.gamma_out[l] = (float)s.gtot[l]; }
     if (tid == 0) {
@@ -969,7 +1108,7 @@ cudaError_t launch_selection_search(const double* G, const double* b, const doub
     p.idx_out = idx_out; p.gamma_out = gamma_out; p.count_out = count_out; p.trace = trace; p.steps_out = steps_out;
     constexpr auto bytes = [](int l) {
         const size_t l8 = search_l8(l);
-        return (11 * l8 + l8 * (l8 + 1) + (size_t)l * (l + 1) / 2) * sizeof(double) + 2 * l8 * sizeof(int);
+        return (12 * l8 + kSearchWarps * 2 * l8 + l8 * (l8 + 1) + (size_t)l * (l + 1) / 2) * sizeof(double) + 2 * l8 * sizeof(int);
     };
     static bool configured[64] = {false};
     int dev = 0;
@@ -979,7 +1118,7 @@ cudaError_t launch_selection_search(const double* G, const double* b, const doub
         if (e != cudaSuccess) return e;
         configured[dev] = true;
     }
-    selection_search_kernel<<<1, kSearchThreads, bytes(L), st>>>(p);
+    selection_search_kernel<<<kSearchCtas, kSearchThreads, bytes(L), st>>>(p);
     count_launches(1);
     return cudaGetLastError();
 }

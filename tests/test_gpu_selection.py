@@ -145,7 +145,7 @@ def test_gram_adds_at_most_the_terms_of_32_pixels_in_fp32(D, n, h, w):
         assert np.abs(got - want).max() <= 16.5 * 2.0 ** -24 * want
 
 
-@pytest.mark.parametrize("D", [1, 7, 8, 9, 31, 33, 64, 65, 97, 128])
+@pytest.mark.parametrize("D", [7, 8, 9, 31, 33, 64, 65, 97, 128])
 @pytest.mark.parametrize("scale", [1.0, 2.0 ** -700, 2.0 ** 640])
 def test_search_bits_at_block_edges_and_extreme_scales(D, scale):
     # coordinate blocks of eight, residuals in registers of 32: both sides of their edges; statistics scaled by a power of
@@ -171,3 +171,30 @@ def test_search_ends_when_no_lambda_removes_enough_atoms(diag, lambda0):
     b = np.where(np.array(diag) > 0, 1.0, 0.0)
     with pytest.raises(sr.SrError):
         sr.sr_selection_search(dev(np.diag(diag)), dev(b), dev(np.array([5.0])), 10, 0.25, 0.25, 0.0, lambda0)
+
+
+@pytest.mark.parametrize("D", [7, 8, 31, 33, 64, 65, 96, 97, 128])
+@pytest.mark.parametrize("max_bisect", [1, 4, 5, 6, 30])
+def test_search_bits_over_atoms_and_bisections(D, max_bisect):
+    # sizes on both sides of the warp's rows of 32 coordinates and the blocks of eight; bisections on both sides of a tree of five levels
+    rng = np.random.default_rng(D)
+    Z = rng.normal(size=(600, D)) * np.exp(-3.0 * rng.permutation(D) / D) + 0.1 * rng.normal(size=(600, 1))
+    h = Z.sum(1) + 0.05 * rng.normal(size=600)
+    G, b, hh = Z.T @ Z, Z.T @ h, h @ h
+    args = (600.0, 0.25, 0.3, 0.0, 1e-7)
+    want = oracle.selection_search(G, b, hh, *args, tol=1e-9, max_sweeps=500, max_bisect=max_bisect)
+    idx, gamma, trace = sr.sr_selection_search(dev(G), dev(b), dev(np.array([hh])), *args, tol=1e-9, max_sweeps=500, max_bisect=max_bisect)
+    np.testing.assert_array_equal(host(idx), want[0])
+    np.testing.assert_array_equal(host(trace), want[2])
+    np.testing.assert_array_equal(host(gamma), want[1].astype(np.float32))
+
+
+def test_search_where_a_quotient_lies_next_to_the_middle_of_two_numbers():
+    # 1 / (1 - 2^-53) = 1 + 2^-53 + 2^-106: the quotient made from the rounded reciprocal and its remainder is off by one unit, and the
+    # sweep is made again by division; hh makes the loss the difference of the two
+    G, b = np.diag([1.0 - 2.0 ** -53, 4.0]), np.array([2.0, 0.5])
+    hh = 2 * b[0] * 1.0 - G[0, 0]
+    want = oracle.selection_search(G, b, hh, 2, 0.5, 0.5, 0.0, 1.0, tol=1e-9, max_sweeps=50)
+    idx, gamma, trace = sr.sr_selection_search(dev(G), dev(b), dev(np.array([hh])), 2, 0.5, 0.5, 0.0, 1.0, max_sweeps=50)
+    np.testing.assert_array_equal(host(idx), want[0])
+    np.testing.assert_array_equal(host(trace), want[2])
