@@ -11,6 +11,9 @@
 // per pixel and atom and is held by the shared-memory pipe at a quarter of that rate. 180 x 320 x3, D = 72, k = 5:
 // 118 -> 69 us (27 at the FMA pipe's rate); 540 x 960 x4: 1885 -> 784 us. Where the rest goes: up-sampling, set-up and
 // filtering are a third of the instructions, and 12 warps per SM (168 registers) do not hide every load.
+// With aligned rows a lane copies the sixteen bytes it reads itself, from a running address: no warp barrier and no table of
+// planes in the loop over the atoms (540 x 960 x2, D = 72: 209.4 -> 203.5 us; 3 x 3 270 x 480 x4: 118.3 -> 111; 7 x 7, D = 128,
+// 180 x 320 x3: 205 -> 197; the first shape 64.0 -> 63.4).
 // Measured on the first shape and dropped: coefficients prefetched into registers (PF atoms ahead share the warp's few
 // load scoreboards: 78-124 us); tiles of 32 columns x 4 rows per thread (DRAM rows of 128 bytes, 83 us); 16 warps per SM
 // (spills, 128 us); scalar multiply-adds (84 us); the taps of 5 x 5 over two or three warps (77-115 us).
@@ -58,8 +61,9 @@ constexpr int kStageBytes = 512;                         // a ring slot: 128 pix
 
 template <int K> __host__ __device__ constexpr int dict_pitch() { return (K * K / 4) * 4 + 4; }   // the 16-byte units, the last tap, zeros
 
-// K: atom side; NS: warps that share the taps; GPC: such groups (rows) per block; CTAS: blocks per SM; VEC: 16-byte copies
-template <int K, int NS, int GPC, int CTAS, int DEPTH, bool VEC>
+// K: atom side; NS: warps that share the taps; GPC: such groups (rows) per block; CTAS: blocks per SM; VEC: 16-byte copies; GATHER: planes by table (always
+// without VEC), else one after the other
+template <int K, int NS, int GPC, int CTAS, int DEPTH, bool VEC, bool GATHER>
 __global__ void __launch_bounds__(32 * NS * GPC, CTAS) regress_tile_kernel(const __grid_constant__ TileParams p)
 {
     constexpr int kk = K * K, P = (K - 1) / 2, UNITS = kk / 4, U = UNITS / NS, PITCH = dict_pitch<K>();
@@ -96,14 +100,16 @@ __global__ void __launch_bounds__(32 * NS * GPC, CTAS) regress_tile_kernel(const
     const int row = min(w.y0 + grp, H - 1), x = w.x0 + PX * lane;
     const float* row0 = p.coef + (int64_t)row * W + w.x0;
     const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring);
+    const float* mine = row0 + (x < W ? PX * lane : 0) + (GATHER ? 0 : (int64_t)w.f * p.planes * HW);   // VEC: this lane's pixels
+    const uint32_t mine_bytes = x < W ? 16u : 0u, mine_s = ring_s + 16 * lane;
     auto fetch = [&](int l, uint32_t slot) {
         if (l < natoms) {
-            const float* src = row0 + sOff[l];
-            const uint32_t dst = ring_s + slot;
             if constexpr (VEC) {
-                const bool in = x < W;
-                cp16(dst + 16 * lane, src + (in ? PX * lane : 0), in ? 16u : 0u);
+                cp16(mine_s + slot, GATHER ? mine + sOff[l] : mine, mine_bytes);
+                if (!GATHER) mine += HW;
             } else {
+                const float* src = row0 + sOff[l];
+                const uint32_t dst = ring_s + slot;
 #pragma unroll
                 for (int i = 0; i < PX; ++i) {
                     const int c = lane + 32 * i;
@@ -144,7 +150,7 @@ __global__ void __launch_bounds__(32 * NS * GPC, CTAS) regress_tile_kernel(const
 #pragma unroll 2
     for (int l = 0; l < natoms; ++l, dl += PITCH) {
         cp_wait<DEPTH - 2>();
-        __syncwarp();                                        // every lane's part of the piece has landed; the slot read last is free
+        if (!VEC) __syncwarp();                              // every lane's part of the piece has landed; the slot read last is free (VEC: a lane reads what it copied)
         const float4 v4 = *reinterpret_cast<const float4*>(ring + slot + 16 * lane);
         const float v[PX] = {v4.x, v4.y, v4.z, v4.w};
         fetch(l + DEPTH - 1, free_slot);
@@ -269,13 +275,13 @@ template <int K> size_t plan_tile(TileParams& prm, const Problem& pb)
     return (size_t)prm.off_ring * sizeof(float) + (size_t)S::NS * S::GPC * S::DEPTH * kStageBytes;
 }
 
-template <int K, bool VEC>
+template <int K, bool VEC, bool GATHER>
 cudaError_t launch_v(TileParams& prm, const Problem& pb, cudaStream_t st)
 {
     using S = Shape<K>;
     const size_t smem = plan_tile<K>(prm, pb);
     if (smem > (size_t)kTileSmemMax) return cudaErrorNotSupported;
-    auto kern = regress_tile_kernel<K, S::NS, S::GPC, S::CTAS, S::DEPTH, VEC>;
+    auto kern = regress_tile_kernel<K, S::NS, S::GPC, S::CTAS, S::DEPTH, VEC, GATHER>;
     static bool configured[64] = {false};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
@@ -294,8 +300,9 @@ cudaError_t launch_v(TileParams& prm, const Problem& pb, cudaStream_t st)
 template <int K>
 cudaError_t launch_t(TileParams& prm, const Problem& pb, cudaStream_t st)
 {
-    if ((pb.W & 3) == 0 && (reinterpret_cast<uintptr_t>(prm.coef) & 15) == 0) return launch_v<K, true>(prm, pb, st);
-    return launch_v<K, false>(prm, pb, st);
+    if ((pb.W & 3) == 0 && (reinterpret_cast<uintptr_t>(prm.coef) & 15) == 0)
+        return prm.gather ? launch_v<K, true, true>(prm, pb, st) : launch_v<K, true, false>(prm, pb, st);
+    return launch_v<K, false, true>(prm, pb, st);
 }
 
 // The kernel's expected time, us: a launch, the dictionary by atom, what an SM's tiles cost together and what each turn of the
