@@ -10,6 +10,7 @@
 #include "sr_common.cuh"
 #include "sr_regress_listed.cuh"
 #include "sr_regress_rows.cuh"
+#include "sr_regress_split.cuh"
 #include "sr_regress_subset.cuh"
 #include "sr_producer.cuh"
 #include "sr_regress_tc.cuh"
@@ -283,6 +284,7 @@ static int default_kernel(const RegressArgs& a, bool shaped = false)
 {
     const int forced = g_force_kernel.load(std::memory_order_relaxed);
     if (forced >= 0 && kernel_supported(forced, a)) return forced;
+    if (!shaped && regress_split_pays(a.mode, a.coef_dtype, a.pb)) return kKernelGeneral;
     if (kernel_supported(kKernelSubset, a)) return kKernelSubset;
     if (!shaped && a.mode == kModeCompact && a.coef_dtype == SR_F16 && compact_prefers_general(a.pb)) return kKernelGeneral;
     if (!shaped && a.mode == kModeIdx && idx_prefers_general(a.pb)) return kKernelGeneral;

@@ -1,12 +1,14 @@
 // General regression kernel on the fp32 FMA pipe: every shape, fp32 or binary16 coefficients, all modes.
 // It is the path for small and narrow frames and the fallback for shapes and alignments the others do not take; dense and
-// global-subset frames large enough go to the register-tiled kernel (fp32) or the row kernel (binary16; launch_regress_fma).
+// global-subset frames large enough go to the register-tiled kernel (fp32) or the row kernel (binary16), those that one block per
+// multiprocessor covers to the split kernel (launch_regress_fma).
 //
 // One thread per HR pixel, 32 x 8 pixel tiles. Per pixel: assemble the filter F = Phi_i D in registers
 // (dictionary rows broadcast from shared memory), then y_c = F . B_c against an up-sampled tile with a
 // halo of p = (k-1)/2 that lives only in shared memory. Neither F nor the patch matrix B reaches HBM.
 #include "sr_pick.cuh"
 #include "sr_regress_rows.cuh"
+#include "sr_regress_split.cuh"
 #include "sr_regress_tile.cuh"
 #include <type_traits>
 
@@ -251,6 +253,7 @@ float regress_general_us(int mode, int coef_dtype, const Problem& pb)
 cudaError_t launch_regress_fma(int mode, const float* lr, const void* coef, int coef_dtype, const uint8_t* idx,
                                const float* gamma, const float* dict, float* out, const Problem& pb, cudaStream_t st)
 {
+    if (regress_split_pays(mode, coef_dtype, pb)) return launch_regress_split(mode, lr, coef, coef_dtype, idx, gamma, dict, out, pb, st);
     if (regress_tile_supported(mode, coef_dtype, pb)) return launch_regress_tile(mode, lr, coef, idx, gamma, dict, out, pb, st);
     if (regress_rows_form(mode, coef_dtype, pb) && regress_rows_pay(mode, pb)) return launch_regress_rows(mode, lr, coef, idx, gamma, dict, out, pb, st);
     if (coef_dtype == SR_F16) return launch_k<__half>(mode, lr, coef, idx, gamma, dict, out, pb, st);

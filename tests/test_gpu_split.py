@@ -1,0 +1,43 @@
+"""Frames that one block per multiprocessor covers: every pixel's atoms dealt over four threads (32 x 4 pixel tiles, eighty atoms
+in flight), against the oracle at the edges of tiles, batches of atoms and forms."""
+import numpy as np
+import pytest
+
+import oracle
+import paper_2303_08999_b200 as sr
+import sr_inputs
+from gpu_util import dev, host, max_abs_err, signed_asymmetric_dictionary, signed_gamma, tol_for
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dt", ["f16", "f32"])
+@pytest.mark.parametrize("n,c,h,w,r,D,k", [(1, 3, 2, 8, 4, 72, 5), (1, 3, 3, 11, 3, 12, 5), (2, 2, 5, 33, 1, 79, 3), (1, 4, 9, 16, 2, 80, 5), (1, 1, 4, 65, 1, 81, 7),
+                                           (3, 3, 1, 1, 1, 161, 3), (1, 3, 64, 64, 2, 72, 5), (1, 3, 17, 31, 4, 33, 9), (1, 4, 6, 5, 3, 256, 9), (2, 1, 7, 43, 3, 40, 7)])
+def test_dense(n, c, h, w, r, D, k, dt):
+    lr, d, coef = sr_inputs.make_inputs(sr_inputs.Workload("split", n, c, h, w, r, D=D, k=k, coef_dtype=dt))
+    d = signed_asymmetric_dictionary(d, seed=k)
+    args = (dev(lr), dev(coef), dev(d), r, k)
+    want = oracle.dict_regress_dense(lr, coef, d, r, k)
+    got = host(sr.sr_dict_regress_dense(*args))
+    scale = max(1.0, np.abs(want).max())                      # (fp32 sums: errors grow with what is summed)
+    assert max_abs_err(got, want) <= tol_for(coef) * scale
+    clamped = np.clip(got, 0, 1)
+    np.testing.assert_array_equal(host(sr.sr_dict_regress_dense(*args, sr.SR_CLAMP01)), clamped)
+    np.testing.assert_array_equal(host(sr.sr_dict_regress_dense(*args, sr.SR_CLAMP01 | sr.SR_OUT_F16)), clamped.astype(np.float16))
+    np.testing.assert_array_equal(host(sr.sr_dict_regress_dense(*args, sr.SR_OUT_U8)), np.rint(clamped * np.float32(255)).astype(np.uint8))
+
+
+@pytest.mark.parametrize("dt", ["f16", "f32"])
+@pytest.mark.parametrize("s,D,k,compact,gamma", [(12, 72, 5, False, True), (20, 96, 3, True, True), (81, 100, 5, False, False), (28, 28, 7, True, False)])
+def test_subset(s, D, k, compact, gamma, dt):
+    lr, d, coef = sr_inputs.make_inputs(sr_inputs.Workload("split", 2, 3, 9, 21, 3, D=D, k=k, coef_dtype=dt))
+    d = signed_asymmetric_dictionary(d, seed=k)
+    idx = np.random.default_rng(s).permutation(D)[:s].astype(np.uint8)
+    g = signed_gamma(s) if gamma else None
+    flags, given = sr.SR_IDX_GLOBAL, coef
+    if compact:
+        flags, given = flags | sr.SR_COEF_COMPACT, np.ascontiguousarray(coef[:, idx])
+    want = oracle.dict_regress_selected(lr, given, idx, g, d, 3, k, s, flags=flags)
+    got = host(sr.sr_dict_regress_selected(dev(lr), dev(given), dev(idx), None if g is None else dev(g), dev(d), 3, k, s, flags))
+    assert max_abs_err(got, want) <= tol_for(coef) * max(1.0, np.abs(want).max())
