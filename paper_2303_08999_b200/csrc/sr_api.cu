@@ -276,7 +276,8 @@ static bool kernel_supported(int kernel, const RegressArgs& a)
     }
 }
 
-// The host rules: small global subsets on the FMA-pipe subset kernel; per-pixel lists with their values on the gather
+// The host rules: dense calls and global subsets on frames that one block per multiprocessor covers to the split kernel (as a form
+// of the general one); other small global subsets on the FMA-pipe subset kernel; per-pixel lists with their values on the gather
 // kernel; the second tensor-core layout for the other
 // global subsets and for dense launches with few atoms; the first layout for the rest it supports; else the general kernel.
 // `shaped`: the layouts, subset and gather kernels before the general one, however small the frame.
@@ -303,7 +304,9 @@ static cudaError_t run_kernel(const TuneChoice& c, const RegressArgs& a)
     case kKernelListed: return launch_regress_listed(a.lr, a.coef, a.idx, a.dict, a.out, a.pb, a.st, c.sub_th);
     case kKernelSecondLayout: return launch_regress_tc(a.mode, a.lr, a.coef, a.idx, a.gamma, a.dict, a.out, a.pb, a.st, c.tc);
     case kKernelFirstLayout: return launch_regress_umma(a.mode, a.lr, a.coef, a.idx, a.gamma, a.dict, a.out, a.pb, a.st);
-    default: return launch_regress_fma(a.mode, a.lr, a.coef, a.coef_dtype, a.idx, a.gamma, a.dict, a.out, a.pb, a.st);
+    default:
+        return launch_regress_fma(a.mode, a.lr, a.coef, a.coef_dtype, a.idx, a.gamma, a.dict, a.out, a.pb, a.st,
+                                  g_force_kernel.load(std::memory_order_relaxed) != kKernelGeneral);
     }
 }
 

@@ -57,10 +57,10 @@ void count_launches(int n);
 // Issue-rate probe (sr_probe.cu): kind 0 integer max/min, 1 fp32 multiply-add; lane operations per second.
 cudaError_t probe_rate(int kind, int* scratch2, double* lane_ops_per_s, cudaStream_t st);
 
-// Launchers. Each returns a cudaError_t from the launch.
+// Launchers. Each returns a cudaError_t from the launch. `split`: whether small frames may go to the split kernel.
 cudaError_t launch_bicubic(const float* lr, float* hr, const Problem& pb, cudaStream_t st);
 cudaError_t launch_regress_fma(int mode, const float* lr, const void* coef, int coef_dtype, const uint8_t* idx,
-                               const float* gamma, const float* dict, float* out, const Problem& pb, cudaStream_t st);
+                               const float* gamma, const float* dict, float* out, const Problem& pb, cudaStream_t st, bool split = true);
 // Its thread-per-pixel kernel's expected time on a dense or global-subset launch, us.
 float regress_general_us(int mode, int coef_dtype, const Problem& pb);
 cudaError_t launch_select(const void* coef, int coef_dtype, uint8_t* idx, void* sel, const Problem& pb, cudaStream_t st);

@@ -2,6 +2,7 @@
 in flight), against the oracle at the edges of tiles, batches of atoms and forms."""
 import numpy as np
 import pytest
+import torch
 
 import oracle
 import paper_2303_08999_b200 as sr
@@ -41,3 +42,20 @@ def test_subset(s, D, k, compact, gamma, dt):
     want = oracle.dict_regress_selected(lr, given, idx, g, d, 3, k, s, flags=flags)
     got = host(sr.sr_dict_regress_selected(dev(lr), dev(given), dev(idx), None if g is None else dev(g), dev(d), 3, k, s, flags))
     assert max_abs_err(got, want) <= tol_for(coef) * max(1.0, np.abs(want).max())
+
+
+@pytest.mark.parametrize("dt", ["f16", "f32"])
+def test_forced_general_kernel_is_the_thread_per_pixel_kernel(dt):
+    # 5 blocks of 32 x 4 a frame: 30 frames are more than one block per multiprocessor takes, and too few for the row and the tiled kernel.
+    # A pixel's sum is the same bits in either call; the split kernel's four parts have another order
+    lr, d, coef = sr_inputs.make_inputs(sr_inputs.Workload("split", 1, 3, 9, 9, 2, D=40, k=3, coef_dtype=dt))
+    dlr, dco, ddi = dev(lr), dev(coef), dev(signed_asymmetric_dictionary(d, seed=3))
+    by_rule = sr.sr_dict_regress_dense(dlr, dco, ddi, 2, 3)
+    batch = sr.sr_dict_regress_dense(dlr.repeat(30, 1, 1, 1), dco.repeat(30, 1, 1, 1), ddi, 2, 3)
+    sr.sr_test_force_kernel(0)
+    try:
+        forced = sr.sr_dict_regress_dense(dlr, dco, ddi, 2, 3)
+    finally:
+        sr.sr_test_force_kernel(-1)
+    assert torch.equal(forced[0], batch[0]) and torch.equal(forced[0], batch[29])
+    assert not torch.equal(forced, by_rule)
