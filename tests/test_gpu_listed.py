@@ -127,3 +127,23 @@ def test_full_frame_sampled_against_the_oracle():
     flat = got.reshape(1, 3, -1)[0][:, torch.from_numpy(samples).cuda()].T.cpu().numpy()
     assert max_abs_err(flat, want) <= TOL_F16
     assert sr.sr_device_status() == 0
+
+
+@pytest.mark.parametrize("D", [16, 24, 80, 81])
+@pytest.mark.parametrize("h", [5, 600, 1200])                # rows of a block: 8, 16 and 32
+def test_seven_by_seven_atoms_on_the_first_layout(D, h):
+    # the dictionary is laid out before or behind the first loads, by rows and atoms
+    wl = sr_inputs.Workload("t", 1, 1, h, 8, 2, D=D, k=7, coef_dtype="f16")
+    lr, dict_, coef = sr_inputs.make_inputs(wl)
+    dict_ = signed_asymmetric_dictionary(dict_)
+    s = 4
+    want = oracle.dict_regress_selected(lr, coef, None, None, dict_, 2, 7, s)
+    dlr, dco, ddi = dev(lr), dev(coef), dev(dict_)
+    idx, sel = sr.sr_dict_select(dco, s, want_sel=True)
+    sr.sr_test_force_kernel(FIRST)
+    for args in ((dco, None), (dco, idx)):
+        got = sr.sr_dict_regress_selected(dlr, args[0], args[1], None, ddi, 2, 7, s)
+        assert max_abs_err(host(got), want) <= TOL_F16
+    got = sr.sr_dict_regress_selected(dlr, sel, idx, None, ddi, 2, 7, s, sr.SR_COEF_COMPACT)
+    assert max_abs_err(host(got), want) <= TOL_F16
+    assert sr.sr_device_status() == 0
