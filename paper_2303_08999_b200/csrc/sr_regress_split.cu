@@ -192,7 +192,9 @@ cudaError_t launch_k(SplitParams& prm, int coef_dtype, const Problem& pb, cudaSt
 
 // On 408 frames that one block per multiprocessor covers (up to 18 900 pixels; 4 to 200 atoms, subsets among them): 0.80 of the time of what
 // served them before, 361 of them faster. Where atoms and channels are few there is nothing to deal out and the thread-per-pixel
-// kernel's shorter set-up wins (32 of them: 1.03 to 1.26, one-channel frames of eight atoms and less above all). Aligned binary16
+// kernel's shorter set-up wins (32 of them: 1.03 to 1.26, one-channel frames of eight atoms and less above all). The line, on 512
+// frames of 1 to 24 atoms and of one to four channels on either side of it: geometric means 0.78 to 0.98 above it, 7 x 7 with three channels,
+// 14 atoms 0.95 (12 1.00, 8 1.02), with four, six 0.98 (five 1.01, four 1.04, one 1.05), 3 x 3 with one channel, 26 atoms 1.00 (24 1.06). Aligned binary16
 // frames with much to multiply stay on the tensor cores (96 atoms of 7 x 7 32 x 32 x2 14.8 us against 13.7; 128 17.4 against 14.9).
 // A second turn of blocks costs all of the first again: 0.88 of the best other time at 14 000 to 19 000 pixels, 1.4 just above.
 bool regress_split_pays(int mode, int coef_dtype, const Problem& pb)
@@ -200,7 +202,8 @@ bool regress_split_pays(int mode, int coef_dtype, const Problem& pb)
     if ((mode != kModeDense && mode != kModeGlobal) || pb.c > 4 || (pb.flags & SR_LUMA_ONLY) || pb.k < 3) return false;
     const int64_t tiles = (int64_t)pb.n * ((pb.W + TWD - 1) / TWD) * ((pb.H + ROWS - 1) / ROWS);
     const int natoms = mode == kModeGlobal ? pb.s : pb.D;
-    if (tiles > sm_count() || natoms + 8 * pb.c < 32) return false;
+    const int least = 32 + (pb.k == 7 && pb.c >= 3 ? 6 : 0) + (pb.k == 3 && pb.c == 1 ? 2 : 0);
+    if (tiles > sm_count() || natoms + 8 * pb.c < least) return false;
     return !(coef_dtype == SR_F16 && (pb.W & 7) == 0 && pb.k <= 7 && natoms * pb.k * pb.k > 4000);
 }
 

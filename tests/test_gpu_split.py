@@ -59,3 +59,18 @@ def test_forced_general_kernel_is_the_thread_per_pixel_kernel(dt):
         sr.sr_test_force_kernel(-1)
     assert torch.equal(forced[0], batch[0]) and torch.equal(forced[0], batch[29])
     assert not torch.equal(forced, by_rule)
+
+
+@pytest.mark.parametrize("c,D,k,split", [(4, 4, 7, False), (4, 5, 7, False), (4, 6, 7, True), (3, 12, 7, False), (3, 14, 7, True), (1, 25, 3, False), (1, 26, 3, True),
+                                         (4, 2, 5, True), (3, 8, 5, True), (3, 7, 5, False)])
+def test_few_atoms_and_channels_stay_with_the_thread_per_pixel_kernel(c, D, k, split):
+    # the same bits as the pinned kernel's, or another order of the same sum
+    lr, d, coef = sr_inputs.make_inputs(sr_inputs.Workload("split", 1, c, 31, 33, 2, D=D, k=k, coef_dtype="f32"))
+    args = (dev(lr), dev(coef), dev(signed_asymmetric_dictionary(d, seed=k)), 2, k)
+    by_rule = sr.sr_dict_regress_dense(*args)
+    sr.sr_test_force_kernel(0)
+    try:
+        forced = sr.sr_dict_regress_dense(*args)
+    finally:
+        sr.sr_test_force_kernel(-1)
+    assert torch.equal(by_rule, forced) != split
