@@ -11,9 +11,9 @@
 // per pixel and atom and is held by the shared-memory pipe at a quarter of that rate. 180 x 320 x3, D = 72, k = 5:
 // 118 -> 69 us (27 at the FMA pipe's rate); 540 x 960 x4: 1885 -> 784 us. Where the rest goes: up-sampling, set-up and
 // filtering are a third of the instructions, and 12 warps per SM (168 registers) do not hide every load.
-// With aligned rows a lane copies the sixteen bytes it reads itself, from a running address: no warp barrier and no table of
-// planes in the loop over the atoms (540 x 960 x2, D = 72: 209.4 -> 203.5 us; 3 x 3 270 x 480 x4: 118.3 -> 111; 7 x 7, D = 128,
-// 180 x 320 x3: 205 -> 197; the first shape 64.0 -> 63.4).
+// With aligned rows a lane copies the sixteen bytes it reads itself, from a running address where the planes follow one another: no
+// warp barrier, and no table of planes to make and wait for before the first copy (180 x 320 x3, D = 72: 5 x 5 63.9 -> 62.0 us, 3 x 3
+// 37.4 -> 34.5, 7 x 7 124.5 -> 116.3; with the table still made 63.1, 35.6 and 119.4, and 9 x 9 with few atoms slower than before).
 // Measured on the first shape and dropped: coefficients prefetched into registers (PF atoms ahead share the warp's few
 // load scoreboards: 78-124 us); tiles of 32 columns x 4 rows per thread (DRAM rows of 128 bytes, 83 us); 16 warps per SM
 // (spills, 128 us); scalar multiply-adds (84 us); the taps of 5 x 5 over two or three warps (77-115 us).
@@ -90,12 +90,14 @@ __global__ void __launch_bounds__(32 * NS * GPC, CTAS) regress_tile_kernel(const
     LrWindow w;
     decode_tile(g, blockIdx.x, w.f, w.y0, w.x0, w.rows);
     lr_window_of_tile<P>(g, w);
-    for (int l = tid; l < natoms; l += NT) {
-        const int plane = p.gather ? min((int)__ldg(p.idx + l), pb.D - 1) : l;
-        sOff[l] = ((int64_t)w.f * p.planes + plane) * HW;
+    if constexpr (GATHER) {
+        for (int l = tid; l < natoms; l += NT) {
+            const int plane = p.gather ? min((int)__ldg(p.idx + l), pb.D - 1) : l;
+            sOff[l] = ((int64_t)w.f * p.planes + plane) * HW;
+        }
     }
     for (int i = tid; i < (p.off_red - p.off_v) / 4; i += NT) reinterpret_cast<float4*>(sV)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    __syncthreads();
+    if constexpr (GATHER) __syncthreads();
     // this lane's copies of atom l's piece of the row into slot l mod DEPTH; every call commits one group
     const int row = min(w.y0 + grp, H - 1), x = w.x0 + PX * lane;
     const float* row0 = p.coef + (int64_t)row * W + w.x0;
