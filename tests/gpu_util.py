@@ -1,6 +1,10 @@
-"""Helpers for the GPU parity tests: device copies and error reporting."""
+"""Helpers for the GPU parity tests: device copies, error reporting, calls pinned to a kernel."""
+from contextlib import contextmanager
+
 import numpy as np
 import torch
+
+import paper_2303_08999_b200 as sr
 
 TOL_F32 = 1e-5   # max abs error with fp32 coefficients (images in [0,1], fp32 accumulation)
 TOL_F16 = 2e-3   # max abs error with binary16 coefficients
@@ -12,6 +16,17 @@ def dev(a: np.ndarray) -> torch.Tensor:
 
 def host(t: torch.Tensor) -> np.ndarray:
     return t.detach().cpu().numpy()
+
+
+@contextmanager
+def on_kernel(kernel: int):
+    """Regression calls inside run on `kernel` where it takes them: -1 = the host rules, 0 general (thread per pixel on small
+    frames), 1 and 2 the tensor-core layouts, 3 subset, 4 gather."""
+    sr.sr_test_force_kernel(kernel)
+    try:
+        yield
+    finally:
+        sr.sr_test_force_kernel(-1)
 
 
 def tol_for(coef: np.ndarray) -> float:

@@ -1,6 +1,6 @@
 """Bilinear variant of stage 1 (`sr_bilinear_upsample`, `SR_UPSAMPLE_BILINEAR`): every entry point and mode against
-the oracle, element by element, on shapes that reach the tensor-core kernels (both tile heights), the general FMA
-kernel and the stand-alone block / direct up-sampling kernels; plus the 1080p x4 frame on sampled pixels.
+the oracle, element by element, on shapes that the tensor-core kernels take (by the host rules and pinned to each layout and the
+general kernel), others, and those of the stand-alone block / direct up-sampling kernels; plus the 1080p x4 frame on sampled pixels.
 """
 import numpy as np
 import pytest
@@ -8,7 +8,7 @@ import pytest
 import oracle
 import paper_2303_08999_b200 as sr
 import sr_inputs
-from gpu_util import TOL_F16, TOL_F32, dev, host
+from gpu_util import TOL_F16, TOL_F32, dev, host, on_kernel
 
 pytestmark = pytest.mark.gpu
 
@@ -39,7 +39,13 @@ CASES = [
 
 @pytest.mark.parametrize("case", CASES, ids=[c[0] for c in CASES])
 @pytest.mark.parametrize("clamp", [0, sr.SR_CLAMP01])
-def test_all_modes(case, clamp):
+@pytest.mark.parametrize("kernel", [-1, 0, 1, 2])
+def test_all_modes(case, clamp, kernel):
+    with on_kernel(kernel):
+        _all_modes(case, clamp)
+
+
+def _all_modes(case, clamp):
     name, n, c, h, w, r, D, k, dt, s = case
     wl = sr_inputs.Workload(name, n, c, h, w, r, D, k, dt, s)
     lr, dict_, coef = sr_inputs.make_inputs(wl, seed=77)

@@ -1,6 +1,7 @@
 """SR_LUMA_ONLY: the per-pixel filter acts on the BT.601 luma of the up-sampled image, the chroma differences keep
 their up-sampled values. Every mode against the oracle, with each output type, on shapes that the other kernels would
-otherwise take (the flag has to route them to the general kernel) and with both stage-1 interpolations.
+otherwise take and with both stage-1 interpolations: fp32 output is composed of a one-channel regression, by the host rules and pinned
+to each kernel, and the chroma; the other output types go to the general kernel.
 """
 import numpy as np
 import pytest
@@ -9,7 +10,7 @@ import torch
 import oracle
 import paper_2303_08999_b200 as sr
 import sr_inputs
-from gpu_util import TOL_F16, TOL_F32, dev, host, signed_asymmetric_dictionary, signed_gamma
+from gpu_util import TOL_F16, TOL_F32, dev, host, on_kernel, signed_asymmetric_dictionary, signed_gamma
 
 pytestmark = pytest.mark.gpu
 
@@ -24,7 +25,13 @@ CASES = [
 
 
 @pytest.mark.parametrize("case", CASES, ids=[c[0] for c in CASES])
-def test_every_mode_matches_the_oracle(case):
+@pytest.mark.parametrize("kernel", [-1, 0, 1, 2, 3])
+def test_every_mode_matches_the_oracle(case, kernel):
+    with on_kernel(kernel):
+        _every_mode(case)
+
+
+def _every_mode(case):
     name, n, h, w, r, D, k, dt, s = case
     wl = sr_inputs.Workload(name, n, 3, h, w, r, D, k, dt, s)
     lr, dict_, coef = sr_inputs.make_inputs(wl, seed=5)

@@ -1,5 +1,5 @@
 """SR_OUT_F16: the regression calls store their fp32 result rounded to binary16.  Every mode against the oracle on
-shapes that reach the tensor-core kernels and the general kernel; the bound is the path's own tolerance plus half a
+shapes that the tensor-core kernels take, by the host rules and pinned to each of the layouts and the general kernel; the bound is the path's own tolerance plus half a
 binary16 unit in the last place of the exact value, and the stored values equal the fp32 output rounded to nearest.
 """
 import numpy as np
@@ -9,7 +9,7 @@ import torch
 import oracle
 import paper_2303_08999_b200 as sr
 import sr_inputs
-from gpu_util import TOL_F16, TOL_F32, dev, host
+from gpu_util import TOL_F16, TOL_F32, dev, host, on_kernel
 
 pytestmark = pytest.mark.gpu
 
@@ -31,7 +31,13 @@ def _check(got16, want, tol):
 
 
 @pytest.mark.parametrize("case", CASES, ids=[c[0] for c in CASES])
-def test_all_modes_store_binary16(case):
+@pytest.mark.parametrize("kernel", [-1, 0, 1, 2])
+def test_all_modes_store_binary16(case, kernel):
+    with on_kernel(kernel):
+        _all_modes(case)
+
+
+def _all_modes(case):
     name, n, c, h, w, r, D, k, dt, s = case
     wl = sr_inputs.Workload(name, n, c, h, w, r, D, k, dt, s)
     lr, dict_, coef = sr_inputs.make_inputs(wl, seed=91)

@@ -2,8 +2,9 @@
 
 The rounding decision is taken in the kernel's precision (fp32), so the codes must be bit-equal to the same call's fp32
 output quantised the same way; against the fp64 oracle's codes they may differ by one where the fp32 value sits within
-the path's tolerance of a rounding boundary, and nowhere else. Every mode, on shapes that reach each kernel (both
-tensor-core layouts, the FMA-pipe subset kernel, the general kernel).
+the path's tolerance of a rounding boundary, and nowhere else. Every mode, by the host rules (which give dense calls and global
+subsets on frames as small as these to the split kernel, lists to the general and the gather kernel) and pinned to the general
+kernel and to either tensor-core layout where it takes the call.
 """
 import numpy as np
 import pytest
@@ -12,15 +13,15 @@ import torch
 import oracle
 import paper_2303_08999_b200 as sr
 import sr_inputs
-from gpu_util import TOL_F16, TOL_F32, dev, host
+from gpu_util import TOL_F16, TOL_F32, dev, host, on_kernel
 
 pytestmark = pytest.mark.gpu
 
 U8 = sr.SR_OUT_U8
 CASES = [
-    ("first_layout", 1, 3, 24, 40, 4, 72, 5, "f16", 8),
-    ("second_layout_few_atoms", 2, 3, 30, 32, 2, 16, 3, "f16", 12),
-    ("second_layout_k7", 1, 3, 16, 48, 3, 24, 7, "f16", 12),
+    ("first_layout_shape", 1, 3, 24, 40, 4, 72, 5, "f16", 8),
+    ("second_layout_shape_few_atoms", 2, 3, 30, 32, 2, 16, 3, "f16", 12),
+    ("second_layout_shape_k7", 1, 3, 16, 48, 3, 24, 7, "f16", 12),
     ("short_last_tile", 1, 3, 13, 32, 3, 16, 5, "f16", 4),
     ("general_f32", 1, 3, 17, 19, 2, 16, 5, "f32", 4),
     ("one_channel", 1, 1, 20, 32, 2, 40, 5, "f16", 8),
@@ -42,7 +43,8 @@ def _check_against_oracle(codes: np.ndarray, want_value: np.ndarray, want_codes:
 
 
 @pytest.mark.parametrize("case", CASES, ids=[c[0] for c in CASES])
-def test_all_modes_store_eight_bit_codes(case):
+@pytest.mark.parametrize("kernel", [-1, 0, 1, 2])
+def test_all_modes_store_eight_bit_codes(case, kernel):
     name, n, c, h, w, r, D, k, dt, s = case
     wl = sr_inputs.Workload(name, n, c, h, w, r, D, k, dt, s)
     lr, dict_, coef = sr_inputs.make_inputs(wl, seed=77)
@@ -64,10 +66,11 @@ def test_all_modes_store_eight_bit_codes(case):
                    lambda fl: oracle.dict_regress_selected(lr, coef, S, gamma, dict_, r, k, S.size, flags=fl | oracle.IDX_GLOBAL)),
     }
     for mode, (gpu, ref) in calls.items():
-        codes = gpu(U8)
-        assert codes.dtype == torch.uint8, mode
-        assert torch.equal(codes, _quantise_f32(gpu(0))), mode              # same fp32 value, same rounding rule
-        assert torch.equal(codes, gpu(U8 | sr.SR_CLAMP01)), mode            # the clamp is implied
+        with on_kernel(kernel):
+            codes = gpu(U8)
+            assert codes.dtype == torch.uint8, mode
+            assert torch.equal(codes, _quantise_f32(gpu(0))), mode              # same fp32 value, same rounding rule
+            assert torch.equal(codes, gpu(U8 | sr.SR_CLAMP01)), mode            # the clamp is implied
         _check_against_oracle(host(codes), ref(0), ref(oracle.OUT_U8), tol)
     assert sr.sr_device_status() == 0
 

@@ -11,7 +11,7 @@ import torch
 import oracle
 import paper_2303_08999_b200 as sr
 import sr_inputs
-from gpu_util import TOL_F16, TOL_F32, dev, host, max_abs_err, signed_asymmetric_dictionary, signed_gamma, tol_for
+from gpu_util import TOL_F16, TOL_F32, dev, host, max_abs_err, on_kernel, signed_asymmetric_dictionary, signed_gamma, tol_for
 
 pytestmark = pytest.mark.gpu
 
@@ -58,15 +58,22 @@ DENSE_CASES = [
 ]
 
 
+# The host rules (-1) give most of these frames to the split kernel; the kernels they were written for, the general one, both
+# layouts and the subset and gather kernels, stay tested by pinning each in turn (where it does not take a call, the rules do).
+ON_KERNELS = pytest.mark.parametrize("kernel", [-1, 0, 1, 2, 3, 4])
+
+
 @pytest.mark.parametrize("case", DENSE_CASES, ids=lambda c: "-".join(map(str, c)))
 @pytest.mark.parametrize("clamp", [0, 1])
-def test_dense(case, clamp):
+@pytest.mark.parametrize("kernel", [-1, 0, 1, 2])
+def test_dense(case, clamp, kernel):
     n, c, h, w, r, D, k, dt = case
     lr, dict_, coef = sr_inputs.make_inputs(_wl(n, c, h, w, r, D, k, dt))
     if k == 1:  # a difference of Gaussians has no 1x1 form (0/0): use plain seeded weights instead
         dict_ = np.random.default_rng(1).uniform(-1, 1, dict_.shape).astype(np.float32)
     flags = sr.SR_CLAMP01 if clamp else 0
-    got = host(sr.sr_dict_regress_dense(dev(lr), dev(coef), dev(dict_), r, k, flags))
+    with on_kernel(kernel):
+        got = host(sr.sr_dict_regress_dense(dev(lr), dev(coef), dev(dict_), r, k, flags))
     want = oracle.dict_regress_dense(lr, coef, dict_, r, k, flags=flags)
     assert sr.sr_device_status() == 0
     assert max_abs_err(got, want) <= tol_for(coef)
@@ -76,7 +83,7 @@ def test_dense(case, clamp):
 @pytest.mark.parametrize("case", [(1, 3, 24, 40, 2, 16, 3), (2, 1, 33, 48, 2, 8, 5), (1, 2, 20, 72, 3, 17, 5), (1, 3, 24, 40, 2, 32, 7), (1, 3, 20, 32, 1, 16, 1),
                                   (2, 3, 9, 34, 4, 1, 5), (1, 1, 40, 56, 1, 33, 3), (1, 2, 17, 40, 4, 24, 7)], ids=lambda c: "-".join(map(str, c)))
 def test_both_layouts_on_small_frames_of_few_atoms(kernel, case):
-    # the host rules give such frames to the general kernel; what the layouts do with them stays tested
+    # the host rules give such frames to the split and the general kernel; what the layouts do with them stays tested
     n, c, h, w, r, D, k = case
     lr, d, coef = sr_inputs.make_inputs(_wl(n, c, h, w, r, D, k, "f16"))
     d = signed_asymmetric_dictionary(d, seed=k) if k > 1 else np.random.default_rng(1).uniform(-1, 1, d.shape).astype(np.float32)
@@ -229,7 +236,13 @@ SEL_CASES = [
 
 
 @pytest.mark.parametrize("case", SEL_CASES, ids=lambda c: "-".join(map(str, c)))
-def test_selected_all_modes(case):
+@ON_KERNELS
+def test_selected_all_modes(case, kernel):
+    with on_kernel(kernel):
+        _selected_all_modes(case)
+
+
+def _selected_all_modes(case):
     n, c, h, w, r, D, k, dt, s = case
     wl = _wl(n, c, h, w, r, D, k, dt)
     lr, dict_, coef = sr_inputs.make_inputs(wl)
@@ -308,19 +321,25 @@ def test_layout_rules_of_small_and_middling_frames(n, h, w, r, D, k, s):
 
 SIGNED_CASES = [
     # n, c, h, w, r, D, k, dtype, s
-    (1, 3, 24, 64, 2, 72, 5, "f16", 8),    # every mode on the tensor-core kernel
+    (1, 3, 24, 64, 2, 72, 5, "f16", 8),    # the tensor-core kernel takes every mode
     (2, 3, 33, 50, 4, 72, 5, "f16", 8),    # HR width 200: dense / in-kernel selection / subset on the tensor cores, index planes on the general kernel
-    (1, 3, 20, 30, 2, 72, 5, "f32", 8),    # fp32 coefficients: general kernel
+    (1, 3, 20, 30, 2, 72, 5, "f32", 8),    # fp32 coefficients: general and split kernel
     (1, 3, 12, 40, 2, 32, 7, "f16", 4),
     (1, 3, 12, 32, 2, 72, 3, "f16", 12),
     (1, 1, 9, 16, 2, 7, 9, "f32", 3),      # 9 x 9 atoms: general kernel
-    (1, 3, 30, 35, 4, 72, 5, "f16", 8),    # HR width 140: general kernel with binary16 coefficients
+    (1, 3, 30, 35, 4, 72, 5, "f16", 8),    # HR width 140: general and split kernel with binary16 coefficients
     (1, 3, 40, 64, 4, 72, 5, "f16", 8),    # several 16-row tiles, two tile columns
 ]
 
 
 @pytest.mark.parametrize("case", SIGNED_CASES, ids=lambda c: "-".join(map(str, c)))
-def test_signed_asymmetric_dictionary_and_negative_gamma_all_modes(case):
+@ON_KERNELS
+def test_signed_asymmetric_dictionary_and_negative_gamma_all_modes(case, kernel):
+    with on_kernel(kernel):
+        _signed_all_modes(case)
+
+
+def _signed_all_modes(case):
     """Atoms without any symmetry and with both signs, re-weights with both signs: a 180-degree tap flip, a transposed
     patch or a lost sign in the binary16 hi / lo split of the dictionary fails here (it passes with the generator's
     point-symmetric, non-negative atoms)."""
@@ -357,7 +376,13 @@ def test_signed_asymmetric_dictionary_and_negative_gamma_all_modes(case):
 
 @pytest.mark.parametrize("dt,w", [("f16", 48), ("f32", 48), ("f16", 35)])
 @pytest.mark.parametrize("tap", [(0, 1), (4, 0), (3, 4), (2, 2)])
-def test_off_centre_delta_atom_shifts_the_upsampled_image(dt, w, tap):
+@ON_KERNELS
+def test_off_centre_delta_atom_shifts_the_upsampled_image(dt, w, tap, kernel):
+    with on_kernel(kernel):
+        _off_centre_delta(dt, w, tap)
+
+
+def _off_centre_delta(dt, w, tap):
     """One atom that is a single tap at (a, b), one-hot coefficients: the output is the up-sampled image read at
     (Y + a - p, X + b - p), clamped to the frame. The expected frame is built from the bicubic oracle by indexing
     alone, so the pairing of taps and patch positions is checked without the oracle's own regression."""
@@ -384,7 +409,13 @@ def test_off_centre_delta_atom_shifts_the_upsampled_image(dt, w, tap):
 
 
 @pytest.mark.parametrize("scale,bound", [(2.0 ** 15, TOL_F16 * 2.0 ** 15), (2.0 ** -10, 1e-5)])
-def test_dictionary_magnitude_range_of_the_tensor_core_path(scale, bound):
+@pytest.mark.parametrize("kernel", [-1, 1, 2])
+def test_dictionary_magnitude_range_of_the_tensor_core_path(scale, bound, kernel):
+    with on_kernel(kernel):
+        _dictionary_magnitude_range(scale, bound)
+
+
+def _dictionary_magnitude_range(scale, bound):
     """The tensor-core path keeps the fp32 dictionary as a binary16 hi + lo pair, so its taps must stay below the
     largest binary16 number (65504); taps below 2^-14 fall into the binary16 subnormals and keep an absolute, not a
     relative, precision (2^-25 per tap). A large dictionary (taps up to about 9500) must be as accurate relative to
@@ -403,8 +434,10 @@ def test_dictionary_magnitude_range_of_the_tensor_core_path(scale, bound):
 # ------------------------------------------------------------------ LR pixels that are not finite
 
 # kernel (sr_test_force_kernel; -1 = host rules), mode, n, c, h, w, scale, D, k, coefficients: the kernels that make their
-# up-sampled tiles separably, each with more tiles than thread blocks where its tiles follow one another in a block
+# up-sampled tiles separably, each with more tiles than thread blocks where its tiles follow one another in a block, and those on the smallest frames
 NON_FINITE_LR = [
+    (-1, "dense", 2, 3, 12, 70, 2, 32, 5, "f16"), (-1, "dense", 1, 4, 9, 50, 3, 12, 9, "f32"), (-1, "dense", 1, 1, 20, 131, 1, 40, 3, "f32"),      # the split kernel
+    (0, "dense", 2, 3, 12, 70, 2, 32, 5, "f16"),
     (1, "dense", 2, 3, 130, 320, 2, 32, 5, "f16"), (1, "dense", 2, 1, 400, 500, 1, 24, 3, "f16"), (1, "dense", 2, 1, 90, 136, 4, 72, 7, "f16"),
     (1, "fused", 2, 3, 130, 320, 2, 32, 5, "f16"), (1, "compact", 1, 3, 96, 160, 3, 32, 5, "f16"),
     (2, "dense", 2, 3, 130, 320, 2, 16, 5, "f16"), (4, "compact", 2, 3, 130, 320, 2, 32, 5, "f16"),
@@ -524,7 +557,13 @@ ROW_CASES = [  # k, n, c, h, w, scale, D: binary16 rows of any width; K-steps of
 
 @pytest.mark.parametrize("case", ROW_CASES, ids=lambda c: "-".join(map(str, c)))
 @pytest.mark.parametrize("magnitude", [1.0, 2.0 ** 20, 2.0 ** -30])
-def test_binary16_rows_of_any_width(case, magnitude):
+@pytest.mark.parametrize("kernel", [-1, 0])                  # the smaller ones: the split kernel, the thread-per-pixel kernel
+def test_binary16_rows_of_any_width(case, magnitude, kernel):
+    with on_kernel(kernel):
+        _binary16_rows_of_any_width(case, magnitude)
+
+
+def _binary16_rows_of_any_width(case, magnitude):
     k, n, c, h, w, r, D = case
     wl = sr_inputs.Workload("rows", n, c, h, w, r, D=D, k=k)
     lr, d, coef = sr_inputs.make_inputs(wl)
@@ -626,7 +665,13 @@ def test_row_kernel_at_the_ends_of_the_dictionary_range(magnitude):
     assert np.abs(got - want).max() <= TOL_F32
 
 
-def test_binary16_rows_keep_a_non_finite_coefficient_to_its_pixel():       # (a small frame: the general kernel)
+@pytest.mark.parametrize("kernel", [-1, 0])                  # a small frame: the split kernel, the thread-per-pixel kernel
+def test_binary16_rows_keep_a_non_finite_coefficient_to_its_pixel(kernel):
+    with on_kernel(kernel):
+        _keep_a_non_finite_coefficient()
+
+
+def _keep_a_non_finite_coefficient():
     wl = sr_inputs.Workload("rows", 1, 3, 20, 27, 3, D=20, k=5)
     lr, d, coef = sr_inputs.make_inputs(wl)
     clean = host(sr.sr_dict_regress_dense(dev(lr), dev(coef), dev(d), 3, 5))

@@ -74,3 +74,23 @@ def test_few_atoms_and_channels_stay_with_the_thread_per_pixel_kernel(c, D, k, s
     finally:
         sr.sr_test_force_kernel(-1)
     assert torch.equal(by_rule, forced) != split
+
+
+@pytest.mark.parametrize("dt", ["f16", "f32"])
+@pytest.mark.parametrize("k,D", [(3, 72), (5, 53), (9, 33)])
+def test_coefficients_that_are_not_finite(k, D, dt):
+    # in the first, the last and an inner atom: the same infinities and NaN as the sum has, in that pixel alone
+    lr, d, coef = sr_inputs.make_inputs(sr_inputs.Workload("split", 2, 3, 15, 33, 2, D=D, k=k, coef_dtype=dt))
+    d = signed_asymmetric_dictionary(d, seed=k)
+    d[D - 1] = np.abs(d[D - 1]) + 0.01                        # with finite taps of one sign: an infinity, not NaN
+    clean = host(sr.sr_dict_regress_dense(dev(lr), dev(coef), dev(d), 2, k))
+    bad, hit = coef.copy(), np.zeros(clean.shape, bool)
+    for j, (f, y, x) in enumerate([(0, 0, 0), (0, 3, 31), (0, 4, 32), (1, 29, 65), (1, 28, 63), (0, 29, 64), (1, 13, 7), (1, 0, 65)]):
+        bad[f, [D - 1, 0, D // 2][j % 3], y, x] = [np.inf, -np.inf, np.nan, np.inf][j % 4]
+        hit[f, :, y, x] = True
+    out = host(sr.sr_dict_regress_dense(dev(lr), dev(bad), dev(d), 2, k))
+    np.testing.assert_array_equal(out[~hit], clean[~hit])
+    want = oracle.dict_regress_dense(lr, bad, d, 2, k)[hit]
+    np.testing.assert_array_equal(np.isnan(out[hit]), np.isnan(want))
+    np.testing.assert_array_equal(out[hit][~np.isnan(want)], want[~np.isnan(want)].astype(np.float32))
+    assert np.isinf(want).any() and np.isnan(want).any()

@@ -12,7 +12,7 @@ import torch
 
 import paper_2303_08999_b200 as sr
 import sr_inputs
-from gpu_util import dev
+from gpu_util import dev, on_kernel
 
 pytestmark = pytest.mark.gpu
 
@@ -20,11 +20,8 @@ SHORT_BUDGET = 2_000_000   # SM cycles: about a millisecond
 
 
 def _on_kernel(kernel, fn):
-    sr.sr_test_force_kernel(kernel)
-    try:
+    with on_kernel(kernel):
         return fn()
-    finally:
-        sr.sr_test_force_kernel(-1)
 
 
 def _calls():
@@ -34,13 +31,14 @@ def _calls():
     idx, sel = sr.sr_dict_select(dco, 8, want_sel=True)
     S = dev(np.arange(0, 72, 6, dtype=np.uint8))          # twelve atoms: more than the FMA-pipe subset kernel (no waits) takes
     return {
-        "dense": lambda: sr.sr_dict_regress_dense(dlr, dco, ddi, 2, 5),
+        # pinned to the first layout, as the ones below: the host rules give frames as small as this to a kernel without waits, so
+        # that the calls before and after would not meet the tensor memory and barriers of the one that failed
+        "dense": lambda: _on_kernel(1, lambda: sr.sr_dict_regress_dense(dlr, dco, ddi, 2, 5)),
         "fused_select": lambda: sr.sr_dict_regress_selected(dlr, dco, None, None, ddi, 2, 5, 8),
         "index_planes": lambda: sr.sr_dict_regress_selected(dlr, dco, idx, None, ddi, 2, 5, 8),
         # pinned to the first tensor-core layout: the host rules give this shape to the gather kernel, which has no waits
         "compact": lambda: _on_kernel(1, lambda: sr.sr_dict_regress_selected(dlr, sel, idx, None, ddi, 2, 5, 8, sr.SR_COEF_COMPACT)),
-        # pinned to the second layout: the host rules give frames as small as this to the general kernel, which has no waits,
-        # so that the calls before and after would not meet the tensor memory and barriers of the one that failed
+        # pinned to the second layout
         "global_subset": lambda: _on_kernel(2, lambda: sr.sr_dict_regress_selected(dlr, dco, S, None, ddi, 2, 5, 12, sr.SR_IDX_GLOBAL)),
         "dense_few_atoms": lambda: _on_kernel(2, lambda: sr.sr_dict_regress_dense(dlr, dco[:, :16].contiguous(), ddi[:16].contiguous(), 2, 5)),
     }
