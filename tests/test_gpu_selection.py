@@ -145,7 +145,7 @@ def test_gram_adds_at_most_the_terms_of_32_pixels_in_fp32(D, n, h, w):
         assert np.abs(got - want).max() <= 16.5 * 2.0 ** -24 * want
 
 
-@pytest.mark.parametrize("D", [7, 8, 9, 31, 33, 64, 65, 97, 128])
+@pytest.mark.parametrize("D", [1, 7, 8, 9, 31, 33, 64, 65, 97, 128])
 @pytest.mark.parametrize("scale", [1.0, 2.0 ** -700, 2.0 ** 640])
 def test_search_bits_at_block_edges_and_extreme_scales(D, scale):
     # coordinate blocks of eight, residuals in registers of 32: both sides of their edges; statistics scaled by a power of
@@ -198,3 +198,21 @@ def test_search_where_a_quotient_lies_next_to_the_middle_of_two_numbers():
     idx, gamma, trace = sr.sr_selection_search(dev(G), dev(b), dev(np.array([hh])), 2, 0.5, 0.5, 0.0, 1.0, max_sweeps=50)
     np.testing.assert_array_equal(host(idx), want[0])
     np.testing.assert_array_equal(host(trace), want[2])
+
+
+@pytest.mark.parametrize("e", [1, 10, 20, 30, 40, 46, 50])
+def test_search_bits_where_residuals_lie_just_above_the_threshold(e):
+    # numerators of about 2^-e of the threshold: what the quick quotient rounds away grows with 2^e against the quotient
+    rng = np.random.default_rng(e)
+    D = 12
+    off = np.triu(rng.uniform(-0.02, 0.02, (D, D)), 1)
+    G = np.diag(rng.uniform(1, 2, D)) + off + off.T
+    b = np.full(D, 0.5)
+    b[::2] = 1 + rng.uniform(1, 2, D // 2) * 2.0 ** -e
+    args = (2.0, 0.5, 0.5, 0.0, 1.0)
+    want = oracle.selection_search(G, b, 0.0, *args, tol=1e-30, max_sweeps=200)
+    idx, gamma, trace = sr.sr_selection_search(dev(G), dev(b), dev(np.array([0.0])), *args, tol=1e-30, max_sweeps=200)
+    assert len(want[0]) == D // 2
+    np.testing.assert_array_equal(host(idx), want[0])
+    np.testing.assert_array_equal(host(trace), want[2])
+    np.testing.assert_array_equal(host(gamma), want[1].astype(np.float32))
