@@ -488,7 +488,8 @@ cudaError_t launch_gram_k(const GramParams& p, int T, int ctas, size_t smem, cud
 //
 // The bisection's solves all start from the same coefficients until one of them is kept. So each round solves the whole
 // tree of the next five mid points, one per warp of a cluster of eight blocks (a warp per scheduler: nobody slows the
-// chains down), and then walks it as the sequential program would. The blocks run everything else alike.
+// chains down), and then walks it as the sequential program would. The blocks run everything else alike. Where the context has no
+// room for a cluster of eight, fewer blocks walk shallower trees: the same solves one round later, the same bits.
 // 72 atoms down to 8 in four steps (about 90 solves, 90 000 steps, 33 000 of them in bisections): 8.7 -> 6.0 ms against one block
 // with eleven operations to a step, a bisection's solves one after the other (46 ms with one warp that divided inside the chain).
 // A round lasts as long as its slowest solve, which costs what a walk that ends early saves: 187 searches of 16 to 128 atoms, eps from
@@ -496,9 +497,7 @@ cudaError_t launch_gram_k(const GramParams& p, int T, int ctas, size_t smem, cud
 // Left are some 165 clocks a step: about 60 instructions of one warp, fp64 at two clocks each, around a chain of 75.
 constexpr int kSearchThreads = 128;
 constexpr int kSearchWarps = kSearchThreads / 32;
-constexpr int kSearchCtas = 8;                     // blocks of the cluster
-constexpr int kTreeLevels = 5;                     // 31 of the 32 warps have a node
-static_assert((1 << kTreeLevels) - 1 <= kSearchCtas * kSearchWarps, "a warp per node");
+constexpr int kSearchCtas = 8;                     // blocks of the cluster, at most: 31 of the 32 warps have a node of five levels
 constexpr int kCdBlock = 8;
 
 struct SearchParams {
@@ -809,14 +808,15 @@ __device__ bool refit_gamma(const SearchState& s, int ns)
     return true;
 }
 
-__global__ void __cluster_dims__(kSearchCtas, 1, 1) __launch_bounds__(kSearchThreads, 1)
+__global__ void __launch_bounds__(kSearchThreads, 1)
 selection_search_kernel(const __grid_constant__ SearchParams p)
 {
     extern __shared__ __align__(16) double ssm[];
     __shared__ int sCount[kSearchWarps], sAt[kSearchWarps];   // this block's nodes: coefficients that are not zero, and where they are
     __shared__ int sTree[kSearchCtas * kSearchWarps][2];      // the same of all blocks
     cg::cluster_group cluster = cg::this_cluster();
-    const int cta = (int)cluster.block_rank();
+    const int cta = (int)cluster.block_rank(), warps = (int)cluster.num_blocks() * kSearchWarps;
+    const int levels = 31 - __clz(warps);                     // of a round's tree: a warp per node
     SearchState s;
     const int L = p.L;
     s.L8 = search_l8(L); s.Lp = s.L8 + 1; s.tid = threadIdx.x; s.lane = threadIdx.x & 31; s.nrows = p.nrows;
@@ -880,7 +880,7 @@ selection_search_kernel(const __grid_constant__ SearchParams p)
             if (stale) residuals(s, s.best);
             stale = false;
             const int node = cta * kSearchWarps + (tid >> 5) + 1, level = 31 - __clz(node);
-            if (level < kTreeLevels && it + level < p.max_bisect) {
+            if (level < levels && it + level < p.max_bisect) {
                 double lo = left, hi = right, mid = __dmul_rn(0.5, __dadd_rn(lo, hi));
                 for (int u = level - 1; u >= 0; --u) {
                     if ((node >> u) & 1) lo = mid;
@@ -892,13 +892,13 @@ selection_search_kernel(const __grid_constant__ SearchParams p)
                 if (s.lane == 0) { sCount[tid >> 5] = count; sAt[tid >> 5] = (int)(now - s.solve); }
             }
             cluster.sync();
-            if (tid < kSearchCtas * kSearchWarps) {
+            if (tid < warps) {
                 sTree[tid][0] = cluster.map_shared_rank(sCount, tid / kSearchWarps)[tid % kSearchWarps];
                 sTree[tid][1] = cluster.map_shared_rank(sAt, tid / kSearchWarps)[tid % kSearchWarps];
             }
             __syncthreads();
             int at = 1;
-            while (at < (1 << kTreeLevels) && fabs(__dadd_rn(target, -(double)nnz)) > band && it < p.max_bisect) {
+            while (at < (1 << levels) && fabs(__dadd_rn(target, -(double)nnz)) > band && it < p.max_bisect) {
                 const double mid = __dmul_rn(0.5, __dadd_rn(left, right));
                 ++solves;
                 ++it;
@@ -1120,9 +1120,25 @@ cudaError_t launch_selection_search(const double* G, const double* b, const doub
         if (e != cudaSuccess) return e;
         configured[dev] = true;
     }
-    selection_search_kernel<<<kSearchCtas, kSearchThreads, bytes(L), st>>>(p);
-    count_launches(1);
-    return cudaGetLastError();
+    cudaLaunchAttribute shape{};
+    shape.id = cudaLaunchAttributeClusterDimension;
+    shape.val.clusterDim.y = shape.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.blockDim = dim3(kSearchThreads);
+    cfg.dynamicSmemBytes = bytes(L);
+    cfg.stream = st;
+    cfg.attrs = &shape;
+    cfg.numAttrs = 1;
+    for (int ctas = kSearchCtas;; ctas /= 2) {
+        shape.val.clusterDim.x = ctas;
+        cfg.gridDim = dim3(ctas);
+        int fit = 0;
+        if (ctas == 1 || (cudaOccupancyMaxActiveClusters(&fit, selection_search_kernel, &cfg) == cudaSuccess && fit > 0)) break;
+        (void)cudaGetLastError();                            // (a shape that cannot run leaves nothing behind)
+    }
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, selection_search_kernel, p);
+    if (e == cudaSuccess) count_launches(1);
+    return e;
 }
 
 } // namespace sr
