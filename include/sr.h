@@ -339,8 +339,8 @@ int sr_test_lose_arrival(int launches);
  * Test hook: regression calls that follow are run by kernel `kernel` (the numbering of sr_tune_result.kernel)
  * whenever that kernel supports the call, instead of the one the host rules or the tuning table pick; -1 restores
  * the rules.  Kernel 0 stands for its thread-per-pixel, row and register-tiled forms here; the form for dense calls and global
- * subsets on the smallest frames (one thread block per multiprocessor) is left to the rules.  Lets a test compare two kernels that serve the same call.  Returns SR_OK, or SR_ERR_SHAPE for a number
- * that names no kernel.  The paper has no counterpart.
+ * subsets on the smallest frames (one thread block per multiprocessor) is left to the rules.  Lets a test compare two kernels
+ * that serve the same call.  Returns SR_OK, or SR_ERR_SHAPE for a number that names no kernel.  The paper has no counterpart.
  */
 int sr_test_force_kernel(int kernel);
 

@@ -253,7 +253,8 @@ float regress_general_us(int mode, int coef_dtype, const Problem& pb)
 cudaError_t launch_regress_fma(int mode, const float* lr, const void* coef, int coef_dtype, const uint8_t* idx,
                                const float* gamma, const float* dict, float* out, const Problem& pb, cudaStream_t st, bool split)
 {
-    if (split && regress_split_pays(mode, coef_dtype, pb)) return launch_regress_split(mode, lr, coef, coef_dtype, idx, gamma, dict, out, pb, st);
+    if (split && regress_split_pays(mode, coef_dtype, pb))
+        return launch_regress_split(mode, lr, coef, coef_dtype, idx, gamma, dict, out, pb, st);
     if (regress_tile_supported(mode, coef_dtype, pb)) return launch_regress_tile(mode, lr, coef, idx, gamma, dict, out, pb, st);
     if (regress_rows_form(mode, coef_dtype, pb) && regress_rows_pay(mode, pb)) return launch_regress_rows(mode, lr, coef, idx, gamma, dict, out, pb, st);
     if (coef_dtype == SR_F16) return launch_k<__half>(mode, lr, coef, idx, gamma, dict, out, pb, st);

@@ -124,9 +124,9 @@ __global__ void __launch_bounds__(kThreads, 1) regress_listed_kernel(const __gri
         }
     }
 
-    // ---- set-up, behind the first tile's window and lists. A thread reads a unit of the dictionary once and writes its eight copies, every lane
-    // of a wavefront another one. A thread per copy read it eight times, before the window was asked for: 136 x 160 x4, s = 8, select and
-    // regress 42.2 -> 41.3 us, 270 x 480 x4 191.2 -> 189.3, 540 x 960 x4 702 -> 699.
+    // ---- set-up, behind the first tile's window and lists. A thread reads a unit of the dictionary once and writes its eight
+    // copies, every lane of a wavefront another one. A thread per copy read it eight times, before the window was asked for: 136 x
+    // 160 x4, s = 8, select and regress 42.2 -> 41.3 us, 270 x 480 x4 191.2 -> 189.3, 540 x 960 x4 702 -> 699.
     float v[4];
     auto read_unit = [&](int i) {
         const int a = i / NU, j = i - a * NU;

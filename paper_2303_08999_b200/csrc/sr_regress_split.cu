@@ -2,13 +2,13 @@
 //
 // A frame of some ten thousand pixels gives a thread per pixel a warp or two per scheduler, and each of them waits for one trip
 // to memory per dozen atoms, then for the dictionary, then for the LR image: the time is a sum of latencies. Here a pixel has NS threads,
-// one per warp of a row's group, with every NS-th atom each. A thread asks for its coefficients first (up to twenty, eighty atoms of a pixel),
-// then for its entries of the dictionary and the LR taps of its values of the up-sampled tile, and waits once for all of
-// them. Each warp applies its part of the filter to the patch, and the parts' sums meet in shared memory, a channel per warp.
-// One block of 32 x 4 pixels per SM. 64 x 64 x2, D = 72, 5 x 5, fp32: 13.0 -> 8.6 us of device time.
-// Bound: launch and one trip to memory (3.7 us), a channel's part of the tile and of the filtering (0.5 us), 0.045 us an atom of 5 x 5
-// (issue slots of sixteen warps). Tiles of 32 x 2 with 256 threads took 9.4 us there; the up-sampled tile in two passes through shared
-// memory, after its LR window, 8.8.
+// one per warp of a row's group, with every NS-th atom each. A thread asks for its coefficients first (up to twenty, eighty atoms
+// of a pixel), then for its entries of the dictionary and the LR taps of its values of the up-sampled tile, and waits once for all
+// of them. Each warp applies its part of the filter to the patch, and the parts' sums meet in shared memory, a channel per warp.
+// One block of 32 x 4 pixels per SM. 64 x 64 x2, D = 72, 5 x 5, fp32: 13.0 -> 8.6 us of device time. Bound: launch and one trip to
+// memory (3.7 us), a channel's part of the tile and of the filtering (0.5 us), 0.045 us an atom of 5 x 5 (issue slots of sixteen
+// warps). Tiles of 32 x 2 with 256 threads took 9.4 us there; the up-sampled tile in two passes through shared memory, after its LR
+// window, 8.8.
 
 #include "sr_regress_split.cuh"
 #include "sr_tile_upsample.cuh"
@@ -190,13 +190,14 @@ cudaError_t launch_k(SplitParams& prm, int coef_dtype, const Problem& pb, cudaSt
 
 } // namespace
 
-// On 408 frames that one block per multiprocessor covers (up to 18 900 pixels; 4 to 200 atoms, subsets among them): 0.80 of the time of what
-// served them before, 361 of them faster. Where atoms and channels are few there is nothing to deal out and the thread-per-pixel
-// kernel's shorter set-up wins (32 of them: 1.03 to 1.26, one-channel frames of eight atoms and less above all). The line, on 512
-// frames of 1 to 24 atoms and of one to four channels on either side of it: geometric means 0.78 to 0.98 above it, 7 x 7 with three channels,
-// 14 atoms 0.95 (12 1.00, 8 1.02), with four, six 0.98 (five 1.01, four 1.04, one 1.05), 3 x 3 with one channel, 26 atoms 1.00 (24 1.06). Aligned binary16
-// frames with much to multiply stay on the tensor cores (96 atoms of 7 x 7 32 x 32 x2 14.8 us against 13.7; 128 17.4 against 14.9).
-// A second turn of blocks costs all of the first again: 0.88 of the best other time at 14 000 to 19 000 pixels, 1.4 just above.
+// On 408 frames that one block per multiprocessor covers (up to 18 900 pixels; 4 to 200 atoms, subsets among them): 0.80 of the
+// time of what served them before, 361 of them faster. Where atoms and channels are few there is nothing to deal out and the
+// thread-per-pixel kernel's shorter set-up wins (32 of them: 1.03 to 1.26, one-channel frames of eight atoms and less above all).
+// The line, on 512 frames of 1 to 24 atoms and of one to four channels on either side of it: geometric means 0.78 to 0.98 above it,
+// 7 x 7 with three channels, 14 atoms 0.95 (12 1.00, 8 1.02), with four, six 0.98 (five 1.01, four 1.04, one 1.05), 3 x 3 with one
+// channel, 26 atoms 1.00 (24 1.06). Aligned binary16 frames with much to multiply stay on the tensor cores (96 atoms of 7 x 7 32 x
+// 32 x2 14.8 us against 13.7; 128 17.4 against 14.9). A second turn of blocks costs all of the first again: 0.88 of the best other
+// time at 14 000 to 19 000 pixels, 1.4 just above.
 bool regress_split_pays(int mode, int coef_dtype, const Problem& pb)
 {
     if ((mode != kModeDense && mode != kModeGlobal) || pb.c > 4 || (pb.flags & SR_LUMA_ONLY) || pb.k < 3) return false;

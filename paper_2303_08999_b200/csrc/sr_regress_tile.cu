@@ -61,8 +61,8 @@ constexpr int kStageBytes = 512;                         // a ring slot: 128 pix
 
 template <int K> __host__ __device__ constexpr int dict_pitch() { return (K * K / 4) * 4 + 4; }   // the 16-byte units, the last tap, zeros
 
-// K: atom side; NS: warps that share the taps; GPC: such groups (rows) per block; CTAS: blocks per SM; VEC: 16-byte copies; GATHER: planes by table (always
-// without VEC), else one after the other
+// K: atom side; NS: warps that share the taps; GPC: such groups (rows) per block; CTAS: blocks per SM; VEC: 16-byte copies; GATHER:
+// planes by table (always without VEC), else one after the other
 template <int K, int NS, int GPC, int CTAS, int DEPTH, bool VEC, bool GATHER>
 __global__ void __launch_bounds__(32 * NS * GPC, CTAS) regress_tile_kernel(const __grid_constant__ TileParams p)
 {
@@ -152,7 +152,8 @@ __global__ void __launch_bounds__(32 * NS * GPC, CTAS) regress_tile_kernel(const
 #pragma unroll 2
     for (int l = 0; l < natoms; ++l, dl += PITCH) {
         cp_wait<DEPTH - 2>();
-        if (!VEC) __syncwarp();                              // every lane's part of the piece has landed; the slot read last is free (VEC: a lane reads what it copied)
+        // every lane's part of the piece has landed; the slot read last is free (VEC: a lane reads what it copied itself)
+        if (!VEC) __syncwarp();
         const float4 v4 = *reinterpret_cast<const float4*>(ring + slot + 16 * lane);
         const float v[PX] = {v4.x, v4.y, v4.z, v4.w};
         fetch(l + DEPTH - 1, free_slot);

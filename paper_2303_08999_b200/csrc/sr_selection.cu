@@ -609,9 +609,9 @@ __device__ __forceinline__ double with_sign_of(double magnitude, double x)   // 
 // no later than num (from the two terms of num: they cancel where the residual barely exceeds the threshold, and t keeps their rounding).
 // That is the rounded quotient but where the quotient lies within about 2^-52 max(1, thr / |num|) units in the last place of the
 // middle of two numbers. So every q is checked, off the chain: with the remainder of q, q + remainder y rounds to the
-// rounded quotient if q is one of the quotient's two neighbours (Markstein, IBM J. Res. Dev. 34 (1990)), and it differs from q if q is further
-// off (or if anything over- or underflowed). A sweep with a q that fails is made again in the plain form, from the coefficients
-// and residuals it started with.
+// rounded quotient if q is one of the quotient's two neighbours (Markstein, IBM J. Res. Dev. 34 (1990)), and it differs from q if q
+// is further off (or if anything over- or underflowed). A sweep with a q that fails is made again in the plain form, from the
+// coefficients and residuals it started with.
 template <int NK, bool FROZEN>
 __device__ __noinline__ double* cd_sweeps(const SearchState& s, double thr, double* buf, double tol, int max_sweeps)
 {
@@ -625,7 +625,8 @@ __device__ __noinline__ double* cd_sweeps(const SearchState& s, double thr, doub
         row[k] = s.G + min(m, s.L8 - 1) * s.Lp;
     }
     double *cur = buf, *nxt = buf + s.L8;
-    double r0 = s.r[0], r1 = s.r[1];                         // residuals of this step's coordinate and, without the last step, the next one's
+    // residuals of this step's coordinate and, without the last step, the next one's
+    double r0 = s.r[0], r1 = s.r[1];
 #pragma unroll 1
     for (int sweep = 0; sweep < max_sweeps; ++sweep) {
         double was[NK];

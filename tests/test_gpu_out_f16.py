@@ -1,6 +1,7 @@
 """SR_OUT_F16: the regression calls store their fp32 result rounded to binary16.  Every mode against the oracle on
-shapes that the tensor-core kernels take, by the host rules and pinned to each of the layouts and the general kernel; the bound is the path's own tolerance plus half a
-binary16 unit in the last place of the exact value, and the stored values equal the fp32 output rounded to nearest.
+shapes that the tensor-core kernels take, by the host rules and pinned to each of the layouts and the general kernel; the bound is
+the path's own tolerance plus half a binary16 unit in the last place of the exact value, and the stored values equal the fp32
+output rounded to nearest.
 """
 import numpy as np
 import pytest

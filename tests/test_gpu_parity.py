@@ -434,7 +434,8 @@ def _dictionary_magnitude_range(scale, bound):
 # ------------------------------------------------------------------ LR pixels that are not finite
 
 # kernel (sr_test_force_kernel; -1 = host rules), mode, n, c, h, w, scale, D, k, coefficients: the kernels that make their
-# up-sampled tiles separably, each with more tiles than thread blocks where its tiles follow one another in a block, and those on the smallest frames
+# up-sampled tiles separably, each with more tiles than thread blocks where its tiles follow one another in a block, and those on
+# the smallest frames
 NON_FINITE_LR = [
     (-1, "dense", 2, 3, 12, 70, 2, 32, 5, "f16"), (-1, "dense", 1, 4, 9, 50, 3, 12, 9, "f32"), (-1, "dense", 1, 1, 20, 131, 1, 40, 3, "f32"),      # the split kernel
     (0, "dense", 2, 3, 12, 70, 2, 32, 5, "f16"),
