@@ -223,8 +223,8 @@ typedef struct sr_search_opts {
  * step with the feasible solution that keeps the most atoms taken when no lambda lands in the band.
  * `scratch`: device memory of at least sr_selection_search_scratch_bytes(D) bytes, 8-byte aligned: asked for and checked as
  * before, although the factorisation it was for now stays on the chip and nothing is written to it.  fp64 throughout;
- * one cluster of eight blocks (it starts once eight multiprocessors of a processing cluster are free beside other work), every sum
- * in a fixed order: the same inputs give the same bits on every run.
+ * one cluster of eight blocks (fewer where the context has no room for eight; it starts once that many multiprocessors of a
+ * processing cluster are free beside other work), every sum in a fixed order: the same inputs give the same bits on every run.
  */
 size_t sr_selection_search_scratch_bytes(int32_t D);
 int sr_selection_search(const double* G, const double* b, const double* hh, double nrows, int32_t D,
